@@ -70,7 +70,13 @@ enum { LENIA_GROWTH_SIGNED = 0, LENIA_GROWTH_PAPER = 1 };
  * b1, r2, w2, b2 after the growth planes; needs n_rings > 0. */
 enum { LENIA_LOC_MU = 1, LENIA_LOC_SIGMA = 2, LENIA_LOC_H = 4, LENIA_LOC_KERNEL = 8 };
 /* Convolution routes: AUTO picks FFT for power-of-two worlds with R > 6,
- * else DIRECT (FP32 sums).  DIRECT_BF16 and DIRECT_BF16X3 run the direct
+ * else DIRECT (FP32 sums).  Where a time model says it is faster, AUTO's
+ * direct worlds convolve in overlapping 64 x 64 or 128 x 128 windows of
+ * spectral transforms instead (lenia_conv_path still reports DIRECT; alpha and
+ * Delta_sum decisions that the rounding could turn are settled by the direct
+ * sums at those sites, values of A outside [0, 1] excepted), and so do FFT
+ * worlds without gene maintenance; an explicit LENIA_CONV_DIRECT always
+ * sums.  DIRECT_BF16 and DIRECT_BF16X3 run the direct
  * convolution on the tensor cores as banded Toeplitz products (tcgen05,
  * FP32 accumulation): BF16 operands (8 significant bits: a potential moves
  * by at most (2^-7 + 2^-16) of its value), or both operands split into BF16
@@ -330,7 +336,9 @@ LENIA_API lenia_status lenia_host_wait(lenia_ctx* ctx, void* stream);
  * max_launches kernel launches (event creation only; no device memory).
  * lenia_profile_stop waits for those events and fills total_ms[kind] (summed
  * milliseconds) and counts[kind] for the launch kinds 0..LENIA_PROFILE_KINDS-1
- * (names from lenia_profile_kind_name), then turns recording off. */
+ * (names from lenia_profile_kind_name), then turns recording off.  A
+ * convolution in windows is one launch, recorded as cols_conv (FFT path) or
+ * direct_conv. */
 #define LENIA_PROFILE_KINDS 9
 LENIA_API lenia_status lenia_profile_start(lenia_ctx* ctx, int32_t max_launches);
 LENIA_API lenia_status lenia_profile_stop(lenia_ctx* ctx, float* total_ms, int32_t* counts);

@@ -1,0 +1,527 @@
+// The per-site rule after the convolution (diffusion, growth, alpha, masking,
+// clipped update; arXiv 2304.05639, Sections 2.1-2.4, Algorithm 2) for any
+// kernel count, channel count and growth-gene layout, and diffusion radius 1 or 2.
+//
+// A thread takes four adjacent columns of one row and walks the kernels: each
+// gene plane's stencil comes in as float4 rows plus the two or four neighbours to
+// the left and right, the kernel's genes are diffused, its growth added to
+// its channel, and the diffused genes go straight back out (zeros once alpha is
+// known to be false; sites that turn out false later rewrite theirs).  A
+// block covers 32 columns x 16 rows at a time and strides over the world.
+//
+// Where the genes are maintained, a site whose disk holds no first gene above
+// eps_p has alpha = 0 whatever the rest says: its genes are zero and its update
+// is the per-channel constant.  Such sites (the empty part of a world, most
+// of it in the worlds of the paper) read one gene plane instead of all of
+// them and no potential.
+//
+// The arithmetic is the hardware reciprocal (with one correction for the genes)
+// and exponential.  Alpha tests that its rounding, or the rounding of the
+// windows' potentials, could turn are settled by the other update kernels'
+// arithmetic on the direct sums (`settle`), so that a world's decisions do
+// not depend on the kernel or the convolution it takes.
+//
+// What bounds it: on a mostly empty world the writes of the gene planes, on a
+// full one instruction issue.
+#include <string.h>
+
+#include "lenia_internal.cuh"
+#include "ptx_util.cuh"
+
+namespace lenia {
+namespace {
+
+constexpr int ES_Q = 8, ES_Y = 16;                 // quads and rows of a block (128 threads)
+constexpr int ES_T = ES_Q * ES_Y, ES_NW = ES_T / 32;
+
+struct SitesParams {
+    EpiParams e;
+    int n_worlds;              // worlds of a batched launch (lists in e), else 1
+    int tx, ty;                // blocks of 32 x 16 sites per world
+    int gate;
+    int fast;                  // settle with reciprocals and the hardware exponential, else divisions and expf
+    GuardParams g;
+};
+
+// One gene plane around a quad: rows y - RD .. y + RD, columns x - RD .. x + 3 + RD.
+template <int RD>
+struct Stencil {
+    float v[2 * RD + 1][4 + 2 * RD];
+    __device__ __forceinline__ static constexpr int half(int dy)
+    {
+        return RD == 0 ? 0 : RD == 1 ? (dy == 0 ? 1 : 0) : (dy == 0 ? 2 : (dy == 2 || dy == -2) ? 0 : 1);
+    }
+    // pl: the plane at the quad; ro[]: row offsets from y; xl[], xr[]: offsets of the
+    // columns to the left and right; c: the quad itself
+    __device__ __forceinline__ void load(const float* pl, const int* ro, const int* xl, const int* xr, float4 c)
+    {
+#pragma unroll
+        for (int j = 0; j <= 2 * RD; j++) {
+            const float* row = pl + ro[j];
+            const float4 f = j == RD ? c : __ldg(reinterpret_cast<const float4*>(row));
+            v[j][RD] = f.x;
+            v[j][RD + 1] = f.y;
+            v[j][RD + 2] = f.z;
+            v[j][RD + 3] = f.w;
+#pragma unroll
+            for (int i = 1; i <= RD; i++)
+                if (i <= half(j - RD)) {
+                    v[j][RD - i] = __ldg(row + xl[i - 1]);
+                    v[j][RD + 3 + i] = __ldg(row + xr[i - 1]);
+                }
+        }
+    }
+    __device__ __forceinline__ bool any_above(float eps) const
+    {
+        float m = v[RD][RD];
+#pragma unroll
+        for (int j = 0; j <= 2 * RD; j++)
+#pragma unroll
+            for (int i = 0; i < 4 + 2 * RD; i++)
+                if (i >= RD - half(j - RD) && i < 4 + RD + half(j - RD)) m = fmaxf(m, v[j][i]);
+        return m > eps;
+    }
+    // P^ of the four columns: the disk's sum (rows, then columns) over the count above eps_p, clipped
+    __device__ __forceinline__ void diffused(float eps, float* out) const
+    {
+        float one[2 * RD + 1][4 + 2 * RD];
+#pragma unroll
+        for (int j = 0; j <= 2 * RD; j++)
+#pragma unroll
+            for (int i = 0; i < 4 + 2 * RD; i++)
+                if (i >= RD - half(j - RD) && i < 4 + RD + half(j - RD)) one[j][i] = v[j][i] > eps ? 1.f : 0.f;
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            float s = 0.f, n = 0.f;
+#pragma unroll
+            for (int j = 0; j <= 2 * RD; j++)
+#pragma unroll
+                for (int d = -RD; d <= RD; d++)
+                    if (d <= half(j - RD) && -d <= half(j - RD)) {
+                        const bool first = j == 0;
+                        s = first ? v[j][RD + c + d] : s + v[j][RD + c + d];
+                        n = first ? one[j][RD + c + d] : n + one[j][RD + c + d];
+                    }
+            const float rn = rcp_approx(n), t = s * rn;
+            const float r = fmaf(fmaf(-t, n, s), rn, t);
+            out[c] = n > 0.f ? __saturatef(r) : 0.f;
+        }
+    }
+};
+
+// Kernel k's direct sum at (y, x), in k_direct_conv's order (tap columns, then rows).
+__device__ __forceinline__ float direct_at(const SitesParams& q, const float* A, int k, int y, int x)
+{
+    const int H = q.e.H, W = q.e.W, R = q.g.R[k];
+    const float* plane = A + (size_t)q.e.kt.src[k] * H * W;
+    const float* w = q.g.w + q.g.w_off[k];
+    const int* yr = q.g.yr + q.g.yr_off[k];
+    float acc = 0.f;
+    for (int dx = -R; dx <= R; dx++) {
+        const int r = __ldg(&yr[dx + R]);
+        int xx = x + dx;
+        xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
+        const float* wc = w + (dx + R) * (2 * R + 1) + R;
+        for (int dy = -r; dy <= r; dy++) {
+            int yy = y + dy;
+            yy = yy < 0 ? yy + H : (yy >= H ? yy - H : yy);
+            acc = fmaf(__ldg(&wc[dy]), __ldg(&plane[(size_t)yy * W + xx]), acc);
+        }
+    }
+    return acc;
+}
+
+// The same sum by a whole warp: the lanes load a tap column's values side by side
+// (two columns in flight) and every lane adds them in order.
+__device__ __forceinline__ float direct_warp(const SitesParams& q, const float* A, int k, int y, int x)
+{
+    const int H = q.e.H, W = q.e.W, R = q.g.R[k], lane = threadIdx.x & 31;
+    const float* plane = A + (size_t)q.e.kt.src[k] * H * W;
+    const float* w = q.g.w + q.g.w_off[k];
+    const int* yr = q.g.yr + q.g.yr_off[k];
+    float acc = 0.f;
+    auto fetch = [&](int dx, int dy0, int r, float& v, float& wv) {
+        const int dy = dy0 + lane;
+        v = wv = 0.f;
+        if (dx > R || dy > r) return;
+        int xx = x + dx, yy = y + dy;
+        xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
+        yy = yy < 0 ? yy + H : (yy >= H ? yy - H : yy);
+        v = __ldg(&plane[(size_t)yy * W + xx]);
+        wv = __ldg(&w[(dx + R) * (2 * R + 1) + R + dy]);
+    };
+    int r = __ldg(&yr[0]);
+    float v, wv;
+    fetch(-R, -r, r, v, wv);
+    for (int dx = -R; dx <= R; dx++) {
+        const int rn = dx < R ? __ldg(&yr[dx + 1 + R]) : -1;
+        float vn, wn;
+        fetch(dx + 1, -rn, rn, vn, wn);
+        for (int dy0 = -r; dy0 <= r; dy0 += 32) {
+            if (dy0 > -r) fetch(dx, dy0, r, v, wv);
+            const int n = min(32, r - dy0 + 1);
+            for (int i = 0; i < n; i++)
+                acc = fmaf(__shfl_sync(0xffffffffu, wv, i), __shfl_sync(0xffffffffu, v, i), acc);
+        }
+        v = vn;
+        wv = wn;
+        r = rn;
+    }
+    return acc;
+}
+
+// (growth bump, alpha test) at one site as the other update kernels compute them from
+// the potential u.
+__device__ __forceinline__ float2 settled(const SitesParams& q, float u, float m, float sg, float hh)
+{
+    float gk = 0.f;
+    if (sg > 0.f) {
+        if (q.fast) {
+            const float z = (u - m) * rcp_approx(sg);
+            gk = ex2_approx(-0.721347520444481703680f * (z * z));            // -log2(e) / 2
+        } else {
+            const float z = (u - m) / sg;
+            gk = expf(-0.5f * z * z);
+        }
+    }
+    return make_float2(gk, q.e.alpha_on ? u : hh * gk);
+}
+
+// sum_k of the alpha tests at one site, settled, for a Delta_sum(U) decision near
+// its threshold.
+__device__ __noinline__ float tests_at(const SitesParams& q, const float* A, const float* P, const float* U, int y, int x)
+{
+    const EpiParams& p = q.e;
+    const int H = p.H, W = p.W, K = p.kt.K, RD = p.r_diff;
+    const size_t N = (size_t)H * W;
+    float sum = 0.f;
+    for (int k = 0; k < K; k++) {
+        float g[3] = {0.f, 0.f, 0.f};
+        for (int pp = 0; pp < p.n_p; pp++) {
+            const float* pl = P + (size_t)(pp * K + k) * N;
+            float s = 0.f, n = 0.f;
+            for (int dy = -RD; dy <= RD; dy++)
+                for (int dx = -RD; dx <= RD; dx++) {
+                    if (dy * dy + dx * dx > RD * RD) continue;
+                    int yy = y + dy, xx = x + dx;
+                    yy = yy < 0 ? yy + H : (yy >= H ? yy - H : yy);
+                    xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
+                    const float v = __ldg(&pl[(size_t)yy * W + xx]);
+                    s += v;
+                    n += v > p.eps_p ? 1.f : 0.f;
+                }
+            const float r = q.fast ? s * rcp_approx(n) : s / n;
+            g[pp] = n > 0.f ? __saturatef(r) : 0.f;
+        }
+        const float m = p.p_mu >= 0 ? g[p.p_mu] : p.kt.mu[k];
+        const float sg = p.p_sigma >= 0 ? g[p.p_sigma] : p.kt.sigma[k];
+        const float hh = p.p_h >= 0 ? g[p.p_h] : p.kt.h[k];
+        const float u = q.g.du > 0.f ? direct_at(q, A, k, y, x) : __ldg(&U[(size_t)k * N + (size_t)y * W + x]);
+        sum += settled(q, u, m, sg, hh).y;
+    }
+    return sum;
+}
+
+// LOC: the localized growth genes (LENIA_LOC_* bits).
+template <int LOC, int CT, int RD>
+__global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_sites(const __grid_constant__ SitesParams q)
+{
+    pdl_enter();
+    constexpr int NP = ((LOC & 1) != 0) + ((LOC & 2) != 0) + ((LOC & 4) != 0);
+    constexpr int NQ = NP > 0 ? NP : 1;
+    constexpr int PMU = (LOC & 1) ? 0 : -1;
+    constexpr int PSG = (LOC & 2) ? ((LOC & 1) ? 1 : 0) : -1;
+    constexpr int PH = (LOC & 4) ? NP - 1 : -1;
+    const EpiParams& p = q.e;
+    // statistics: each thread's own sums over its tiles
+    __shared__ float ssum[CT * 5][ES_T];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int H = p.H, W = p.W, K = p.kt.K, C = p.kt.C;
+    const size_t N = (size_t)H * W;
+    const float eps_p = p.eps_p, eps_u = p.eps_u;
+    if (p.partials) {
+#pragma unroll
+        for (int v = 0; v < CT * 5; v++) ssum[v][threadIdx.x] = 0.f;
+    }
+    const int per_world = q.tx * q.ty;
+    for (int t = blockIdx.x; t < per_world * q.n_worlds; t += gridDim.x) {
+        const int wz = t / per_world, tt = t - wz * per_world;
+        const int by = tt / q.tx, bx = tt - by * q.tx;
+        const float* pA = p.A_list ? p.A_list[wz] : p.A;
+        const float* pP = p.P_list ? p.P_list[wz] : p.P;
+        float* pAo = p.Aout_list ? p.Aout_list[wz] : p.A_out;
+        float* pPo = p.Pout_list ? p.Pout_list[wz] : p.P_out;
+        const float* pU = p.U + (size_t)wz * p.u_stride;
+        // lanes beyond the world's edge stand on its last quad and store nothing, so
+        // that the warp stays together
+        const int xq = (bx * ES_Q + (lane & (ES_Q - 1))) * 4, yq = by * ES_Y + warp * (32 / ES_Q) + lane / ES_Q;
+        const bool in = xq < W && yq < H;
+        const int x = xq < W ? xq : W - 4, y = yq < H ? yq : H - 1;
+        {
+            const int i0 = y * W + x;
+            // row offsets from row y, columns left and right of the quad
+            int ro[2 * RD + 1], xl[2], xr[2];
+#pragma unroll
+            for (int j = 0; j <= 2 * RD; j++) {
+                const int r = y + j - RD;
+                ro[j] = (j - RD + (r < 0 ? H : (r >= H ? -H : 0))) * W;
+            }
+#pragma unroll
+            for (int i = 0; i < 2; i++) {
+                xl[i] = -1 - i + (x - 1 - i < 0 ? W : 0);
+                xr[i] = 4 + i - (x + 4 + i >= W ? W : 0);
+            }
+            auto quad = [&](const float* base) { return __ldg(reinterpret_cast<const float4*>(base)); };
+            // the quads of the next kernel's planes and potential are fetched one kernel
+            // ahead; the rows above and below are other threads' quads and mostly
+            // found in L1
+            float4 nc[NQ], nu;
+            Stencil<RD> s0;
+            bool live = in;
+            if constexpr (NP > 0) {
+                nc[0] = quad(pP + i0);
+                s0.load(pP + i0, ro, xl, xr, nc[0]);
+                if (q.gate) live = in && s0.any_above(eps_p);
+            }
+            float acc[CT][4];
+#pragma unroll
+            for (int c = 0; c < CT; c++)
+#pragma unroll
+                for (int i = 0; i < 4; i++) acc[c][i] = 0.f;
+            bool al[4] = {live, live, live, live};
+            float tsum[4] = {0.f, 0.f, 0.f, 0.f}, tband[4] = {0.f, 0.f, 0.f, 0.f};
+            bool wrote = false;                     // a non-zero gene went out already
+            int k = 0;
+            if (__any_sync(0xffffffffu, live)) {
+                const float* up = pU + i0;
+                const float* gp = pP + i0;          // kernel k's first plane at the quad
+                float* go = pPo + i0;
+                const size_t KN = (size_t)K * N;
+                bool want = live;               // something left to compute for this quad
+                if (want) {
+                    nu = quad(up);
+#pragma unroll
+                    for (int pp = 1; pp < NP; pp++) nc[pp] = quad(gp + pp * KN);
+                }
+#pragma unroll 1
+                for (; k < K; k++) {
+                    float ph[NQ][4], u[4], gk[4], tk[4];
+                    const float km = p.kt.mu[k], ks = p.kt.sigma[k], kh = p.kt.h[k];
+                    auto mu_of = [&](int c) { return PMU >= 0 ? ph[PMU >= 0 ? PMU : 0][c] : km; };
+                    auto sg_of = [&](int c) { return PSG >= 0 ? ph[PSG >= 0 ? PSG : 0][c] : ks; };
+                    auto h_of = [&](int c) { return PH >= 0 ? ph[PH >= 0 ? PH : 0][c] : kh; };
+                    uint32_t near = 0;              // sites whose test is to be settled
+                    up += N;
+                    if (want) {
+                        float4 cc4[NQ];
+                        u[0] = nu.x, u[1] = nu.y, u[2] = nu.z, u[3] = nu.w;
+#pragma unroll
+                        for (int pp = 0; pp < NP; pp++) cc4[pp] = nc[pp];
+                        if (k + 1 < K) {
+                            nu = quad(up);
+#pragma unroll
+                            for (int pp = 0; pp < NP; pp++) nc[pp] = quad(gp + pp * KN + N);
+                        }
+#pragma unroll
+                        for (int pp = 0; pp < NP; pp++) {
+                            Stencil<RD> s;
+                            s.load(gp + pp * KN, ro, xl, xr, cc4[pp]);
+                            s.diffused(eps_p, ph[pp]);
+#pragma unroll
+                            for (int c = 0; c < 4; c++) al[c] = al[c] & (ph[pp][c] > eps_p);
+                        }
+#pragma unroll
+                        for (int c = 0; c < 4; c++) {
+                            const float sg = sg_of(c);
+                            const float rs = rcp_approx(sg), z = (u[c] - mu_of(c)) * rs, z2 = z * z;
+                            const float e = ex2_approx(-0.721347520444481703680f * z2);      // -log2(e) / 2
+                            gk[c] = sg > 0.f ? e : 0.f;
+                            tk[c] = p.alpha_on ? u[c] : h_of(c) * gk[c];
+                            if (NP > 0) {
+                                // how far the test may be off: rounding, and the potential's du
+                                // through |d t / d u| = t |z| / s (doubled for its curvature); a
+                                // bump narrower than du's reach is always settled
+                                const float off = p.alpha_on
+                                                      ? q.g.du + 1e-7f * fabsf(u[c])
+                                                      : fabsf(tk[c]) * fmaf(2e-6f, z2, fmaf(2.f * q.g.du * rs, fabsf(z), 2e-6f));
+                                const bool narrow = sg < q.g.du * 64.f;
+                                if (p.empty_out) tband[c] += narrow ? fabsf(h_of(c)) : off;
+                                near |= (al[c] & (narrow | (fabsf(tk[c] - eps_u) <= off)) ? 1u : 0u) << c;
+                            }
+                        }
+                    }
+                    if (NP > 0) {
+                        // one site after the other, the warp summing its potential together
+                        for (uint32_t nm = __ballot_sync(0xffffffffu, near != 0); nm;
+                             nm = __ballot_sync(0xffffffffu, near != 0)) {
+                            const int L = __ffs(nm) - 1;
+                            const int i = __ffs(__shfl_sync(0xffffffffu, near, L)) - 1;
+                            const int ys = __shfl_sync(0xffffffffu, y, L), xs = __shfl_sync(0xffffffffu, x, L) + i;
+                            float ud = 0.f;
+                            if (q.g.du > 0.f) ud = direct_warp(q, pA, k, ys, xs);
+                            if (lane == L) {
+#pragma unroll
+                                for (int c = 0; c < 4; c++)
+                                    if (c == i) {
+                                        const float2 r = settled(q, q.g.du > 0.f ? ud : u[c], mu_of(c), sg_of(c), h_of(c));
+                                        gk[c] = r.x;
+                                        tk[c] = r.y;
+                                    }
+                                near &= near - 1;
+                            }
+                        }
+                    }
+                    float G[4];
+                    if (want) {
+#pragma unroll
+                        for (int c = 0; c < 4; c++) {
+                            if (NP > 0) al[c] = al[c] & (tk[c] > eps_u);
+                            tsum[c] += tk[c];
+                            G[c] = p.growth_form == 0 ? fmaf(2.f * gk[c], h_of(c), -h_of(c)) : h_of(c) * gk[c];
+                        }
+                        const int d = p.kt.dst[k];
+#pragma unroll
+                        for (int cc = 0; cc < CT; cc++)
+                            if (CT == 1 || cc == d)
+#pragma unroll
+                                for (int c = 0; c < 4; c++) acc[cc][c] += G[c];
+                    }
+                    if (NP > 0) {
+                        const bool any = al[0] | al[1] | al[2] | al[3];
+                        wrote |= any;
+                        if (in)
+#pragma unroll
+                        for (int pp = 0; pp < NP; pp++)
+                            *reinterpret_cast<float4*>(go + pp * KN) =
+                                make_float4(al[0] ? ph[pp][0] : 0.f, al[1] ? ph[pp][1] : 0.f,
+                                            al[2] ? ph[pp][2] : 0.f, al[3] ? ph[pp][3] : 0.f);
+                        gp += N;
+                        go += N;
+                        // alpha is false at all four sites: nothing more to compute, unless
+                        // Delta_sum wants every kernel's growth
+                        want = want && (any || p.empty_out);
+                        if (!__any_sync(0xffffffffu, want)) {
+                            k++;
+                            break;
+                        }
+                    }
+                }
+            }
+            if (NP > 0 && in) {
+                const bool all = al[0] & al[1] & al[2] & al[3], any = al[0] | al[1] | al[2] | al[3];
+                const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int pp = 0; pp < NP; pp++) {
+                    float* o = pPo + (size_t)pp * K * N + i0;
+                    // planes of the kernels that were not reached (alpha is false)
+                    for (int j = k; j < K; j++) *reinterpret_cast<float4*>(o + (size_t)j * N) = z4;
+                    // planes written before alpha was known to be false
+                    if (wrote && !any)
+                        for (int j = 0; j < k; j++) *reinterpret_cast<float4*>(o + (size_t)j * N) = z4;
+                    else if (wrote && !all)
+                        for (int j = 0; j < k; j++)
+#pragma unroll
+                            for (int c = 0; c < 4; c++)
+                                if (!al[c]) o[(size_t)j * N + c] = 0.f;
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < CT; c++) {
+                if (c >= C || !in) break;
+                const float4 a4 = __ldg(reinterpret_cast<const float4*>(pA + (size_t)c * N + i0));
+                const float a[4] = {a4.x, a4.y, a4.z, a4.w};
+                float o[4];
+#pragma unroll
+                for (int i = 0; i < 4; i++) o[i] = __saturatef(a[i] + p.dt * ((NP == 0 || al[i]) ? acc[c][i] : p.acc0[c]));
+                *reinterpret_cast<float4*>(pAo + (size_t)c * N + i0) = make_float4(o[0], o[1], o[2], o[3]);
+                if (p.partials) {
+                    // (the tables start at any float: scalar loads)
+                    const float* sx = p.sin_x + x;
+                    const float* cx = p.cos_x + x;
+                    const float m = (o[0] + o[1]) + (o[2] + o[3]);
+                    float* a5 = &ssum[c * 5][threadIdx.x];
+                    a5[0] += m;
+                    a5[ES_T] += m * __ldg(&p.sin_y[y]);
+                    a5[2 * ES_T] += m * __ldg(&p.cos_y[y]);
+                    a5[3 * ES_T] += (o[0] * __ldg(sx) + o[1] * __ldg(sx + 1)) + (o[2] * __ldg(sx + 2) + o[3] * __ldg(sx + 3));
+                    a5[4 * ES_T] += (o[0] * __ldg(cx) + o[1] * __ldg(cx + 1)) + (o[2] * __ldg(cx + 2) + o[3] * __ldg(cx + 3));
+                }
+            }
+            if (in && p.alpha_out)
+                *reinterpret_cast<uchar4*>(p.alpha_out + i0) =
+                    NP == 0 ? make_uchar4(1, 1, 1, 1) : make_uchar4(al[0], al[1], al[2], al[3]);
+            if (NP > 0 && in && p.empty_out)
+#pragma unroll
+                for (int c = 0; c < 4; c++)
+                    if (fabsf(tsum[c] - eps_u) <= tband[c] + 1e-6f) tsum[c] = tests_at(q, pA, pP, pU, y, x + c);
+            if (in && p.empty_out)
+                *reinterpret_cast<uchar4*>(p.empty_out + i0) =
+                    make_uchar4(!(tsum[0] > eps_u), !(tsum[1] > eps_u), !(tsum[2] > eps_u), !(tsum[3] > eps_u));
+        }
+    }
+    if (p.partials) {
+        // one warp per value: lanes, then a shuffle tree, in compensated pairs
+        __syncthreads();
+        for (int v = warp; v < C * 5; v += ES_NW) {
+            float2 s = make_float2(0.f, 0.f);
+            for (int i = lane; i < ES_T; i += 32) s = ff_add(s, make_float2(ssum[v][i], 0.f));
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) s = ff_add(s, ff_shfl_down(s, off));
+            if (lane == 0) p.partials[(size_t)blockIdx.x * C * 5 + v] = s;
+        }
+    }
+}
+
+template <int LOC, int CT, int RD>
+cudaError_t launch_sites(SitesParams& q, int max_blocks, cudaStream_t s, int* n_blocks)
+{
+    const long long tiles = (long long)q.tx * q.ty * q.n_worlds;
+    const int blocks = (int)(tiles < max_blocks ? tiles : max_blocks);
+    if (n_blocks) *n_blocks = blocks;
+    launch_pdl(k_epilogue_sites<LOC, CT, RD>, dim3(blocks), dim3(ES_T), 0, s, q);
+    return cudaGetLastError();
+}
+
+template <int LOC, int RD>
+cudaError_t launch_sites_c(SitesParams& q, int max_blocks, cudaStream_t s, int* n_blocks)
+{
+    const int C = q.e.kt.C;
+    if (C == 1) return launch_sites<LOC, 1, RD>(q, max_blocks, s, n_blocks);
+    if (C <= 3) return launch_sites<LOC, 3, RD>(q, max_blocks, s, n_blocks);
+    return launch_sites<LOC, kMaxChannels, RD>(q, max_blocks, s, n_blocks);
+}
+
+}  // namespace
+
+bool epilogue_sites_supported(const EpiParams& p)
+{
+    if (p.n_rings || p.p_kern >= 0 || (size_t)p.H * p.W >= (1u << 30)) return false;
+    const int loc = (p.p_mu >= 0 ? 1 : 0) | (p.p_sigma >= 0 ? 2 : 0) | (p.p_h >= 0 ? 4 : 0);
+    return loc == 0 || ((loc == 3 || loc == 7) && p.maintain && p.eps_p == 0.f && (p.r_diff == 1 || p.r_diff == 2));
+}
+
+bool epilogue_gated(const EpiParams& p)
+{
+    return p.maintain && p.n_p > 0 && p.eps_p >= 0.f && !p.empty_out;
+}
+
+cudaError_t launch_epilogue_sites(const EpiParams& p, bool fast, const GuardParams* guard, int n_worlds, int max_blocks,
+                                  cudaStream_t s, int* n_blocks)
+{
+    if (!epilogue_sites_supported(p) || n_worlds < 1 || max_blocks < 1) return cudaErrorInvalidValue;
+    SitesParams q;
+    memset(&q, 0, sizeof(q));
+    q.e = p;
+    if (guard) q.g = *guard;
+    q.n_worlds = n_worlds;
+    q.tx = (p.W + 4 * ES_Q - 1) / (4 * ES_Q);
+    q.ty = (p.H + ES_Y - 1) / ES_Y;
+    q.gate = epilogue_gated(p);
+    q.fast = fast;
+    if (p.n_p == 0) return launch_sites_c<0, 0>(q, max_blocks, s, n_blocks);
+    if (p.r_diff == 1)
+        return p.n_p == 2 ? launch_sites_c<3, 1>(q, max_blocks, s, n_blocks) : launch_sites_c<7, 1>(q, max_blocks, s, n_blocks);
+    return p.n_p == 2 ? launch_sites_c<3, 2>(q, max_blocks, s, n_blocks) : launch_sites_c<7, 2>(q, max_blocks, s, n_blocks);
+}
+
+}  // namespace lenia

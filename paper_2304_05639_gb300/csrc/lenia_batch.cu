@@ -47,6 +47,14 @@ struct Group {
     float2* Uhat = nullptr;                // [n][K][M][H]
     float* U = nullptr;                    // [n][K][H][W]
     const float** S = nullptr;             // per-world kernel spectra (worlds may differ in kernels)
+    // worlds that convolve in windows: one launch per window size (their radii,
+    // and so their window sizes, may differ), the worlds' buffers per direction
+    struct TileSet {
+        lenia::TileParams p;
+        std::vector<int> member;           // positions in `worlds`
+        lenia::TileWorld* list[2] = {nullptr, nullptr};
+    };
+    std::vector<TileSet> tiles;
     // per-world pointer lists for the two ping-pong directions:
     // [0] caller's state -> batch state, [1] batch state -> caller's state
     const float** Ain[2] = {nullptr, nullptr};
@@ -128,6 +136,9 @@ void free_group(Group& g)
                     g.Pout[0], g.Pout[1], g.qw[0], g.qw[1], g.counter};
     for (void* p : ptrs)
         if (p) cudaFree(p);
+    for (Group::TileSet& t : g.tiles)
+        for (lenia::TileWorld* p : t.list)
+            if (p) cudaFree(p);
 }
 
 // The epilogue parameters of a group for direction `dir`.
@@ -153,6 +164,9 @@ cudaError_t group_epilogue(const Group& g, int dir, cudaStream_t s)
 {
     const lenia::EpiParams ep = group_epi(g, dir);
     const int n = (int)g.worlds.size();
+    // several kernels: the per-site kernel, as a world takes on its own
+    if (g.epi == 0 && ep.kt.K > 1 && g.aligned_all && lenia::epilogue_sites_supported(ep))
+        return lenia::launch_epilogue_sites(ep, false, nullptr, n, 1 << 20, s, nullptr);
     if (g.epi == 1) return lenia::launch_epilogue_queue(ep, g.qw[dir], n, g.bands, 0, g.counter, g.v.fp.status, s);
     // the four-column form needs 16-byte aligned state buffers
     return lenia::launch_epilogue_batch(ep, n, s, g.br < 0 && !g.aligned_all ? 2 : g.br);
@@ -162,6 +176,13 @@ cudaError_t group_epilogue(const Group& g, int dir, cudaStream_t s)
 lenia_status group_step(const Group& g, int dir, cudaStream_t s)
 {
     const int n = (int)g.worlds.size();
+    for (const Group::TileSet& t : g.tiles) {
+        lenia::TileParams tp = t.p;
+        tp.worlds = t.list[dir];
+        tp.aligned = g.aligned ? 1 : 0;
+        if (lenia::launch_tile_conv(tp, s) != cudaSuccess) return LENIA_ECUDA;
+    }
+    if (!g.tiles.empty()) return group_epilogue(g, dir, s) == cudaSuccess ? LENIA_OK : LENIA_ECUDA;
     lenia::FftParams fp = g.v.fp;
     fp.A = nullptr;
     fp.A_list = g.Ain[dir];
@@ -457,7 +478,7 @@ lenia_status lenia_batch_init(int32_t n_worlds, const lenia_config* cfgs, const 
             std::vector<double> key = {(double)c0.height, (double)c0.width, (double)c0.n_channels,
                                        (double)c0.n_kernels, c0.dt, (double)c0.growth_form, (double)c0.localized,
                                        (double)c0.maintain_genes, c0.eps_u, c0.eps_p, (double)c0.r_diff,
-                                       (double)c0.alpha_on, (double)c0.n_rings};
+                                       (double)c0.alpha_on, (double)c0.n_rings, (double)v.tile};
             // kernel shapes may differ (each world's spectra are read through a list)
             for (int k = 0; k < c0.n_kernels; k++) {
                 const lenia_kernel_desc& d = ks[k];
@@ -477,18 +498,49 @@ lenia_status lenia_batch_init(int32_t n_worlds, const lenia_config* cfgs, const 
             lenia::ctx_view(b->ctx[g.worlds[0]], &g.v);
             const size_t n = g.worlds.size();
             const size_t H = cfgs[g.worlds[0]].height, W = cfgs[g.worlds[0]].width, M = W / 2;
-            bool okg = cudaMalloc(&g.Ahat, n * g.v.C * M * H * sizeof(float2)) == cudaSuccess &&
-                       cudaMalloc(&g.Uhat, n * g.v.K * M * H * sizeof(float2)) == cudaSuccess &&
-                       cudaMalloc(&g.U, n * g.v.K * g.v.N * sizeof(float)) == cudaSuccess &&
-                       cudaMalloc(&g.S, n * sizeof(float*)) == cudaSuccess;
-            if (okg) {
-                std::vector<const float*> spec(n);
-                for (size_t j = 0; j < n; j++) {
+            bool okg = cudaMalloc(&g.U, n * g.v.K * g.v.N * sizeof(float)) == cudaSuccess;
+            if (g.v.tile) {
+                std::map<int, std::vector<int>> by_size;
+                for (size_t j = 0; okg && j < n; j++) {
+                    lenia_ctx* c = b->ctx[g.worlds[j]];
+                    // widths of 256 k: the window size that suits the whole group.  At
+                    // others a grouped world keeps the window size it has on its
+                    // own, and with it its results bit for bit
+                    if (W % 256 == 0) okg = lenia::ctx_group_tiles(c, (int)n, s) == cudaSuccess;
                     lenia::lenia_ctx_view vj;
-                    lenia::ctx_view(b->ctx[g.worlds[j]], &vj);
-                    spec[j] = vj.fp.S;
+                    lenia::ctx_view(c, &vj);
+                    by_size[vj.tl.N].push_back((int)j);
                 }
-                okg = cudaMemcpy(g.S, spec.data(), n * sizeof(float*), cudaMemcpyHostToDevice) == cudaSuccess;
+                for (auto& bs : by_size) {
+                    Group::TileSet t;
+                    t.member = bs.second;
+                    lenia::lenia_ctx_view vj;
+                    lenia::ctx_view(b->ctx[g.worlds[t.member[0]]], &vj);
+                    t.p = vj.tl;
+                    t.p.n_worlds = (int)t.member.size();
+                    t.p.kpb = 64;                       // every kernel of a channel in one block
+                    t.p.tiles = 0;
+                    for (int j : t.member) {
+                        lenia::ctx_view(b->ctx[g.worlds[j]], &vj);
+                        t.p.tiles = std::max(t.p.tiles, vj.tl.g.tiles_x * vj.tl.g.tiles_y);
+                    }
+                    for (int d = 0; okg && d < 2; d++)
+                        okg = cudaMalloc(&t.list[d], t.member.size() * sizeof(lenia::TileWorld)) == cudaSuccess;
+                    g.tiles.push_back(t);
+                }
+            } else {
+                okg = okg && cudaMalloc(&g.Ahat, n * g.v.C * M * H * sizeof(float2)) == cudaSuccess &&
+                      cudaMalloc(&g.Uhat, n * g.v.K * M * H * sizeof(float2)) == cudaSuccess &&
+                      cudaMalloc(&g.S, n * sizeof(float*)) == cudaSuccess;
+                if (okg) {
+                    std::vector<const float*> spec(n);
+                    for (size_t j = 0; j < n; j++) {
+                        lenia::lenia_ctx_view vj;
+                        lenia::ctx_view(b->ctx[g.worlds[j]], &vj);
+                        spec[j] = vj.fp.S;
+                    }
+                    okg = cudaMemcpy(g.S, spec.data(), n * sizeof(float*), cudaMemcpyHostToDevice) == cudaSuccess;
+                }
             }
             for (int d = 0; okg && d < 2; d++)
                 okg = cudaMalloc(&g.Ain[d], n * sizeof(float*)) == cudaSuccess &&
@@ -592,6 +644,17 @@ lenia_status lenia_batch_rollout(lenia_batch* b, float* const* A, float* const* 
                       cudaMemcpy(g.Pin[1], p1.data(), pb, cudaMemcpyHostToDevice) == cudaSuccess &&
                       cudaMemcpy(g.Aout[1], ao1.data(), pb, cudaMemcpyHostToDevice) == cudaSuccess &&
                       cudaMemcpy(g.Pout[1], po1.data(), pb, cudaMemcpyHostToDevice) == cudaSuccess;
+            for (Group::TileSet& t : g.tiles)
+                for (int d = 0; ok && d < 2; d++) {
+                    std::vector<lenia::TileWorld> tw;
+                    for (int j : t.member) {
+                        lenia::lenia_ctx_view vj;
+                        lenia::ctx_view(b->ctx[g.worlds[j]], &vj);
+                        tw.push_back({d ? a1[j] : a0[j], g.U + (size_t)j * g.v.K * g.v.N, vj.tl.S, vj.tl.S0, vj.tl.g});
+                    }
+                    ok = cudaMemcpy(t.list[d], tw.data(), tw.size() * sizeof(lenia::TileWorld),
+                                    cudaMemcpyHostToDevice) == cudaSuccess;
+                }
             if (!ok) return LENIA_ECUDA;
             if (g.qw[0]) {
                 // per-world tensor maps of the queued streaming epilogue, both directions

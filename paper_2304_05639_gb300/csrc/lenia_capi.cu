@@ -52,6 +52,15 @@ struct lenia_ctx {
     TcConvParams tp;
     int* d_yr = nullptr;
     int* d_yr_off = nullptr;
+    // convolution in overlapping spectral windows (tile_conv.cu), where that is
+    // faster than the path's other form
+    bool tile = false;
+    TileParams tl;
+    bool gate_pays = false;                // more windows than run at once: skipping some saves time
+    float guard_du = 0.f;                  // how far the windows' and the direct sums' potentials may be apart
+    float* d_tS = nullptr;
+    float* d_tS0 = nullptr;
+    float2* d_ttw = nullptr;
     float* d_S = nullptr;
     float2* d_twM = nullptr;
     float2* d_twW = nullptr;
@@ -130,6 +139,10 @@ static_assert(KIND_COUNT == LENIA_PROFILE_KINDS, "profile kinds and the header d
 static_assert(sizeof(kKindNames) / sizeof(kKindNames[0]) == KIND_COUNT, "one name per profile kind");
 
 namespace {
+
+// blocks of the per-site kernel per SM: enough to even out live and empty parts of
+// a world, few enough for their statistics records
+constexpr int kSitesBlocksPerSm = 24;
 
 const double kTwoPi = 6.283185307179586476925286766559;
 
@@ -319,6 +332,36 @@ std::vector<float2> pass_twiddles(int n, int rmax)
     return t;
 }
 
+// FP32 spectra of every convolution plane on an H x W torus into S ([plane]
+// [kx][ky], on the device), from FP64 sums rounded once.  Waits for the work.
+cudaError_t build_spectra(lenia_ctx* c, int H, int W, float* S, cudaStream_t s)
+{
+    const int M = W / 2, HS = H / 2 + 1;
+    std::vector<double> cosH(H), cosW(W);
+    for (int m = 0; m < H; m++) cosH[m] = cos(kTwoPi * m / H);
+    for (int m = 0; m < W; m++) cosW[m] = cos(kTwoPi * m / W);
+    double *d_cosH = nullptr, *d_cosW = nullptr, *d_Kd = nullptr, *d_T = nullptr;
+    const size_t kmax = (size_t)(2 * c->max_R + 1) * (2 * c->max_R + 1);
+    bool ok = cudaMalloc(&d_cosH, H * sizeof(double)) == cudaSuccess &&
+              cudaMalloc(&d_cosW, W * sizeof(double)) == cudaSuccess &&
+              cudaMalloc(&d_Kd, kmax * sizeof(double)) == cudaSuccess &&
+              cudaMalloc(&d_T, (size_t)(2 * c->max_R + 1) * (M + 1) * sizeof(double)) == cudaSuccess;
+    cudaError_t e = ok ? cudaSuccess : cudaErrorMemoryAllocation;
+    if (e == cudaSuccess) e = cudaMemcpy(d_cosH, cosH.data(), H * sizeof(double), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(d_cosW, cosW.data(), W * sizeof(double), cudaMemcpyHostToDevice);
+    for (size_t k = 0; k < c->conv_w.size() && e == cudaSuccess; k++) {
+        e = cudaMemcpyAsync(d_Kd, c->conv_w[k].data(), c->conv_w[k].size() * sizeof(double), cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess)
+            e = launch_spectra(d_Kd, c->conv_R[k], H, W, d_cosH, d_cosW, d_T, S + k * (size_t)(M + 1) * HS, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    }
+    cudaFree(d_cosH);
+    cudaFree(d_cosW);
+    cudaFree(d_Kd);
+    cudaFree(d_T);
+    return e;
+}
+
 std::vector<float2> twiddles(int n, int count)
 {
     std::vector<float2> t((size_t)count);
@@ -327,6 +370,40 @@ std::vector<float2> twiddles(int n, int count)
         t[m] = make_float2((float)cos(a), (float)-sin(a));
     }
     return t;
+}
+
+// Spectra and twiddles of the context's windows (c->tl.N).  Waits for the work.
+lenia_status build_tiles(lenia_ctx* c, cudaStream_t s)
+{
+    const int n = c->tl.N, ca = n / 8, NC = (int)c->conv_w.size();
+    const size_t ns = tile_spectrum_floats(n), hs = (size_t)(n / 2 + 1) * (n / 2 + 1);
+    for (void* q : {(void*)c->d_tS, (void*)c->d_tS0, (void*)c->d_ttw})
+        if (q) cudaFree(q);
+    c->d_tS = c->d_tS0 = nullptr;
+    c->d_ttw = nullptr;
+    lenia_status st = dalloc(c, &c->d_tS, ns * NC);
+    if (st == LENIA_OK) st = dalloc(c, &c->d_tS0, (size_t)n * NC);
+    if (st == LENIA_OK) st = dalloc(c, &c->d_ttw, (size_t)n);
+    float* d_tmp = nullptr;
+    if (st == LENIA_OK) st = dalloc(c, &d_tmp, hs * NC);
+    if (st != LENIA_OK) return st;
+    std::vector<float2> tw(n);
+    for (int b = 0; b < 8; b++)
+        for (int n1 = 0; n1 < ca; n1++) {
+            const double a = kTwoPi * n1 * b / n;
+            tw[b * ca + n1] = make_float2((float)cos(a), (float)-sin(a));
+        }
+    cudaError_t e = cudaMemcpy(c->d_ttw, tw.data(), n * sizeof(float2), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = build_spectra(c, n, n, d_tmp, s);
+    for (int k = 0; k < NC && e == cudaSuccess; k++)
+        e = launch_tile_spectra(n, d_tmp + hs * k, c->d_tS + ns * k, c->d_tS0 + (size_t)n * k, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaFree(d_tmp);
+    if (e != cudaSuccess) return fail(c, LENIA_ECUDA, std::string("window spectra: ") + cudaGetErrorString(e));
+    c->tl.S = c->d_tS;
+    c->tl.S0 = c->d_tS0;
+    c->tl.tw = c->d_ttw;
+    return LENIA_OK;
 }
 
 // Records an event pair around each launch while profiling is on.
@@ -353,9 +430,20 @@ struct ProfScope {
     }
 };
 
-lenia_status potentials(lenia_ctx* c, const float* A, float* U, cudaStream_t s)
+// gate: a gene plane outside whose neighbourhood the potentials are not needed, or null
+lenia_status potentials(lenia_ctx* c, const float* A, float* U, cudaStream_t s, const float* gate = nullptr,
+                        bool windows = true)
 {
-    if (c->path == LENIA_CONV_FFT) {
+    if (c->tile && windows) {
+        TileParams tl = c->tl;
+        tl.A = A;
+        tl.U = U;
+        tl.gate = gate;
+        tl.gate_eps = c->cfg.eps_p;
+        tl.gate_r = c->cfg.r_diff;
+        ProfScope ps(c, c->path == LENIA_CONV_FFT ? KIND_COLS : KIND_DIRECT, s);
+        CUDA_OR_FAIL(c, launch_tile_conv(tl, s));
+    } else if (c->path == LENIA_CONV_FFT) {
         FftParams fp = c->fp;
         fp.A = A;
         fp.U = U;
@@ -446,18 +534,36 @@ lenia_status step_impl(lenia_ctx* c, const float* A_in, const float* P_in, float
                        float* stats_out, uint8_t* alpha_out, const float* U_given, cudaStream_t s,
                        uint8_t* empty_out = nullptr)
 {
+    EpiParams ep = epi_params(c);
+    ep.empty_out = empty_out;
+    auto aligned16 = [](const void* q) { return ((uintptr_t)q & 15) == 0; };
+    // The per-site kernel where the shape has no kernel of its own (the streaming one,
+    // or the tiled ones of one-kernel worlds), and wherever the windows need
+    // their alpha decisions settled
+    const bool sites_ok = epilogue_sites_supported(ep) && aligned16(A_in) && aligned16(P_in) && aligned16(U_given) &&
+                          aligned16(A_out) && aligned16(P_out) && ((uintptr_t)alpha_out & 3) == 0;
+    // (one-kernel worlds without statistics: four columns per thread, float4 rows;
+    // 1024^2: 21.5 against 25.6 us per step with the streaming kernel, whose
+    // pipelines are short here)
+    const bool quads11 = !stats_out && !alpha_out && !empty_out && ep.kt.K == 1 && ep.kt.C == 1 && ep.W % 128 == 0 &&
+                         ep.H % 8 == 0 && epilogue_batch_supported(ep);
+    // worlds with alpha decisions take the windows only where the per-site kernel
+    // settles them
+    const bool windows = c->tile && (!c->cfg.maintain_genes || sites_ok);
+    const bool settle = windows && c->cfg.maintain_genes && !U_given;
+    const bool sites = sites_ok && (settle || !((ep.kt.K == 1 && ep.kt.C == 1) || epilogue_rows_supported(ep)));
     if (!U_given) {
-        lenia_status st = potentials(c, A_in, c->d_U, s);
+        // sites without a first gene around them need no potentials
+        const float* gate = sites && c->gate_pays && epilogue_gated(ep) ? P_in : nullptr;
+        lenia_status st = potentials(c, A_in, c->d_U, s, gate, windows);
         if (st != LENIA_OK) return st;
     }
-    EpiParams ep = epi_params(c);
     ep.A = A_in;
     ep.P = P_in;
     ep.U = U_given ? U_given : c->d_U;
     ep.A_out = A_out;
     ep.P_out = c->n_p ? P_out : nullptr;
     ep.alpha_out = alpha_out;
-    ep.empty_out = empty_out;
     ep.partials = stats_out ? c->d_partials : nullptr;
     int nb = 0;
     bool fused_stats = false;
@@ -465,12 +571,21 @@ lenia_status step_impl(lenia_ctx* c, const float* A_in, const float* P_in, float
         ProfScope ps(c, KIND_EPI, s);
         const bool aligned = ((uintptr_t)ep.A % 16 == 0) && ((uintptr_t)ep.U % 16 == 0) &&
                              (!ep.P || (uintptr_t)ep.P % 16 == 0);
-        // one-kernel worlds without statistics: the tiled kernel with four
-        // columns per thread (float4 rows; 1024^2: 21.5 against 25.6 us per
-        // step with the streaming kernel, whose pipelines are short here)
         const bool aligned_out = ((uintptr_t)ep.A_out % 16 == 0) && (!ep.P_out || (uintptr_t)ep.P_out % 16 == 0);
-        if (!stats_out && !alpha_out && !empty_out && ep.kt.K == 1 && ep.kt.C == 1 && ep.W % 128 == 0 &&
-            ep.H % 8 == 0 && epilogue_batch_supported(ep) && aligned && aligned_out) {
+        if (sites) {
+            // the arithmetic of the kernel that the shape otherwise takes
+            const bool fast = epilogue_rows_supported(ep) && !quads11;
+            GuardParams g;
+            if (settle) {
+                g.w = c->d_w;
+                g.w_off = c->d_w_off;
+                g.yr = c->d_yr;
+                g.yr_off = c->d_yr_off;
+                for (int k = 0; k < c->cfg.n_kernels; k++) g.R[k] = c->conv_R[k];
+                g.du = c->guard_du;
+            }
+            CUDA_OR_FAIL(c, launch_epilogue_sites(ep, fast, settle ? &g : nullptr, 1, kSitesBlocksPerSm * c->num_sms, s, &nb));
+        } else if (quads11 && aligned && aligned_out) {
             CUDA_OR_FAIL(c, launch_epilogue_batch(ep, 1, s, -1));
         } else if (aligned && epilogue_rows_supported(ep)) {
             ep.stats_out = stats_out;        // reduced by the kernel's last block
@@ -500,6 +615,15 @@ lenia_status transposed_conv(lenia_ctx* c, const float* gU, float* V, cudaStream
                              const float* add = nullptr, float* out = nullptr)
 {
     const int K = c->cfg.n_kernels;
+    if (c->tile && c->path != LENIA_CONV_FFT) {
+        TileParams tl = c->tl;
+        tl.A = gU;
+        tl.U = out ? out : V;
+        tl.add = out ? add : nullptr;
+        CUDA_OR_FAIL(c, launch_tile_conv_adj(tl, s));
+        *per_channel = true;
+        return LENIA_OK;
+    }
     if (c->path == LENIA_CONV_FFT) {
         FftParams fp = c->fp;
         fp.A = gU;
@@ -541,12 +665,25 @@ namespace lenia {
 bool ctx_view(lenia_ctx* c, lenia_ctx_view* v)
 {
     if (!c || !v || c->path != LENIA_CONV_FFT) return false;
+    v->tile = c->tile;
+    v->tl = c->tl;
     v->fp = c->fp;
+    v->fp.H = c->cfg.height;
+    v->fp.W = c->cfg.width;
+    v->fp.status = c->d_status;
     v->ep = epi_params(c);
     v->N = c->N;
     v->C = c->cfg.n_channels;
     v->K = (int)c->conv_w.size();
     return true;
+}
+
+cudaError_t ctx_group_tiles(lenia_ctx* c, int n_worlds, cudaStream_t s)
+{
+    if (!c || !c->tile) return cudaErrorInvalidValue;
+    const int n = c->tl.N;
+    tile_choose(&c->tl, c->cfg.height, c->cfg.width, c->tl.kcount, c->max_R, n_worlds);
+    return c->tl.N == n || build_tiles(c, s) == LENIA_OK ? cudaSuccess : cudaErrorUnknown;
 }
 }  // namespace lenia
 
@@ -585,8 +722,10 @@ int32_t lenia_launches_per_step(const lenia_ctx* ctx)
 {
     if (!ctx) return -1;
     EpiParams ep = epi_params(const_cast<lenia_ctx*>(ctx));
-    const bool fused = epilogue_rows_supported(ep);   // stats reduced inside the epilogue
-    const int conv = ctx->path == LENIA_CONV_FFT ? 3 : (ctx->path == LENIA_CONV_DIRECT ? 1 : 2);
+    // statistics reduced inside the epilogue (the streaming kernel)
+    const bool fused = epilogue_rows_supported(ep) &&
+                       !(ctx->tile && ctx->cfg.maintain_genes && epilogue_sites_supported(ep));
+    const int conv = ctx->tile ? 1 : ctx->path == LENIA_CONV_FFT ? 3 : (ctx->path == LENIA_CONV_DIRECT ? 1 : 2);
     return conv + (fused ? 1 : 2);
 }
 
@@ -600,7 +739,8 @@ void lenia_destroy(lenia_ctx* c)
                     c->d_Ahat_t, c->d_Uhat_t, c->d_ticket, c->d_walls, c->d_alpha_e, c->d_empty,
                     c->d_Useg, c->d_hA_in1, c->d_hP_in1, c->d_hA_out1,
                     c->d_hP_out1, c->d_hstats, c->d_tc_hi, c->d_tc_lo, c->d_tc_B, c->d_tc_ks,
-                    c->d_tc_grp, c->d_tc_has, c->d_small_count, c->d_small_taps, c->d_cr_w};
+                    c->d_tc_grp, c->d_tc_has, c->d_small_count, c->d_small_taps, c->d_cr_w, c->d_tS, c->d_tS0,
+                    c->d_ttw};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
@@ -746,10 +886,6 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
         CK_INIT(cudaGetDevice(&dev));
         CK_INIT(cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, dev));
     }
-    // stats records: the larger of the tiled epilogue's blocks and one per SM-resident CTA
-    c->n_part_blocks = std::max(std::max(epilogue_blocks(H, W), ring_epilogue_blocks(H, W)), 8 * c->num_sms);
-    ALLOC(c->d_partials, (size_t)c->n_part_blocks * C * 5);
-
     // circular-mean tables
     {
         std::vector<float> trig(2 * (size_t)H + 2 * (size_t)W);
@@ -771,6 +907,52 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
     for (int k = 0; k < NC; k++) {
         const int sc = c->conv_src[k];
         klist[sc][kcount[sc]++] = k;
+    }
+
+    // Windows of spectral transforms where the time models say so: instead of the FFT
+    // path's three passes in worlds without alpha decisions, and instead of the
+    // direct sums that AUTO falls back to.  The transforms round differently
+    // from the sums, so alpha tests that this could turn are decided by the sums
+    // (GuardParams); a world whose alpha tests potentials against (nearly) zero,
+    // where that would be every empty site, keeps the sums throughout, and so
+    // do ring worlds and an explicit LENIA_CONV_DIRECT.
+    const bool want_adj = cfg->max_rollout_steps > 0 && c->n_p == 0 && !cfg->maintain_genes;
+    if ((path == LENIA_CONV_FFT && !cfg->maintain_genes) ||
+        (path == LENIA_CONV_DIRECT && cfg->conv_path == LENIA_CONV_AUTO && !n_rings &&
+         (!cfg->maintain_genes || (epilogue_sites_supported(epi_params(c)) &&
+                                   !(cfg->alpha_on && fabsf(cfg->eps_u) < 1e-4f))))) {
+        memset(&c->tl, 0, sizeof(c->tl));
+        const double t_tile = tile_choose(&c->tl, H, W, kcount, c->max_R);
+        const double t_else = path == LENIA_CONV_FFT ? fft_passes_cost(H, W, C + NC) : direct_cost(H, W, NC, c->max_R);
+        c->tile = t_tile < t_else;
+    }
+    // stats records: the largest of the tiled epilogue's blocks, and the resident CTAs
+    c->n_part_blocks = std::max(std::max(epilogue_blocks(H, W), ring_epilogue_blocks(H, W)), kSitesBlocksPerSm * c->num_sms);
+
+    ALLOC(c->d_partials, (size_t)c->n_part_blocks * C * 5);
+
+    if (c->tile) {
+        // FP32 rounding of either form, for values in [0, 1] and the kernels' absolute
+        // weights (measured: at most 8e-7 direct, 2.5e-7 windows, for weights that sum to 1)
+        double wabs = 0.0;
+        for (const std::vector<double>& w : c->conv_w) {
+            double t = 0.0;
+            for (double v : w) t += fabs(v);
+            wabs = std::max(wabs, t);
+        }
+        c->guard_du = (float)(4e-6 * wabs);
+        int blocks = 0;
+        for (int ch = 0; ch < C; ch++) blocks += c->tl.g.tiles_x * c->tl.g.tiles_y * ((kcount[ch] + c->tl.kpb - 1) / c->tl.kpb);
+        c->gate_pays = blocks > c->num_sms * (c->tl.N == 128 ? 3 : 8);
+        c->tl.C = C;
+        memcpy(c->tl.kcount, kcount, sizeof(kcount));
+        memcpy(c->tl.klist, klist, sizeof(klist));
+        const lenia_status ts = build_tiles(c, s);
+        if (ts != LENIA_OK) {
+            fprintf(stderr, "lenia_init: %s\n", c->err.c_str());
+            lenia_destroy(c);
+            return ts;
+        }
     }
 
     // small worlds with global genes on the direct route: their rollouts run
@@ -938,7 +1120,7 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
         c->tp.n_dy = n_dy;
         c->tp.n_groups = (int)grp.size() / (2 + TC_NG);
         c->tp.terms = path == LENIA_CONV_DIRECT_BF16X3 ? 3 : 1;
-    } else if (path == LENIA_CONV_FFT) {
+    } else if (path == LENIA_CONV_FFT && (!c->tile || want_adj)) {
         const int M = W / 2, HS = H / 2 + 1;
         ALLOC(c->d_Ahat, (size_t)C * H * M);
         ALLOC(c->d_Uhat, (size_t)NC * H * M);
@@ -950,32 +1132,7 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
         CK_INIT(cudaMemcpy(c->d_twM, twM.data(), twM.size() * sizeof(float2), cudaMemcpyHostToDevice));
         CK_INIT(cudaMemcpy(c->d_twW, twW.data(), twW.size() * sizeof(float2), cudaMemcpyHostToDevice));
         CK_INIT(cudaMemcpy(c->d_twH, twH.data(), twH.size() * sizeof(float2), cudaMemcpyHostToDevice));
-        // FP64 spectra of every kernel on the device, rounded once to FP32
-        std::vector<double> cosH(H), cosW(W);
-        for (int m = 0; m < H; m++) cosH[m] = cos(kTwoPi * m / H);
-        for (int m = 0; m < W; m++) cosW[m] = cos(kTwoPi * m / W);
-        double *d_cosH = nullptr, *d_cosW = nullptr, *d_Kd = nullptr, *d_T = nullptr;
-        const size_t kmax = (size_t)(2 * c->max_R + 1) * (2 * c->max_R + 1);
-        bool ok = cudaMalloc(&d_cosH, H * sizeof(double)) == cudaSuccess &&
-                  cudaMalloc(&d_cosW, W * sizeof(double)) == cudaSuccess &&
-                  cudaMalloc(&d_Kd, kmax * sizeof(double)) == cudaSuccess &&
-                  cudaMalloc(&d_T, (size_t)(2 * c->max_R + 1) * (M + 1) * sizeof(double)) == cudaSuccess;
-        cudaError_t e = ok ? cudaSuccess : cudaErrorMemoryAllocation;
-        if (e == cudaSuccess) e = cudaMemcpy(d_cosH, cosH.data(), H * sizeof(double), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(d_cosW, cosW.data(), W * sizeof(double), cudaMemcpyHostToDevice);
-        for (int k = 0; k < NC && e == cudaSuccess; k++) {
-            e = cudaMemcpyAsync(d_Kd, c->conv_w[k].data(), c->conv_w[k].size() * sizeof(double),
-                                cudaMemcpyHostToDevice, s);
-            if (e == cudaSuccess)
-                e = launch_spectra(d_Kd, c->conv_R[k], H, W, d_cosH, d_cosW, d_T,
-                                   c->d_S + (size_t)k * (M + 1) * HS, s);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        }
-        cudaFree(d_cosH);
-        cudaFree(d_cosW);
-        cudaFree(d_Kd);
-        cudaFree(d_T);
-        CK_INIT(e);
+        CK_INIT(build_spectra(c, H, W, c->d_S, s));
         memset(&c->fp, 0, sizeof(c->fp));
         c->fp.Ahat = c->d_Ahat;
         c->fp.Uhat = c->d_Uhat;
@@ -994,7 +1151,7 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
         memcpy(c->fp.klist, klist, sizeof(klist));
     }
     // adjoint buffers (global genes only; gene maps make alpha decisions)
-    if (cfg->max_rollout_steps > 0 && c->n_p == 0 && !cfg->maintain_genes) {
+    if (want_adj) {
         c->adj = true;
         c->max_steps = cfg->max_rollout_steps;
         c->ckpt = cfg->ckpt_every > 0 ? cfg->ckpt_every : 8;

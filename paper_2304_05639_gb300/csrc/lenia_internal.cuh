@@ -265,6 +265,60 @@ struct FftParams {
     int klist[kMaxChannels][kMaxKernels];
 };
 
+// Spectral convolution in overlapping N x N windows (tile_conv.cu): the
+// geometry of one world's windows, which depends on its sides and radius.
+struct TileGeom {
+    int vx, vy;                // output sites per window
+    int halo_x, halo_y;
+    int cut_x, cut_y;          // window index i stands for offset i below the cut, i - N from it on
+    int tiles_x, tiles_y;
+};
+// One world of a batched launch (device memory).
+struct TileWorld {
+    const float* A;
+    float* U;
+    const float* S;
+    const float* S0;
+    TileGeom g;
+};
+struct TileParams {
+    const float* A;            // [C][H][W] (adjoint: the K gradient planes)
+    float* U;                  // [K][H][W] potentials (adjoint: [C][H][W])
+    const float* add;          // adjoint: added to the output, [C][H][W] (nullable)
+    const float* S;            // [K] kernel spectra in task order, tile_spectrum_floats(N) each
+    const float* S0;           // [K][N] mirrored share of the packed column 0
+    const float2* tw;          // [8][N / 8] exp(-2 pi i n1 b / N)
+    int N, H, W, C;
+    TileGeom g;
+    // worlds batched in one launch (grid y: world * C + channel), or null; every
+    // window count is at most `tiles`
+    const TileWorld* worlds;
+    int tiles, n_worlds;
+    int aligned;               // every listed A and U is 8-byte aligned
+    // a gene plane: windows without a value above gate_eps within gate_r of their
+    // output are skipped and their potentials left as they are; or null
+    const float* gate;
+    float gate_eps;
+    int gate_r;
+    int kpb;                   // kernels per block
+    int vec2, vec2o;           // input / output 8-byte aligned (set by the launcher)
+    int kcount[kMaxChannels];
+    int klist[kMaxChannels][kMaxKernels];
+};
+// Window geometry for an H x W torus and radius R; false where N cannot serve it.
+bool tile_plan(TileParams* p, int N, int H, int W, int R);
+// The faster window size and kernels per block (in p; the model's time in us, or
+// infinity where no window serves R), and the models of the other routes.
+// (n_worlds: worlds of that shape in one launch)
+double tile_choose(TileParams* p, int H, int W, const int* kcount, int R, int n_worlds = 1);
+double fft_passes_cost(int H, int W, int planes);      // planes: channels + convolution outputs
+double direct_cost(int H, int W, int planes, int R);   // planes: convolution outputs
+size_t tile_spectrum_floats(int N);
+// S: [kx][ky] of the N x N torus as launch_spectra writes it
+cudaError_t launch_tile_spectra(int N, const float* S, float* out, float* out0, cudaStream_t s);
+cudaError_t launch_tile_conv(const TileParams& p, cudaStream_t s);
+cudaError_t launch_tile_conv_adj(const TileParams& p, cudaStream_t s);
+
 // Adjoint of one step with global genes.
 struct AdjParams {
     const float* A;            // step input A_t [C][H][W]
@@ -325,11 +379,31 @@ cudaError_t launch_epilogue_queue(const EpiParams& p, const QueueWorld* worlds, 
 // the driver does not provide it).
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 cudaError_t launch_epilogue_rows(const EpiParams& p, int num_sms, int* status, cudaStream_t s, int* n_blocks);
+// The per-site rule for any kernel and channel count (mu and sigma, or mu, sigma and h
+// per site with diffusion radius 1 or 2 and eps_p = 0, or global genes;
+// epilogue_sites.cu).  A, P, U and the outputs 16-byte aligned.
+bool epilogue_sites_supported(const EpiParams& p);
+// whether sites without a first gene around them are known to have alpha = 0
+bool epilogue_gated(const EpiParams& p);
+// The direct sums, for alpha decisions that the windows' rounding could turn:
+// where a potential within du of its value would change the test, that
+// potential is summed directly.
+struct GuardParams {
+    const float* w;            // as ConvParams
+    const int *w_off, *yr, *yr_off;
+    int R[kMaxKernels];
+    float du;                  // 0: no guard
+};
+// fast: the streaming kernel's reciprocals and exponential, else divisions and expf
+cudaError_t launch_epilogue_sites(const EpiParams& p, bool fast, const GuardParams* guard, int n_worlds, int max_blocks,
+                                  cudaStream_t s, int* n_blocks);
 bool fft_size_supported(int H, int W);
 int epilogue_blocks(int H, int W);
 // The batched-worlds runner's view of a context: its convolution and epilogue
 // parameters (false unless the context is on the FFT path).
 struct lenia_ctx_view {
+    bool tile;                 // convolves in windows (tl; fp holds no buffers)
+    TileParams tl;
     FftParams fp;
     EpiParams ep;
     size_t N;
@@ -339,6 +413,8 @@ struct lenia_ctx_view {
 struct lenia_ctx;
 namespace lenia {
 bool ctx_view(lenia_ctx* c, lenia_ctx_view* v);
+// Window size for a world of a group of n_worlds (rebuilds its spectra); waits for the work.
+cudaError_t ctx_group_tiles(lenia_ctx* c, int n_worlds, cudaStream_t s);
 // batched worlds: one tiled-epilogue launch over n_worlds (grid z), pointer lists in EpiParams
 bool epilogue_batch_supported(const EpiParams& p);
 // br: rows per thread of the one-kernel tiled epilogue (1, 2 or 4)

@@ -1087,47 +1087,47 @@ cudaError_t launch_stats_partials(const float* A, int C, int H, int W, const flo
     return cudaGetLastError();
 }
 
-// Final reduction, one block of 1024 threads: for each of the C*5 sums,
-// 64 threads stride over the block records (fixed order), then two fixed
-// shuffle trees and one add, all in compensated FP32 pairs.  out[c] = (mass,
-// centre y, centre x), centres from the circular mean atan2(sum A sin, sum A
-// cos) scaled to [0, n) (FP64, on the pairs' values).
-__global__ void __launch_bounds__(1024) k_stats_final(const float2* partials, int n_blocks, int C,
-                                                      int H, int W, float* out)
+// Final reduction, one block per channel: 192 threads per sum stride over the
+// block records (fixed order), then shuffle trees and an ordered sum of the six
+// warps, all in compensated FP32 pairs.  out[c] = (mass, centre y, centre x),
+// centres from the circular mean atan2(sum A sin, sum A cos) scaled to [0, n)
+// (FP64, on the pairs' values).
+constexpr int SF_T = 192, SF_W = SF_T / 32;
+__global__ void __launch_bounds__(5 * SF_T) k_stats_final(const float2* partials, int n_blocks, int C, int H, int W,
+                                                          float* out)
 {
     pdl_enter();
-    __shared__ float2 part[32];
-    __shared__ float2 tot[kMaxChannels * 5];
-    const int nv = C * 5;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int v0 = 0; v0 < nv; v0 += 16) {
-        const int v = v0 + (threadIdx.x >> 6);     // 16 values per pass, 64 threads each
-        const int stripe = threadIdx.x & 63;
-        float2 s = make_float2(0.f, 0.f);
-        if (v < nv)
-            for (int b = stripe; b < n_blocks; b += 64 * 8) {
-                // eight records in flight per thread, added in block order
-                float2 x[8];
+    __shared__ float2 part[5 * SF_W];
+    __shared__ float2 tot[5];
+    const int c = blockIdx.x, nv = C * 5;
+    const int v = threadIdx.x / SF_T, stripe = threadIdx.x - v * SF_T;
+    const float2* src = partials + c * 5 + v;
+    float2 s = make_float2(0.f, 0.f);
+    for (int b = stripe; b < n_blocks; b += SF_T * 8) {
+        // eight records in flight per thread, added in block order
+        float2 x[8];
 #pragma unroll
-                for (int u = 0; u < 8; u++)
-                    x[u] = b + 64 * u < n_blocks ? partials[(size_t)(b + 64 * u) * nv + v] : make_float2(0.f, 0.f);
+        for (int u = 0; u < 8; u++)
+            x[u] = b + SF_T * u < n_blocks ? src[(size_t)(b + SF_T * u) * nv] : make_float2(0.f, 0.f);
 #pragma unroll
-                for (int u = 0; u < 8; u++) s = ff_add(s, x[u]);
-            }
-        for (int off = 16; off > 0; off >>= 1) s = ff_add(s, ff_shfl_down(s, off));
-        if (lane == 0) part[warp] = s;
-        __syncthreads();
-        if (threadIdx.x < 16 && v0 + threadIdx.x < nv)
-            tot[v0 + threadIdx.x] = ff_add(part[2 * threadIdx.x], part[2 * threadIdx.x + 1]);
-        __syncthreads();
+        for (int u = 0; u < 8; u++) s = ff_add(s, x[u]);
     }
-    if (threadIdx.x < 2 * C) stats_centre(tot, threadIdx.x >> 1, threadIdx.x & 1, H, W, out);
+    for (int off = 16; off > 0; off >>= 1) s = ff_add(s, ff_shfl_down(s, off));
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x < 5) {
+        float2 t = part[threadIdx.x * SF_W];
+        for (int w = 1; w < SF_W; w++) t = ff_add(t, part[threadIdx.x * SF_W + w]);
+        tot[threadIdx.x] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) stats_centre(tot, 0, threadIdx.x, H, W, out + c * 3);
 }
 
 cudaError_t launch_stats_final(const float2* partials, int n_blocks, int C, int H, int W,
                                float* out, cudaStream_t s)
 {
-    launch_pdl(k_stats_final, 1, 1024, 0, s, partials, n_blocks, C, H, W, out);
+    launch_pdl(k_stats_final, C, 5 * SF_T, 0, s, partials, n_blocks, C, H, W, out);
     return cudaGetLastError();
 }
 
