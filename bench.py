@@ -346,7 +346,8 @@ def small_legs(torch, lenia, inputs, stream, fp32_peak=None):
              "conv_path": "fft" if path == lenia.CONV_FFT else "direct",
              "rollout": {lenia.ROUTE_STEPS: f"{lps} launches per step, pairs of steps replayed from a CUDA graph",
                          lenia.ROUTE_COOPERATIVE: "one cooperative launch",
-                         lenia.ROUTE_CLUSTER: "one thread-block cluster"}.get(route, "?"),
+                         lenia.ROUTE_CLUSTER: "one thread-block cluster",
+                         lenia.ROUTE_BLOCK: "one thread block"}.get(route, "?"),
              "launches_per_step": lps if route == lenia.ROUTE_STEPS else 1.0 / steps,
              "alg_bytes_per_site": alg, "frac_of_hbm": v * alg / 1e9 / _peaks()[0]}
         if fp32_peak and path == lenia.CONV_FFT:
@@ -531,7 +532,8 @@ def direct_leg(torch, lenia, inputs, stream, fp32_peak=None, bf16_peak=None, ste
         torch.cuda.synchronize()
         lenia.lenia_check(ctx)
         route = {lenia.ROUTE_STEPS: "launches per step (graph)", lenia.ROUTE_COOPERATIVE: "one cooperative launch",
-                 lenia.ROUTE_CLUSTER: "one thread-block cluster"}.get(lenia.lenia_rollout_route(ctx), "?")
+                 lenia.ROUTE_CLUSTER: "one thread-block cluster",
+                 lenia.ROUTE_BLOCK: "one thread block"}.get(lenia.lenia_rollout_route(ctx), "?")
         out["c1_direct"] = {"workload": "64x64, 1 channel, 1 kernel R=13, global genes, 100-step rollout, direct path",
                             "us_per_step": e0.elapsed_time(e1) * 1e3 / 100, "route": route}
     except StopIteration:

@@ -187,6 +187,10 @@ LENIA_API lenia_status lenia_step(lenia_ctx* ctx, const float* A_in, const float
  * in one thread-block cluster of 16 (or 8) blocks that keep the world in
  * shared memory and meet at the cluster barrier: dense (2R+1)^2 sums in
  * another order, equal to repeated lenia_step calls to FP32 rounding.
+ * One-channel worlds of 64^2 or 128^2 sites with global genes and at most four
+ * kernels on the FFT path run such a rollout in one thread block that keeps the
+ * world in registers and transforms it in shared memory; equal to repeated
+ * lenia_step calls to FP32 rounding.
  * lenia_rollout_route tells which form a context uses. */
 LENIA_API lenia_status lenia_rollout(lenia_ctx* ctx, float* A, float* P, int32_t n_steps,
                            float* stats_out, void* stream);
@@ -388,11 +392,12 @@ LENIA_API int32_t lenia_conv_path(const lenia_ctx* ctx);
 /* Form of lenia_rollout (without stats_out, n_steps >= 2) for this context:
  * LENIA_ROUTE_STEPS (launches per step, pairs of steps replayed from a CUDA
  * graph), LENIA_ROUTE_COOPERATIVE (one cooperative launch) or
- * LENIA_ROUTE_CLUSTER (one thread-block cluster; a caller's A that is not
+ * LENIA_ROUTE_BLOCK (one thread block), LENIA_ROUTE_CLUSTER (one thread-block cluster; a caller's A that is not
  * 16-byte aligned takes the cooperative launch instead); -1 for NULL. */
 #define LENIA_ROUTE_STEPS 0
 #define LENIA_ROUTE_COOPERATIVE 1
 #define LENIA_ROUTE_CLUSTER 2
+#define LENIA_ROUTE_BLOCK 3
 LENIA_API int32_t lenia_rollout_route(const lenia_ctx* ctx);
 
 /* Number of CUDA kernel launches one lenia_step enqueues (with stats). */

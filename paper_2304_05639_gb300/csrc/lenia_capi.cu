@@ -56,6 +56,7 @@ struct lenia_ctx {
     // faster than the path's other form
     bool tile = false;
     TileParams tl;
+    bool block = false;                    // rollouts in one block (the torus is one window)
     bool gate_pays = false;                // more windows than run at once: skipping some saves time
     float guard_du = 0.f;                  // how far the windows' and the direct sums' potentials may be apart
     float* d_tS = nullptr;
@@ -715,6 +716,7 @@ int32_t lenia_conv_path(const lenia_ctx* ctx) { return ctx ? ctx->path : -1; }
 int32_t lenia_rollout_route(const lenia_ctx* ctx)
 {
     if (!ctx) return -1;
+    if (ctx->block) return LENIA_ROUTE_BLOCK;
     return ctx->cr_Q ? LENIA_ROUTE_CLUSTER : (ctx->small ? LENIA_ROUTE_COOPERATIVE : LENIA_ROUTE_STEPS);
 }
 
@@ -925,6 +927,14 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
         const double t_tile = tile_choose(&c->tl, H, W, kcount, c->max_R);
         const double t_else = path == LENIA_CONV_FFT ? fft_passes_cost(H, W, C + NC) : direct_cost(H, W, NC, c->max_R);
         c->tile = t_tile < t_else;
+        // one-channel worlds of one window: whole rollouts in one block, so the
+        // window is the torus whatever a single step would take
+        c->block = path == LENIA_CONV_FFT && c->n_p == 0 && !n_rings && tile_rollout_supported(H, W, C, K) &&
+                   tile_plan(&c->tl, H, H, W, c->max_R);
+        if (c->block) {
+            c->tl.kpb = NC;
+            c->tile = true;
+        }
     }
     // stats records: the largest of the tiled epilogue's blocks, and the resident CTAs
     c->n_part_blocks = std::max(std::max(epilogue_blocks(H, W), ring_epilogue_blocks(H, W)), kSitesBlocksPerSm * c->num_sms);
@@ -1274,6 +1284,26 @@ lenia_status lenia_rollout(lenia_ctx* c, float* A, float* P, int32_t n_steps, fl
         cp.dt = c->cfg.dt;
         ProfScope ps(c, KIND_DIRECT, s);
         CUDA_OR_FAIL(c, launch_cluster_rollout(cp, s));
+        return LENIA_OK;
+    }
+    if (c->block && !stats_out && n_steps >= 2) {
+        TileRolloutParams tp;
+        memset(&tp, 0, sizeof(tp));
+        tp.A = A;
+        tp.S = c->d_tS;
+        tp.S0 = c->d_tS0;
+        tp.tw = c->d_ttw;
+        tp.K = c->cfg.n_kernels;
+        tp.n_steps = n_steps;
+        tp.growth_form = c->cfg.growth_form;
+        tp.dt = c->cfg.dt;
+        for (int k = 0; k < tp.K; k++) {
+            tp.mu[k] = c->kt.mu[k];
+            tp.rsigma[k] = (float)(1.0 / (double)c->kt.sigma[k]);
+            tp.h[k] = c->kt.h[k];
+        }
+        ProfScope ps(c, KIND_COLS, s);
+        CUDA_OR_FAIL(c, launch_tile_rollout(tp, c->tl.N, s));
         return LENIA_OK;
     }
     if (c->small && !stats_out && n_steps >= 2) {

@@ -319,6 +319,21 @@ cudaError_t launch_tile_spectra(int N, const float* S, float* out, float* out0, 
 cudaError_t launch_tile_conv(const TileParams& p, cudaStream_t s);
 cudaError_t launch_tile_conv_adj(const TileParams& p, cudaStream_t s);
 
+// Rollouts of one-channel worlds with global genes whose torus is one window (64^2
+// or 128^2, at most kTileRolloutKernels kernels), in one block.
+constexpr int kTileRolloutKernels = 4;
+struct TileRolloutParams {
+    float* A;                  // [N][N], in and out
+    const float* S;            // as TileParams, of that window size
+    const float* S0;
+    const float2* tw;
+    int K, n_steps, growth_form;
+    float dt;
+    float mu[kTileRolloutKernels], rsigma[kTileRolloutKernels], h[kTileRolloutKernels];
+};
+bool tile_rollout_supported(int H, int W, int C, int K);
+cudaError_t launch_tile_rollout(const TileRolloutParams& p, int N, cudaStream_t s);
+
 // Adjoint of one step with global genes.
 struct AdjParams {
     const float* A;            // step input A_t [C][H][W]

@@ -642,6 +642,135 @@ __global__ void __launch_bounds__(2 * N, N == 128 ? 3 : (ADJ ? 6 : 8)) k_tile_co
     }
 }
 
+// A whole rollout of a one-channel world with global genes whose torus is one
+// window (64^2 or 128^2): one block, every step in shared memory and registers.
+// A thread holds the same eight pairs of sites of its rows through the whole
+// rollout: they are what its last inverse pass yields and its first forward
+// pass takes, so a step is the seven in-place passes above with a barrier after
+// each, the growth in registers, and nothing in global memory.  What bounds it
+// is the latency of those passes (64^2, one kernel: see the launch's comment).
+template <int N, bool ONE>
+__global__ void __launch_bounds__(4 * N) k_tile_rollout(const __grid_constant__ TileRolloutParams p)
+{
+    pdl_enter();
+    using X = TC<N>;
+    constexpr int T = 4 * N, NW = T / 32, RPW = 32 / X::RR, NR = N / (RPW * NW);
+    extern __shared__ __align__(128) unsigned char buf[];
+    float2* F0 = reinterpret_cast<float2*>(buf + (size_t)N * X::M * 8);
+    float2* twc = F0 + N;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int m1 = lane % X::RR;
+    for (int i = threadIdx.x; i < N; i += T) twc[i] = __ldg(&p.tw[i]);
+    int ys[NR], base[NR];
+    float2 a[NR][8];                                     // the state: rows ys[i], pairs m1 + RR m2
+#pragma unroll
+    for (int i = 0; i < NR; i++) {
+        ys[i] = (warp + i * NW) * RPW + lane / X::RR;
+        base[i] = ys[i] * X::PITCH + ((m1 * 8 + (m1 & 7)) ^ row_sw(ys[i])) * 8;
+#pragma unroll
+        for (int m2 = 0; m2 < 8; m2++) {
+            const float* q = p.A + (size_t)ys[i] * N + 2 * (m1 + X::RR * m2);
+            a[i][m2] = make_float2(q[0], q[1]);
+        }
+    }
+    // this thread's column task, one per thread
+    static_assert(8 * X::CH == NW, "one column task per thread");
+    const int b = warp % 8, c = (warp / 8) * 32 + lane;
+    float s1[X::CA];
+    if (ONE) spectrum_of<N>(p.S, c, b, s1);
+    __syncthreads();
+    for (int t = 0; t < p.n_steps; t++) {
+#pragma unroll
+        for (int i = 0; i < NR; i++) {
+            float2 v[8];
+#pragma unroll
+            for (int m2 = 0; m2 < 8; m2++) v[m2] = a[i][m2];
+            DFT<8, false, true>::run(v);
+#pragma unroll
+            for (int j = 0; j < 8; j++) st2(buf, base[i] ^ (j * 8), v[j]);
+        }
+        __syncthreads();
+        for (int u = warp; u < 4 * (N / 32); u += NW) {
+            const int y = (u >> 2) * 32 + lane;
+            switch (u & 3) {
+                case 0: rows_fwd<N, 0>(buf, y); break;
+                case 1: rows_fwd<N, 1>(buf, y); break;
+                case 2: rows_fwd<N, 2>(buf, y); break;
+                default: rows_fwd<N, 3>(buf, y); break;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = warp; u < X::CA * X::CH; u += NW) cols8<N, false>(buf, u % X::CA, (u / X::CA) * 32 + lane);
+        __syncthreads();
+        float2 f[X::CA];
+        cols_fwd<N>(buf, twc, c, b, f);
+        if (c == 0) {
+#pragma unroll
+            for (int i = 0; i < X::CA; i++) F0[i * 8 + b] = f[i];
+        }
+        float2 acc[NR][8];
+        for (int k = 0; k < (ONE ? 1 : p.K); k++) {
+            __syncthreads();                             // F0 complete; the last kernel's rows are read
+            float2 v[X::CA];
+#pragma unroll
+            for (int i = 0; i < X::CA; i++) v[i] = f[i];
+            if (ONE && c != 0) {
+#pragma unroll
+                for (int i = 0; i < X::CA; i++) v[i] = cscale(v[i], s1[i]);
+            } else {
+                spectral_product<N>(p.S + (size_t)k * N * X::M, p.S0 + (size_t)k * N, F0, c, b, v);
+            }
+            cols_inv<N>(buf, twc, c, b, v);
+            __syncthreads();
+#pragma unroll
+            for (int u = warp; u < X::CA * X::CH; u += NW) cols8<N, true>(buf, u % X::CA, (u / X::CA) * 32 + lane);
+            __syncthreads();
+            for (int u = warp; u < 4 * (N / 32); u += NW) {
+                const int y = (u >> 2) * 32 + lane;
+                switch (u & 3) {
+                    case 0: rows_inv<N, 0>(buf, y); break;
+                    case 1: rows_inv<N, 1>(buf, y); break;
+                    case 2: rows_inv<N, 2>(buf, y); break;
+                    default: rows_inv<N, 3>(buf, y); break;
+                }
+            }
+            __syncthreads();
+            const float m = p.mu[k], rs = p.rsigma[k], h = p.h[k];
+            auto growth = [&](float u) {
+                const float z = (u - m) * rs;
+                const float g = ex2_approx(-0.721347520444481703680f * (z * z));     // -log2(e) / 2
+                return p.growth_form == 0 ? h * fmaf(2.f, g, -1.f) : h * g;
+            };
+#pragma unroll
+            for (int i = 0; i < NR; i++) {
+#pragma unroll
+                for (int j = 0; j < 8; j++) v[j] = ld2(buf, base[i] ^ (j * 8));
+                DFT<8, true, true>::run(v);
+#pragma unroll
+                for (int j = 0; j < 8; j++) {
+                    const float2 g = make_float2(growth(v[j].x), growth(v[j].y));
+                    acc[i][j] = k == 0 ? g : make_float2(acc[i][j].x + g.x, acc[i][j].y + g.y);
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < NR; i++)
+#pragma unroll
+            for (int j = 0; j < 8; j++)
+                a[i][j] = make_float2(__saturatef(fmaf(p.dt, acc[i][j].x, a[i][j].x)),
+                                      __saturatef(fmaf(p.dt, acc[i][j].y, a[i][j].y)));
+    }
+#pragma unroll
+    for (int i = 0; i < NR; i++)
+#pragma unroll
+        for (int m2 = 0; m2 < 8; m2++) {
+            float* q = p.A + (size_t)ys[i] * N + 2 * (m1 + X::RR * m2);
+            q[0] = a[i][m2].x;
+            q[1] = a[i][m2].y;
+        }
+}
+
 // Kernel spectra in the order the column tasks read them, from S[kx][ky] of the
 // N x N torus (kx, ky in 0..N/2): row ky = a 8 + b of column c goes to
 // [b][a / 4][c][a % 4]; the factor 1/2 undoes the doubled forward spectrum.
@@ -758,6 +887,23 @@ cudaError_t launch_tile_conv(const TileParams& p0, cudaStream_t s)
     p.vec2 = p.worlds ? p.aligned : ((uintptr_t)p.A & 7) == 0;
     p.vec2o = p.worlds ? p.aligned : ((uintptr_t)p.U & 7) == 0;
     return p.N == 128 ? launch_n<128, false>(p, s) : launch_n<64, false>(p, s);
+}
+
+bool tile_rollout_supported(int H, int W, int C, int K) { return H == W && (H == 64 || H == 128) && C == 1 && K <= kTileRolloutKernels; }
+
+template <int N, bool ONE>
+static cudaError_t launch_rollout_n(const TileRolloutParams& p, cudaStream_t s)
+{
+    cudaError_t e = smem_limit<k_tile_rollout<N, ONE>>(TC<N>::SMEM);
+    if (e != cudaSuccess) return e;
+    launch_pdl(k_tile_rollout<N, ONE>, dim3(1), dim3(4 * N), TC<N>::SMEM, s, p);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_tile_rollout(const TileRolloutParams& p, int N, cudaStream_t s)
+{
+    if (N == 64) return p.K == 1 ? launch_rollout_n<64, true>(p, s) : launch_rollout_n<64, false>(p, s);
+    return p.K == 1 ? launch_rollout_n<128, true>(p, s) : launch_rollout_n<128, false>(p, s);
 }
 
 cudaError_t launch_tile_conv_adj(const TileParams& p0, cudaStream_t s)

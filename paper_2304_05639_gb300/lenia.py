@@ -19,7 +19,7 @@ from . import inputs as _inputs
 
 LENIA_OK, LENIA_EINVAL, LENIA_ENOMEM, LENIA_ECUDA, LENIA_ETIMEOUT, LENIA_ENOTSUP = range(6)
 CONV_AUTO, CONV_FFT, CONV_DIRECT, CONV_DIRECT_BF16, CONV_DIRECT_BF16X3 = 0, 1, 2, 3, 4
-ROUTE_STEPS, ROUTE_COOPERATIVE, ROUTE_CLUSTER = 0, 1, 2
+ROUTE_STEPS, ROUTE_COOPERATIVE, ROUTE_CLUSTER, ROUTE_BLOCK = 0, 1, 2, 3
 
 # Every function the header declares (checked by the tests).
 EXPORTS = ("lenia_init", "lenia_step", "lenia_rollout", "lenia_backward", "lenia_stats",
@@ -392,7 +392,7 @@ def lenia_conv_path(ctx) -> int:
 
 
 def lenia_rollout_route(ctx) -> int:
-    """ROUTE_STEPS, ROUTE_COOPERATIVE or ROUTE_CLUSTER: the form of lenia_rollout."""
+    """ROUTE_STEPS, ROUTE_COOPERATIVE, ROUTE_CLUSTER or ROUTE_BLOCK: the form of lenia_rollout."""
     return load().lenia_rollout_route(ctx)
 
 

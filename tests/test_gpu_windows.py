@@ -146,3 +146,37 @@ def test_window_gradients_match_direct(shape):
         f.close()
     for a, b in zip(*out):
         assert float((a - b).norm()) <= 1e-4 * float(b.norm())
+
+
+@pytest.mark.parametrize("side,n_kernels,form", [(64, 1, 0), (64, 2, 1), (64, 4, 0), (128, 1, 1), (128, 3, 0)])
+def test_one_block_rollout_matches_oracle_and_steps(side, n_kernels, form):
+    """Whole rollouts in one block: 2 steps against the oracle and 7 against
+    repeated single steps, aligned and 4 bytes past a 16-byte boundary."""
+    torch = torch_mod()
+    w = inputs.single_kernel_global(H=side, W=side, R=13, patch=side, sigma=0.05, mu=0.42)
+    w.kernels = [inputs.KernelDesc(0, 0, 13 - 2 * i, inputs.KERNEL_SHELLS, (1.0, 0.5)[:1 + i % 2], h=1.0 - 0.2 * i,
+                                   mu=0.42 + 0.02 * i, sigma=0.05 + 0.01 * i) for i in range(n_kernels)]
+    w.growth_form = form
+    cfg, ks = lenia.config_from_world(w)
+    ctx = lenia.lenia_init(cfg, ks)
+    try:
+        assert lenia.lenia_rollout_route(ctx) == lenia.ROUTE_BLOCK
+        A = to_dev(w.A)
+        lenia.lenia_rollout(ctx, A, None, 2)
+        ref = oracle.rollout(w, 2)[0]
+        assert np.abs(A.cpu().numpy() - ref).max() <= 2 * TOL_STEP
+        S, B = to_dev(w.A), to_dev(w.A)
+        for _ in range(7):
+            T = torch.empty_like(S)
+            lenia.lenia_step(ctx, S, None, T, None)
+            S = T
+        lenia.lenia_rollout(ctx, B, None, 7)
+        flat = torch.empty(S.numel() + 1, device="cuda")
+        D = flat[1:].view_as(S)
+        D.copy_(to_dev(w.A))
+        lenia.lenia_rollout(ctx, D, None, 7)
+        torch.cuda.synchronize()
+        assert torch.equal(B, D)
+        assert float((S - B).abs().max()) <= 7 * TOL_STEP
+    finally:
+        lenia.lenia_destroy(ctx)
