@@ -609,6 +609,52 @@ __global__ void __launch_bounds__(256, 3) k_epilogue_rings(EpiParams p)
         }
         cp_async_commit();
     };
+    const int tid = ty * EP_TX + tx;
+    // Where no site of the block has a first gene above eps_p around it, alpha is false
+    // at all of them: the genes become zero and the update is the constant, and
+    // neither the other planes nor the potentials are needed (on a world a fifth
+    // full, two thirds of the blocks).  Delta_sum needs every site's growth.
+    const bool gate = p.maintain && eps_p >= 0.f && !p.empty_out;
+    if (gate) {
+        const float* g0 = p.P;
+        bool any = __ldg(g0 + g_r0 + g_c0) > eps_p;
+        if (hc) any |= __ldg(g0 + g_r0 + g_c1) > eps_p;
+        if (hr) any |= __ldg(g0 + g_r1 + g_c0) > eps_p;
+        if (hr && hc) any |= __ldg(g0 + g_r1 + g_c1) > eps_p;
+        if (!__syncthreads_or(any)) {
+            if (p.P_out) {
+                const int w = W - x0 < EP_TX ? W - x0 : EP_TX;            // a multiple of 4
+                if (((uintptr_t)p.P_out & 15) == 0) {
+                    const int q = tid & 7, row = (tid >> 3) & 7;
+                    if (4 * q < w && y0 + row < H)
+                        for (int pk = tid >> 6; pk < NP * KT; pk += 4)
+                            *reinterpret_cast<float4*>(p.P_out + (size_t)pk * N + (size_t)(y0 + row) * W + x0 + 4 * q) =
+                                make_float4(0.f, 0.f, 0.f, 0.f);
+                } else if (in) {
+                    for (int pk = 0; pk < NP * KT; pk++) p.P_out[(size_t)pk * N + i] = 0.f;
+                }
+            }
+            float st[CT * 5];
+#pragma unroll
+            for (int c = 0; c < CT; c++) {
+                float an = 0.f;
+                if (in) {
+                    an = fminf(fmaxf(__ldg(&p.A[(size_t)c * N + i]) + p.dt * p.acc0[c], 0.f), 1.f);
+                    p.A_out[(size_t)c * N + i] = an;
+                }
+                if (p.partials) {
+                    st[c * 5 + 0] = an;
+                    st[c * 5 + 1] = an * __ldg(&p.sin_y[yc]);
+                    st[c * 5 + 2] = an * __ldg(&p.cos_y[yc]);
+                    st[c * 5 + 3] = an * __ldg(&p.sin_x[xc]);
+                    st[c * 5 + 4] = an * __ldg(&p.cos_x[xc]);
+                }
+            }
+            if (in && p.alpha_out) p.alpha_out[i] = 0;
+            if (p.partials) block_stats<CT>(st, CT, p.partials);
+            return;
+        }
+    }
     // kernels in order of their source channel (the order of the sums below)
     if (ty == 0)
         for (int r = tx; r < NR; r += EP_TX) cnt_s[r] = p.ring_cnt[r];
@@ -619,7 +665,6 @@ __global__ void __launch_bounds__(256, 3) k_epilogue_rings(EpiParams p)
                 if (p.kt.src[k] == c) ord[n++] = k;
     }
     __syncthreads();
-    const int tid = ty * EP_TX + tx;
     // the thread's own ring potentials of one channel (no block barrier needed:
     // the thread that copies them is the one that reads them)
     auto stage_v = [&](int c) {
@@ -645,6 +690,14 @@ __global__ void __launch_bounds__(256, 3) k_epilogue_rings(EpiParams p)
         cp_async_wait_all();
         __syncthreads();            // kernel j staged; every thread is done with kernel j - 1's buffer
         if (j + 1 < KT) stage(ord[j + 1], tile[(j + 1) & 1]);
+        // a warp (a row of the block) whose sites have all lost alpha only clears
+        // the genes, and loads no more potentials of its own
+        if (gate && !__any_sync(0xffffffffu, alpha && in)) {
+            if (in && p.P_out)
+#pragma unroll
+                for (int pp = 0; pp < NP; pp++) p.P_out[(size_t)(pp * KT + k) * N + i] = 0.f;
+            continue;
+        }
         const float* T = tile[j & 1];
         float g[NP];
 #pragma unroll
