@@ -9,86 +9,100 @@
 //   dL/dmu_k    = sum gpre dt h_k F' g (U - mu) / sigma^2
 //   dL/dsigma_k = sum gpre dt h_k F' g (U - mu)^2 / sigma^3
 //   dL/dh_k     = sum gpre dt F(g)
-// as block partials in compensated FP32 pairs (hi + lo), reduced in a fixed
-// order by a second small kernel (one block per value).  The transposed convolution (gA_src += K~_k (x) gU_k; K~ is
-// point symmetric, so it is the same convolution) runs on the forward
-// machinery; its inverse row pass adds gpre (FFT path) or k_adjoint_gather
-// adds it (direct path).
+// as block partials in compensated FP32 pairs (hi + lo) that every reversed step
+// adds to, reduced once per pass in a fixed order (one block per value).  The
+// transposed convolution (gA_src += K~_k (x) gU_k; K~ is point symmetric, so
+// it is the same convolution) runs on the forward machinery; its inverse pass
+// adds gpre, or - where every gradient plane is convolved by itself - the next
+// reversed step gathers gpre + sum_k V_k as it reads.
 #include "lenia_internal.cuh"
 #include "ptx_util.cuh"
 
 namespace lenia {
 
-constexpr int ADJ_THREADS = 256;
+constexpr int ADJ_THREADS = 128;
+constexpr int ADJ_KB = 16;              // kernels whose gene terms meet in shared memory at a time
 constexpr float ADJ_HALF_LOG2E = 0.721347520444481703680f;   // 0.5 log2(e)
 
 // One site per thread; the growth is recomputed with the same arithmetic as
-// the forward streaming epilogue so that clip decisions match.
-__global__ void __launch_bounds__(ADJ_THREADS) k_adjoint_epilogue(AdjParams p)
+// the forward streaming epilogue so that clip decisions match.  A site's bumps
+// and channel sums sit in its thread's column of shared memory (kernel counts
+// and routing are run-time values), and the gene terms of ADJ_KB kernels at a
+// time are summed over the block from there: a warp per value, four loads and
+// one shuffle tree, instead of a tree per warp and value (256^2, 15 kernels:
+// 17 -> 8 us with the gather).
+__global__ void __launch_bounds__(ADJ_THREADS) k_adjoint_epilogue(const __grid_constant__ AdjParams p)
 {
     pdl_enter();
-    const int K = p.kt.K, C = p.kt.C;
+    extern __shared__ float adj_sm[];
+    const int K = p.kt.K, C = p.kt.C, tid = threadIdx.x;
+    float* bump = adj_sm;                                   // [K][T]
+    float* chan = bump + (size_t)K * ADJ_THREADS;           // [C][T]: pre-clip sum, then gpre
+    float* inc = chan + (size_t)C * ADJ_THREADS;            // [C][T]: dL/dA_{t+1}
+    float* red = inc + (size_t)C * ADJ_THREADS;             // [3 ADJ_KB][T]
     const size_t N = (size_t)p.H * p.W;
-    const size_t i = (size_t)blockIdx.x * ADJ_THREADS + threadIdx.x;
+    const size_t i = (size_t)blockIdx.x * ADJ_THREADS + tid;
     const bool valid = i < N;
-    __shared__ float red[ADJ_THREADS / 32][kMaxKernels * 3];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const size_t ic = valid ? i : N - 1;
+    const int lane = tid & 31, warp = tid >> 5;
 
-    float pre[kMaxChannels];
-    float gpre[kMaxChannels];
-    if (valid) {
-        for (int c = 0; c < C; c++) pre[c] = 0.f;
-        for (int k = 0; k < K; k++) {
-            const float u = __ldg(&p.U[(size_t)k * N + i]);
-            const float z = (u - p.kt.mu[k]) * rcp_approx(p.kt.sigma[k]);
-            const float g = ex2_approx(-ADJ_HALF_LOG2E * (z * z));
-            const float h = p.kt.h[k];
-            pre[p.kt.dst[k]] += p.growth_form == 0 ? fmaf(2.f * g, h, -h) : h * g;
-        }
-        for (int c = 0; c < C; c++) {
-            const float a = __ldg(&p.A[(size_t)c * N + i]) + p.dt * pre[c];
-            const float gA = __ldg(&p.gA_next[(size_t)c * N + i]);
-            gpre[c] = (a > 0.f && a < 1.f) ? gA : 0.f;
-            p.gpre[(size_t)c * N + i] = gpre[c];
-        }
+    for (int c = 0; c < C; c++) {
+        chan[c * ADJ_THREADS + tid] = 0.f;
+        inc[c * ADJ_THREADS + tid] = __ldg((p.gpre_prev ? p.gpre_prev : p.gA_next) + (size_t)c * N + ic);
+    }
+    if (p.gpre_prev)
+#pragma unroll 5
+        for (int k = 0; k < K; k++) inc[p.kt.src[k] * ADJ_THREADS + tid] += __ldg(&p.V[(size_t)k * N + ic]);
+#pragma unroll 5
+    for (int k = 0; k < K; k++) {
+        const float u = __ldg(&p.U[(size_t)k * N + ic]);
+        const float z = (u - p.kt.mu[k]) * rcp_approx(p.kt.sigma[k]);
+        const float g = ex2_approx(-ADJ_HALF_LOG2E * (z * z));
+        const float h = p.kt.h[k];
+        bump[k * ADJ_THREADS + tid] = g;
+        chan[p.kt.dst[k] * ADJ_THREADS + tid] += p.growth_form == 0 ? fmaf(2.f * g, h, -h) : h * g;
+    }
+    for (int c = 0; c < C; c++) {
+        const float a = __ldg(&p.A[(size_t)c * N + ic]) + p.dt * chan[c * ADJ_THREADS + tid];
+        const float gpre = valid && a > 0.f && a < 1.f ? inc[c * ADJ_THREADS + tid] : 0.f;
+        chan[c * ADJ_THREADS + tid] = gpre;
+        if (valid) p.gpre[(size_t)c * N + i] = gpre;
     }
     // kernel by kernel: potential gradient and this block's gene partials
-    for (int k = 0; k < K; k++) {
-        float dmu = 0.f, dsg = 0.f, dh = 0.f;
-        if (valid) {
-            const float u = __ldg(&p.U[(size_t)k * N + i]);
-            const float mu = p.kt.mu[k], sg = p.kt.sigma[k], h = p.kt.h[k];
-            const float d = u - mu;
-            const float z = d * rcp_approx(sg);
-            const float g = ex2_approx(-ADJ_HALF_LOG2E * (z * z));
-            const float fp = p.growth_form == 0 ? 2.f : 1.f;          // F'(g)
-            const float gG = gpre[p.kt.dst[k]] * p.dt * h;             // dL/dF
-            const float w = gG * fp * g;                               // dL/d(exp term)
-            const float inv_s2 = 1.f / (sg * sg);
-            p.gU[(size_t)k * N + i] = -w * d * inv_s2;
-            dmu = w * d * inv_s2;
-            dsg = w * d * d * inv_s2 / sg;
-            dh = gpre[p.kt.dst[k]] * p.dt * (p.growth_form == 0 ? 2.f * g - 1.f : g);
+    const float fp = p.growth_form == 0 ? 2.f : 1.f;        // F'(g)
+    for (int k0 = 0; k0 < K; k0 += ADJ_KB) {
+        const int kn = min(ADJ_KB, K - k0);
+#pragma unroll 3
+        for (int j = 0; j < kn; j++) {
+            const int k = k0 + j;
+            const float d = __ldg(&p.U[(size_t)k * N + ic]) - p.kt.mu[k];
+            const float sg = p.kt.sigma[k], h = p.kt.h[k];
+            const float g = bump[k * ADJ_THREADS + tid];
+            const float gp = chan[p.kt.dst[k] * ADJ_THREADS + tid] * p.dt;
+            const float w = gp * h * fp * g;                // dL/d(exp term)
+            const float wd = w * d * p.inv_s2[k];
+            if (valid) p.gU[(size_t)k * N + i] = -wd;
+            red[(3 * j) * ADJ_THREADS + tid] = wd;
+            red[(3 * j + 1) * ADJ_THREADS + tid] = wd * d * rcp_approx(sg);
+            red[(3 * j + 2) * ADJ_THREADS + tid] = gp * (p.growth_form == 0 ? 2.f * g - 1.f : g);
         }
-        float v[3] = {dmu, dsg, dh};
-#pragma unroll
-        for (int j = 0; j < 3; j++) {
-            float t = v[j];
+        __syncthreads();
+        // value-major partials [K * 3][blocks]: the reduction kernel reads them coalesced
+        for (int v = warp; v < 3 * kn; v += ADJ_THREADS / 32) {
+            const float* r = red + v * ADJ_THREADS + lane;
+            float t = (r[0] + r[32]) + (r[64] + r[96]);
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
-            if (lane == 0) red[warp][k * 3 + j] = t;
+            if (lane == 0) {
+                float2* o = p.gene_partials + (size_t)(3 * k0 + v) * gridDim.x + blockIdx.x;
+                *o = ff_add(p.first ? make_float2(0.f, 0.f) : *o, make_float2(t, 0.f));
+            }
         }
-    }
-    __syncthreads();
-    // value-major partials [K * 3][blocks]: the reduction kernel reads them coalesced
-    for (int v = threadIdx.x; v < K * 3; v += ADJ_THREADS) {
-        float2 s = make_float2(0.f, 0.f);
-        for (int w = 0; w < ADJ_THREADS / 32; w++) s = ff_add(s, make_float2(red[w][v], 0.f));
-        p.gene_partials[(size_t)v * gridDim.x + blockIdx.x] = s;
+        __syncthreads();
     }
 }
 
-// gene_acc[v] += sum over the nb block partials of value v (block v): thread t
+// gene_acc[v] = sum over the nb block partials of value v (block v): thread t
 // sums blocks t, t + 256, ... in order, then a fixed shuffle / shared tree,
 // so every launch adds in the same order.
 constexpr int ADJ_RED_THREADS = 256;
@@ -114,7 +128,7 @@ __global__ void __launch_bounds__(ADJ_RED_THREADS) k_adjoint_gene_reduce(const f
     if (threadIdx.x == 0) {
         float2 t = make_float2(0.f, 0.f);
         for (int w = 0; w < ADJ_RED_THREADS / 32; w++) t = ff_add(t, wsum[w]);
-        gene_acc[v] = ff_add(gene_acc[v], t);
+        gene_acc[v] = t;
     }
 }
 
@@ -147,13 +161,20 @@ __global__ void k_adjoint_gene_out(const float2* gene_acc, int nv, float* out)
 
 int adjoint_blocks(int H, int W) { return (int)(((size_t)H * W + ADJ_THREADS - 1) / ADJ_THREADS); }
 
-cudaError_t launch_adjoint_epilogue(const AdjParams& p, cudaStream_t s)
+cudaError_t launch_adjoint_epilogue(const AdjParams& p0, cudaStream_t s)
 {
-    const int nb = adjoint_blocks(p.H, p.W);
-    launch_pdl(k_adjoint_epilogue, nb, ADJ_THREADS, 0, s, p);
-    cudaError_t e = cudaGetLastError();
+    AdjParams p = p0;
+    for (int k = 0; k < p.kt.K; k++) p.inv_s2[k] = (float)(1.0 / ((double)p.kt.sigma[k] * p.kt.sigma[k]));
+    const size_t smem = (size_t)(p.kt.K + 2 * p.kt.C + 3 * ADJ_KB) * ADJ_THREADS * sizeof(float);
+    cudaError_t e = smem_limit<k_adjoint_epilogue>(smem);
     if (e != cudaSuccess) return e;
-    launch_pdl(k_adjoint_gene_reduce, p.kt.K * 3, ADJ_RED_THREADS, 0, s, p.gene_partials, nb, p.gene_acc);
+    launch_pdl(k_adjoint_epilogue, adjoint_blocks(p.H, p.W), ADJ_THREADS, smem, s, p);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_adjoint_gene_reduce(const float2* partials, int H, int W, int nv, float2* gene_acc, cudaStream_t s)
+{
+    launch_pdl(k_adjoint_gene_reduce, nv, ADJ_RED_THREADS, 0, s, partials, adjoint_blocks(H, W), gene_acc);
     return cudaGetLastError();
 }
 

@@ -85,6 +85,9 @@ struct lenia_ctx {
     KernelTable kt;
     std::string err;
     // adjoint (lenia_backward): checkpoints, segment states, gradients
+    // transposed convolution: the path's own passes, windows summed per channel in the
+    // frequency domain, or windows plane by plane (gathered by the next step)
+    enum AdjForm { ADJ_PASSES, ADJ_WINDOWS, ADJ_PLANES } adj_form = ADJ_PASSES;
     bool adj = false;
     int ckpt = 0, max_steps = 0;
     float* d_ckpt = nullptr;               // [n_ckpt][C][H][W]
@@ -92,6 +95,7 @@ struct lenia_ctx {
     float* d_Useg = nullptr;               // [ckpt][K][H][W] potentials of the segment's states
     float* d_gA[2] = {nullptr, nullptr};
     float* d_gpre = nullptr;
+    float* d_gpre2 = nullptr;              // plane by plane: the previous reversed step's
     float* d_gU = nullptr;
     float* d_V = nullptr;
     float2* d_gene_part = nullptr;    // compensated FP32 (hi, lo) pairs
@@ -125,7 +129,12 @@ struct lenia_ctx {
     };
     cudaStream_t cap_stream = nullptr;
     GraphSlot g_rollout, g_backward;
-    uint64_t genes_version = 0;            // bumped by lenia_set_genes
+    uint64_t genes_version = 0;            // bumped by lenia_set_genes when the genes change
+    // Genes that change from call to call (training) would have every call pay a
+    // capture and an instantiation (about 0.3 ms for a 12-step backward) to
+    // replay it once: after a change, arguments seen for the first time are
+    // launched directly and captured when they come again.
+    std::array<uintptr_t, 7> seen_rollout{}, seen_backward{};
     std::vector<cudaEvent_t> ev;
     std::vector<int> ev_kind;
     size_t ev_used = 0;
@@ -616,9 +625,18 @@ lenia_status transposed_conv(lenia_ctx* c, const float* gU, float* V, cudaStream
                              const float* add = nullptr, float* out = nullptr)
 {
     const int K = c->cfg.n_kernels;
-    if (c->tile && c->path != LENIA_CONV_FFT) {
+    if (c->adj_form != lenia_ctx::ADJ_PASSES) {
         TileParams tl = c->tl;
         tl.A = gU;
+        if (c->adj_form == lenia_ctx::ADJ_PLANES) {
+            tl.U = V;
+            tl.C = K;
+            tl.per_plane = 1;
+            tl.kpb = 1;
+            CUDA_OR_FAIL(c, launch_tile_conv(tl, s));
+            *per_channel = false;
+            return LENIA_OK;
+        }
         tl.U = out ? out : V;
         tl.add = out ? add : nullptr;
         CUDA_OR_FAIL(c, launch_tile_conv_adj(tl, s));
@@ -737,7 +755,7 @@ void lenia_destroy(lenia_ctx* c)
     void* ptrs[] = {c->d_w, c->d_w_off, c->d_yr, c->d_yr_off, c->d_S, c->d_twM, c->d_twW, c->d_twH,
                     c->d_Ahat, c->d_Uhat, c->d_U, c->d_partials, c->d_trig, c->d_A2, c->d_P2,
                     c->d_A3, c->d_P3, c->d_stats, c->d_status, c->d_ckpt, c->d_seg, c->d_gA[0],
-                    c->d_gA[1], c->d_gpre, c->d_gU, c->d_V, c->d_gene_part, c->d_gene_acc,
+                    c->d_gA[1], c->d_gpre, c->d_gpre2, c->d_gU, c->d_V, c->d_gene_part, c->d_gene_acc,
                     c->d_Ahat_t, c->d_Uhat_t, c->d_ticket, c->d_walls, c->d_alpha_e, c->d_empty,
                     c->d_Useg, c->d_hA_in1, c->d_hP_in1, c->d_hA_out1,
                     c->d_hP_out1, c->d_hstats, c->d_tc_hi, c->d_tc_lo, c->d_tc_B, c->d_tc_ks,
@@ -936,6 +954,13 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
             c->tile = true;
         }
     }
+    if (want_adj && c->tile) {
+        const double t_win = tile_adj_cost(c->tl, kcount), t_pl = tile_planes_cost(c->tl, K);
+        const double t_own = path == LENIA_CONV_FFT ? fft_passes_cost(H, W, C + NC) : 1e30;
+        // (the gather of K planes costs about what their share of the traffic does)
+        c->adj_form = std::min(t_win, t_pl) >= t_own ? lenia_ctx::ADJ_PASSES
+                      : t_win <= t_pl ? lenia_ctx::ADJ_WINDOWS : lenia_ctx::ADJ_PLANES;
+    }
     // stats records: the largest of the tiled epilogue's blocks, and the resident CTAs
     c->n_part_blocks = std::max(std::max(epilogue_blocks(H, W), ring_epilogue_blocks(H, W)), kSitesBlocksPerSm * c->num_sms);
 
@@ -1130,7 +1155,7 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
         c->tp.n_dy = n_dy;
         c->tp.n_groups = (int)grp.size() / (2 + TC_NG);
         c->tp.terms = path == LENIA_CONV_DIRECT_BF16X3 ? 3 : 1;
-    } else if (path == LENIA_CONV_FFT && (!c->tile || want_adj)) {
+    } else if (path == LENIA_CONV_FFT && (!c->tile || (want_adj && c->adj_form == lenia_ctx::ADJ_PASSES))) {
         const int M = W / 2, HS = H / 2 + 1;
         ALLOC(c->d_Ahat, (size_t)C * H * M);
         ALLOC(c->d_Uhat, (size_t)NC * H * M);
@@ -1175,11 +1200,12 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
         ALLOC(c->d_gA[0], nA1);
         ALLOC(c->d_gA[1], nA1);
         ALLOC(c->d_gpre, nA1);
+        if (c->adj_form == lenia_ctx::ADJ_PLANES) ALLOC(c->d_gpre2, nA1);
         ALLOC(c->d_gU, c->N * K);
         ALLOC(c->d_V, c->N * K);
         ALLOC(c->d_gene_part, (size_t)adjoint_blocks(H, W) * K * 3);
         ALLOC(c->d_gene_acc, (size_t)K * 3);
-        if (path == LENIA_CONV_FFT) {
+        if (path == LENIA_CONV_FFT && c->adj_form == lenia_ctx::ADJ_PASSES) {
             ALLOC(c->d_Ahat_t, (size_t)K * (W / 2) * H);     // spectra of the K gradient planes
             ALLOC(c->d_Uhat_t, (size_t)C * (W / 2) * H);     // their per-channel sums
         }
@@ -1236,6 +1262,15 @@ static lenia_status run_graph(lenia_ctx* c, lenia_ctx::GraphSlot& slot, const st
     return LENIA_OK;
 }
 }  // extern "C++"
+
+// True once for a key that came with changed genes (see seen_rollout).
+static bool first_sight(const lenia_ctx* c, const lenia_ctx::GraphSlot& slot, const std::array<uintptr_t, 7>& key,
+                        std::array<uintptr_t, 7>& seen)
+{
+    if (c->genes_version == 0 || (slot.exec && slot.key == key) || seen == key) return false;
+    seen = key;
+    return true;
+}
 
 static lenia_status rollout_body(lenia_ctx* c, float* A, float* P, int32_t n_steps, float* stats_out, cudaStream_t s)
 {
@@ -1335,6 +1370,7 @@ lenia_status lenia_rollout(lenia_ctx* c, float* A, float* P, int32_t n_steps, fl
     // otherwise pairs of steps replay one cached two-step graph (the state is
     // back in A, P after each pair); an odd last step runs directly
     const std::array<uintptr_t, 7> key{(uintptr_t)A, (uintptr_t)P, (uintptr_t)c->genes_version, 2, 0, 0, 0};
+    if (n_steps < 32 && first_sight(c, c->g_rollout, key, c->seen_rollout)) return rollout_body(c, A, P, n_steps, nullptr, s);
     for (int i = 0; i < n_steps / 2; i++) {
         const lenia_status st =
             run_graph(c, c->g_rollout, key, s, [&](cudaStream_t t) { return rollout_body(c, A, P, 2, nullptr, t); });
@@ -1356,6 +1392,42 @@ static lenia_status backward_body(lenia_ctx* c, int32_t n_steps, cudaStream_t s)
     auto ckpt = [&](int j) { return c->d_ckpt + (size_t)j * nA; };
     auto seg = [&](int j) { return c->d_seg + (size_t)j * nA; };
 
+    int cur = 0;
+    bool first = true;
+    // one reversed step, from the state At and its potentials Ut
+    auto reverse = [&](const float* At, const float* Ut) -> lenia_status {
+        const bool planes = c->adj_form == lenia_ctx::ADJ_PLANES;
+        AdjParams ap;
+        memset(&ap, 0, sizeof(ap));
+        ap.A = At;
+        ap.U = Ut;
+        ap.gA_next = c->d_gA[cur];
+        ap.gpre = planes && cur ? c->d_gpre2 : c->d_gpre;
+        ap.gpre_prev = planes && !first ? (cur ? c->d_gpre : c->d_gpre2) : nullptr;
+        ap.gU = c->d_gU;
+        ap.V = c->d_V;
+        ap.gA_out = c->d_gA[cur ^ 1];
+        ap.gene_partials = c->d_gene_part;
+        ap.first = first;
+        ap.H = c->cfg.height;
+        ap.W = c->cfg.width;
+        ap.growth_form = c->cfg.growth_form;
+        ap.dt = c->cfg.dt;
+        ap.kt = c->kt;
+        CUDA_OR_FAIL(c, launch_adjoint_epilogue(ap, s));
+        bool per_channel = false;
+        const lenia_status st = transposed_conv(c, c->d_gU, c->d_V, s, &per_channel, ap.gpre, c->d_gA[cur ^ 1]);
+        if (st != LENIA_OK) return st;
+        // plane by plane, the next reversed step gathers; the last one's sum is made here
+        if (!per_channel && (!planes || At == c->d_ckpt)) CUDA_OR_FAIL(c, launch_adjoint_gather(ap, s));
+        cur ^= 1;
+        first = false;
+        return LENIA_OK;
+    };
+    auto finish = [&]() -> lenia_status {
+        CUDA_OR_FAIL(c, launch_adjoint_gene_reduce(c->d_gene_part, c->cfg.height, c->cfg.width, K * 3, c->d_gene_acc, s));
+        return LENIA_OK;
+    };
     // forward pass, keeping the states at multiples of the checkpoint interval
     const float* prev = ckpt(0);
     if (L == 1) {
@@ -1367,35 +1439,15 @@ static lenia_status backward_body(lenia_ctx* c, int32_t n_steps, cudaStream_t s)
                 st = step_impl(c, ckpt(t), nullptr, ckpt(t + 1), nullptr, nullptr, nullptr, uall(t), s);
             if (st != LENIA_OK) return st;
         }
-        CUDA_OR_FAIL(c, cudaMemsetAsync(c->d_gene_acc, 0, (size_t)K * 3 * sizeof(float2), s));
-        int cur = 0;
         for (int t = n_steps - 1; t >= 0; t--) {
-            AdjParams ap;
-            memset(&ap, 0, sizeof(ap));
-            ap.A = ckpt(t);
-            ap.U = uall(t);
-            ap.gA_next = c->d_gA[cur];
-            ap.gpre = c->d_gpre;
-            ap.gU = c->d_gU;
-            ap.V = c->d_V;
-            ap.gA_out = c->d_gA[cur ^ 1];
-            ap.gene_partials = c->d_gene_part;
-            ap.gene_acc = c->d_gene_acc;
-            ap.H = c->cfg.height;
-            ap.W = c->cfg.width;
-            ap.growth_form = c->cfg.growth_form;
-            ap.dt = c->cfg.dt;
-            ap.kt = c->kt;
-            CUDA_OR_FAIL(c, launch_adjoint_epilogue(ap, s));
-            bool per_channel = false;
-            lenia_status st = transposed_conv(c, c->d_gU, c->d_V, s, &per_channel, c->d_gpre, c->d_gA[cur ^ 1]);
+            const lenia_status st = reverse(ckpt(t), uall(t));
             if (st != LENIA_OK) return st;
-            if (!per_channel) CUDA_OR_FAIL(c, launch_adjoint_gather(ap, s));
-            cur ^= 1;
         }
-        return LENIA_OK;
+        return finish();
     }
-    for (int t = 0; t + 1 < n_steps; t++) {
+    // (up to the last checkpoint: the last segment's states are recomputed below)
+    const int n_seg = (n_steps + L - 1) / L;
+    for (int t = 0; t < (n_seg - 1) * L; t++) {
         float* dst = ((t + 1) % L == 0) ? ckpt((t + 1) / L) : seg((t + 1) & 1);
         lenia_status st = step_impl(c, prev, nullptr, dst, nullptr, nullptr, nullptr, nullptr, s);
         if (st != LENIA_OK) return st;
@@ -1404,10 +1456,7 @@ static lenia_status backward_body(lenia_ctx* c, int32_t n_steps, cudaStream_t s)
     // backward, segment by segment from the last: recompute the segment's
     // states and their potentials from its checkpoint, then apply the step
     // adjoint in reverse
-    CUDA_OR_FAIL(c, cudaMemsetAsync(c->d_gene_acc, 0, (size_t)K * 3 * sizeof(float2), s));
     auto useg = [&](int j) { return c->d_Useg + (size_t)j * K * c->N; };
-    int cur = 0;
-    const int n_seg = (n_steps + L - 1) / L;
     for (int sg = n_seg - 1; sg >= 0; sg--) {
         const int s0 = sg * L, s1 = std::min(n_steps, s0 + L);
         for (int j = 0; j < s1 - s0; j++) {
@@ -1418,32 +1467,11 @@ static lenia_status backward_body(lenia_ctx* c, int32_t n_steps, cudaStream_t s)
             if (st != LENIA_OK) return st;
         }
         for (int t = s1 - 1; t >= s0; t--) {
-            const float* At = t == s0 ? ckpt(sg) : seg(t - s0);
-            AdjParams ap;
-            memset(&ap, 0, sizeof(ap));
-            ap.A = At;
-            ap.U = useg(t - s0);
-            ap.gA_next = c->d_gA[cur];
-            ap.gpre = c->d_gpre;
-            ap.gU = c->d_gU;
-            ap.V = c->d_V;
-            ap.gA_out = c->d_gA[cur ^ 1];
-            ap.gene_partials = c->d_gene_part;
-            ap.gene_acc = c->d_gene_acc;
-            ap.H = c->cfg.height;
-            ap.W = c->cfg.width;
-            ap.growth_form = c->cfg.growth_form;
-            ap.dt = c->cfg.dt;
-            ap.kt = c->kt;
-            CUDA_OR_FAIL(c, launch_adjoint_epilogue(ap, s));
-            bool per_channel = false;
-            lenia_status st = transposed_conv(c, c->d_gU, c->d_V, s, &per_channel, c->d_gpre, c->d_gA[cur ^ 1]);
+            const lenia_status st = reverse(t == s0 ? ckpt(sg) : seg(t - s0), useg(t - s0));
             if (st != LENIA_OK) return st;
-            if (!per_channel) CUDA_OR_FAIL(c, launch_adjoint_gather(ap, s));
-            cur ^= 1;
         }
     }
-    return LENIA_OK;
+    return finish();
 }
 
 lenia_status lenia_backward(lenia_ctx* c, const float* A0, const float* P0, int32_t n_steps, const float* gA_T,
@@ -1465,7 +1493,9 @@ lenia_status lenia_backward(lenia_ctx* c, const float* A0, const float* P0, int3
     CUDA_OR_FAIL(c, cudaMemcpyAsync(c->d_gA[0], gA_T, nA * sizeof(float), cudaMemcpyDeviceToDevice, s));
     const std::array<uintptr_t, 7> key{(uintptr_t)n_steps, (uintptr_t)c->genes_version, 1, 0, 0, 0, 0};
     const lenia_status st =
-        run_graph(c, c->g_backward, key, s, [&](cudaStream_t t) { return backward_body(c, n_steps, t); });
+        first_sight(c, c->g_backward, key, c->seen_backward)
+            ? backward_body(c, n_steps, s)
+            : run_graph(c, c->g_backward, key, s, [&](cudaStream_t t) { return backward_body(c, n_steps, t); });
     if (st != LENIA_OK) return st;
     const int cur = n_steps & 1;
     if (gA0) CUDA_OR_FAIL(c, cudaMemcpyAsync(gA0, c->d_gA[cur], nA * sizeof(float), cudaMemcpyDeviceToDevice, s));
@@ -1482,6 +1512,12 @@ lenia_status lenia_set_genes(lenia_ctx* c, const float* genes)
         if (!isfinite(mu) || !isfinite(sg) || !isfinite(h)) return fail(c, LENIA_EINVAL, "genes must be finite");
         if (!(c->cfg.localized & LENIA_LOC_SIGMA) && !(sg > 0.f)) return fail(c, LENIA_EINVAL, "sigma must be > 0");
     }
+    bool same = true;
+    for (int k = 0; k < K; k++) {
+        const float now[3] = {c->kt.mu[k], c->kt.sigma[k], c->kt.h[k]};
+        same = same && memcmp(now, genes + 3 * k, sizeof(now)) == 0;
+    }
+    if (same) return LENIA_OK;             // the graphs' parameters hold
     for (int k = 0; k < K; k++) {
         c->kd[k].mu = c->kt.mu[k] = genes[3 * k];
         c->kd[k].sigma = c->kt.sigma[k] = genes[3 * k + 1];

@@ -301,6 +301,7 @@ struct TileParams {
     float gate_eps;
     int gate_r;
     int kpb;                   // kernels per block
+    int per_plane;             // K planes of A, plane k convolved with kernel k (C = K)
     int vec2, vec2o;           // input / output 8-byte aligned (set by the launcher)
     int kcount[kMaxChannels];
     int klist[kMaxChannels][kMaxKernels];
@@ -311,6 +312,10 @@ bool tile_plan(TileParams* p, int N, int H, int W, int R);
 // infinity where no window serves R), and the models of the other routes.
 // (n_worlds: worlds of that shape in one launch)
 double tile_choose(TileParams* p, int H, int W, const int* kcount, int R, int n_worlds = 1);
+// time models of the transposed convolution: summed per channel in the frequency
+// domain, or plane by plane
+double tile_adj_cost(const TileParams& p, const int* kcount);
+double tile_planes_cost(const TileParams& p, int K);
 double fft_passes_cost(int H, int W, int planes);      // planes: channels + convolution outputs
 double direct_cost(int H, int W, int planes, int R);   // planes: convolution outputs
 size_t tile_spectrum_floats(int N);
@@ -344,8 +349,10 @@ struct AdjParams {
     const float* V;            // K~_k (x) gU_k [K][H][W], or summed per source channel [C][H][W]
     int v_per_channel;         // 1: V holds sum_{src(k) = c} K~_k (x) gU_k per channel c
     float* gA_out;             // dL/dA_t [C][H][W]
+    const float* gpre_prev;    // set: dL/dA_{t+1} is gathered from it and V [K][H][W], gA_next unused
+    int first;                 // the pass's first reversed step: the gene partials start from zero
+    float inv_s2[kMaxKernels]; // 1 / sigma^2 (set by the launcher)
     float2* gene_partials;     // [K][3][blocks], compensated (hi, lo) sums
-    float2* gene_acc;          // [K][3]: d/dmu, d/dsigma, d/dh, compensated (hi, lo) sums
     int H, W, growth_form;
     float dt;
     KernelTable kt;
@@ -370,6 +377,7 @@ cudaError_t launch_selftest_wait(long long limit_cycles, int* status, cudaStream
 int adjoint_blocks(int H, int W);
 cudaError_t launch_adjoint_epilogue(const AdjParams& p, cudaStream_t s);
 cudaError_t measure_fp32_peak(cudaStream_t s, double* scalar_tflops, double* pair_tflops);
+cudaError_t launch_adjoint_gene_reduce(const float2* partials, int H, int W, int nv, float2* gene_acc, cudaStream_t s);
 cudaError_t launch_adjoint_gather(const AdjParams& p, cudaStream_t s);
 cudaError_t launch_adjoint_gene_out(const float2* gene_acc, int nv, float* out, cudaStream_t s);
 bool epilogue_rows_supported(const EpiParams& p);

@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(2 * N, N == 128 ? 3 : (ADJ ? 6 : 8)) k_tile_co
     float* gU = tw ? tw->U : p.U;
     const float* gS = tw ? tw->S : p.S;
     const float* gS0 = tw ? tw->S0 : p.S0;
-    const int nk = p.kcount[w.c];
+    const int nk = !ADJ && p.per_plane ? 1 : p.kcount[w.c];
     const int t0 = ADJ ? 0 : (int)blockIdx.z * p.kpb;
     if (t0 >= nk) return;                                                    // uniform over the block
     const int t1 = ADJ ? nk : min(nk, t0 + p.kpb);
@@ -561,7 +561,7 @@ __global__ void __launch_bounds__(2 * N, N == 128 ? 3 : (ADJ ? 6 : 8)) k_tile_co
         tmem_wait_st();
         __syncthreads();
         for (int t = t0; t < t1; t++) {
-            const int k = p.klist[w.c][t];
+            const int k = p.per_plane ? w.c : p.klist[w.c][t];
             float* U = gU + (size_t)k * HW;
             inverse<N, UNR>(
                 w, rows, buf, twc,
@@ -797,8 +797,8 @@ cudaError_t launch_n(const TileParams& p, cudaStream_t s)
 {
     cudaError_t e = smem_limit<k_tile_conv<N, ADJ>>(TC<N>::SMEM);
     if (e != cudaSuccess) return e;
-    int kmax = 0;
-    for (int c = 0; c < p.C && c < kMaxChannels; c++) kmax = p.kcount[c] > kmax ? p.kcount[c] : kmax;
+    int kmax = p.per_plane ? 1 : 0;
+    for (int c = 0; c < p.C && c < kMaxChannels && !p.per_plane; c++) kmax = p.kcount[c] > kmax ? p.kcount[c] : kmax;
     if (kmax == 0) return cudaSuccess;
     const dim3 grid(p.worlds ? p.tiles : p.g.tiles_x * p.g.tiles_y, p.worlds ? p.C * p.n_worlds : p.C, ADJ ? 1 : (kmax + p.kpb - 1) / p.kpb);
     launch_pdl(k_tile_conv<N, ADJ>, grid, TC<N>::T, TC<N>::SMEM, s, p);
@@ -840,18 +840,38 @@ bool tile_plan(TileParams* p, int N, int H, int W, int R)
 // Time model of one launch (us), fitted to measurements at 64^2 .. 2048^2: a
 // block's work is two units for the forward transform and one per kernel; a
 // unit takes t1 on an idle SM and tf with every block slot of the SM taken.
-static double tile_cost(const TileParams& p, const int* kcount, int kpb, int n_worlds)
+static double tile_time(const TileParams& p, double blocks, double units)
 {
     const double slots = 152.0 * (p.N == 128 ? 3 : 8);
     const double t1 = p.N == 128 ? 2.3 : 0.9, tf = p.N == 128 ? 7.7 : 3.9;
+    const double waves = blocks / slots, whole = floor(waves), rest = waves - whole;
+    return 3.0 + units * (whole * tf + (rest > 0 ? t1 + (tf - t1) * rest : 0));
+}
+
+static double tile_cost(const TileParams& p, const int* kcount, int kpb, int n_worlds)
+{
     double blocks = 0;
     int kmax = 0;
     for (int c = 0; c < kMaxChannels; c++) {
         blocks += (double)n_worlds * p.g.tiles_x * p.g.tiles_y * ((kcount[c] + kpb - 1) / kpb);
         kmax = kcount[c] > kmax ? kcount[c] : kmax;
     }
-    const double waves = blocks / slots, whole = floor(waves), rest = waves - whole;
-    return 3.0 + (2 + (kpb < kmax ? kpb : kmax)) * (whole * tf + (rest > 0 ? t1 + (tf - t1) * rest : 0));
+    return tile_time(p, blocks, 2 + (kpb < kmax ? kpb : kmax));
+}
+
+double tile_adj_cost(const TileParams& p, const int* kcount)
+{
+    int kmax = 0, chans = 0;
+    for (int c = 0; c < kMaxChannels; c++) {
+        kmax = kcount[c] > kmax ? kcount[c] : kmax;
+        chans += kcount[c] > 0;
+    }
+    return tile_time(p, (double)p.g.tiles_x * p.g.tiles_y * chans, 1 + 2 * kmax);
+}
+
+double tile_planes_cost(const TileParams& p, int K)
+{
+    return tile_time(p, (double)p.g.tiles_x * p.g.tiles_y * K, 3);
 }
 
 double tile_choose(TileParams* p, int H, int W, const int* kcount, int R, int n_worlds)
