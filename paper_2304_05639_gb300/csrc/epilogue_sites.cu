@@ -109,63 +109,54 @@ struct Stencil {
     }
 };
 
-// Kernel k's direct sum at (y, x), in k_direct_conv's order (tap columns, then rows).
+// Tap t of the list: its value's place in the plane, and its weight.
+__device__ __forceinline__ int tap_site(int2 tap, int y, int x, int H, int W)
+{
+    int yy = y + (tap.x >> 11) - 1024, xx = x + (tap.x & 2047) - 1024;
+    yy = yy < 0 ? yy + H : (yy >= H ? yy - H : yy);
+    xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
+    return yy * W + xx;
+}
+
+// Kernel k's direct sum at (y, x): its non-zero taps in k_direct_conv's order (a zero
+// weight adds nothing there), so the same bits.
 __device__ __forceinline__ float direct_at(const SitesParams& q, const float* A, int k, int y, int x)
 {
-    const int H = q.e.H, W = q.e.W, R = q.g.R[k];
+    const int H = q.e.H, W = q.e.W;
     const float* plane = A + (size_t)q.e.kt.src[k] * H * W;
-    const float* w = q.g.w + q.g.w_off[k];
-    const int* yr = q.g.yr + q.g.yr_off[k];
     float acc = 0.f;
-    for (int dx = -R; dx <= R; dx++) {
-        const int r = __ldg(&yr[dx + R]);
-        int xx = x + dx;
-        xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
-        const float* wc = w + (dx + R) * (2 * R + 1) + R;
-        for (int dy = -r; dy <= r; dy++) {
-            int yy = y + dy;
-            yy = yy < 0 ? yy + H : (yy >= H ? yy - H : yy);
-            acc = fmaf(__ldg(&wc[dy]), __ldg(&plane[(size_t)yy * W + xx]), acc);
-        }
+    for (int t = q.g.off[k]; t < q.g.off[k + 1]; t++) {
+        const int2 tap = __ldg(&q.g.taps[t]);
+        acc = fmaf(__int_as_float(tap.y), __ldg(&plane[tap_site(tap, y, x, H, W)]), acc);
     }
     return acc;
 }
 
-// The same sum by a whole warp: the lanes load a tap column's values side by side
-// (two columns in flight) and every lane adds them in order.
+// The same sum by a whole warp: the lanes load 8 x 32 taps at once and every lane
+// adds them in order.
 __device__ __forceinline__ float direct_warp(const SitesParams& q, const float* A, int k, int y, int x)
 {
-    const int H = q.e.H, W = q.e.W, R = q.g.R[k], lane = threadIdx.x & 31;
+    constexpr int B = 8;
+    const int H = q.e.H, W = q.e.W, lane = threadIdx.x & 31;
     const float* plane = A + (size_t)q.e.kt.src[k] * H * W;
-    const float* w = q.g.w + q.g.w_off[k];
-    const int* yr = q.g.yr + q.g.yr_off[k];
+    const int t1 = q.g.off[k + 1];
     float acc = 0.f;
-    auto fetch = [&](int dx, int dy0, int r, float& v, float& wv) {
-        const int dy = dy0 + lane;
-        v = wv = 0.f;
-        if (dx > R || dy > r) return;
-        int xx = x + dx, yy = y + dy;
-        xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
-        yy = yy < 0 ? yy + H : (yy >= H ? yy - H : yy);
-        v = __ldg(&plane[(size_t)yy * W + xx]);
-        wv = __ldg(&w[(dx + R) * (2 * R + 1) + R + dy]);
-    };
-    int r = __ldg(&yr[0]);
-    float v, wv;
-    fetch(-R, -r, r, v, wv);
-    for (int dx = -R; dx <= R; dx++) {
-        const int rn = dx < R ? __ldg(&yr[dx + 1 + R]) : -1;
-        float vn, wn;
-        fetch(dx + 1, -rn, rn, vn, wn);
-        for (int dy0 = -r; dy0 <= r; dy0 += 32) {
-            if (dy0 > -r) fetch(dx, dy0, r, v, wv);
-            const int n = min(32, r - dy0 + 1);
-            for (int i = 0; i < n; i++)
-                acc = fmaf(__shfl_sync(0xffffffffu, wv, i), __shfl_sync(0xffffffffu, v, i), acc);
+    for (int t0 = q.g.off[k]; t0 < t1; t0 += 32 * B) {
+        float v[B], w[B];
+#pragma unroll
+        for (int j = 0; j < B; j++) {
+            const int t = t0 + 32 * j + lane;
+            const int2 tap = t < t1 ? __ldg(&q.g.taps[t]) : make_int2((1024 << 11) + 1024, 0);
+            w[j] = __int_as_float(tap.y);
+            v[j] = __ldg(&plane[tap_site(tap, y, x, H, W)]);
         }
-        v = vn;
-        wv = wn;
-        r = rn;
+#pragma unroll
+        for (int j = 0; j < B; j++) {
+            const int n = min(32, t1 - (t0 + 32 * j));
+#pragma unroll 8
+            for (int i = 0; i < n; i++)
+                acc = fmaf(__shfl_sync(0xffffffffu, w[j], i), __shfl_sync(0xffffffffu, v[j], i), acc);
+        }
     }
     return acc;
 }
@@ -252,57 +243,104 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
         float* pAo = p.Aout_list ? p.Aout_list[wz] : p.A_out;
         float* pPo = p.Pout_list ? p.Pout_list[wz] : p.P_out;
         const float* pU = p.U + (size_t)wz * p.u_stride;
-        // lanes beyond the world's edge stand on its last quad and store nothing, so
-        // that the warp stays together
-        const int xq = (bx * ES_Q + (lane & (ES_Q - 1))) * 4, yq = by * ES_Y + warp * (32 / ES_Q) + lane / ES_Q;
+        // a warp takes 8 quads of 4 rows and stays together: lanes beyond the world's
+        // edge stand on the torus's continuation and store nothing
+        const int qx = lane & (ES_Q - 1), ry = lane / ES_Q;
+        const int xq = (bx * ES_Q + qx) * 4, yq = by * ES_Y + warp * (32 / ES_Q) + ry;
         const bool in = xq < W && yq < H;
-        const int x = xq < W ? xq : W - 4, y = yq < H ? yq : H - 1;
+        const int x = in || xq < W ? xq : xq % W, y = yq < H ? yq : yq % H;
         {
             const int i0 = y * W + x;
-            // row offsets from row y, columns left and right of the quad
-            int ro[2 * RD + 1], xl[2], xr[2];
-#pragma unroll
-            for (int j = 0; j <= 2 * RD; j++) {
-                const int r = y + j - RD;
-                ro[j] = (j - RD + (r < 0 ? H : (r >= H ? -H : 0))) * W;
-            }
-#pragma unroll
-            for (int i = 0; i < 2; i++) {
-                xl[i] = -1 - i + (x - 1 - i < 0 ? W : 0);
-                xr[i] = 4 + i - (x + 4 + i >= W ? W : 0);
-            }
             auto quad = [&](const float* base) { return __ldg(reinterpret_cast<const float4*>(base)); };
-            // the quads of the next kernel's planes and potential are fetched one kernel
-            // ahead; the rows above and below are other threads' quads and mostly
-            // found in L1
-            float4 nc[NQ], nu;
-            Stencil<RD> s0;
+            // Radius 1: the quads around a quad are other lanes' own (shuffles), but for
+            // the warp's rim, whose lanes also load the row above or below and
+            // the column beside.  Radius 2 loads its neighbours itself (row
+            // offsets from row y, columns left and right).
+            const bool rim_y = ry == 0 || ry == 32 / ES_Q - 1, rim_x = qx == 0 || qx == ES_Q - 1;
+            int ro[2 * RD + 1], xl[2], xr[2], ie = i0, is = i0;
+            if constexpr (RD == 1) {
+                const int yn = ry == 0 ? (y == 0 ? H - 1 : y - 1) : (y == H - 1 ? 0 : y + 1);
+                ie = yn * W + x;
+                is = y * W + (qx == 0 ? (x == 0 ? W - 1 : x - 1) : (x + 4 == W ? 0 : x + 4));
+            }
+            if constexpr (RD == 2) {
+#pragma unroll
+                for (int j = 0; j <= 2 * RD; j++) {
+                    const int r = y + j - RD;
+                    ro[j] = (j - RD + (r < 0 ? H : (r >= H ? -H : 0))) * W;
+                }
+#pragma unroll
+                for (int i = 0; i < 2; i++) {
+                    xl[i] = -1 - i + (x - 1 - i < 0 ? W : 0);
+                    xr[i] = 4 + i - (x + 4 + i >= W ? W : 0);
+                }
+            }
+            // a kernel's planes and potential are fetched one kernel ahead
+            struct Pre {
+                float4 c, e;
+                float s;
+            } nx[NQ];
+            float4 nu = make_float4(0.f, 0.f, 0.f, 0.f);
+            auto fetch = [&](const float* plane, Pre& o) {
+                o.c = quad(plane + i0);
+                if constexpr (RD == 1) {
+                    if (rim_y) o.e = quad(plane + ie);
+                    if (rim_x) o.s = __ldg(plane + is);
+                }
+            };
+            auto gather = [&](const Pre& o, const float* plane, Stencil<RD>& s) {
+                if constexpr (RD == 1) {
+                    const float c[4] = {o.c.x, o.c.y, o.c.z, o.c.w}, e[4] = {o.e.x, o.e.y, o.e.z, o.e.w};
+#pragma unroll
+                    for (int i = 0; i < 4; i++) {
+                        const float u = __shfl_up_sync(0xffffffffu, c[i], ES_Q), d = __shfl_down_sync(0xffffffffu, c[i], ES_Q);
+                        s.v[0][1 + i] = ry == 0 ? e[i] : u;
+                        s.v[1][1 + i] = c[i];
+                        s.v[2][1 + i] = ry == 32 / ES_Q - 1 ? e[i] : d;
+                    }
+                    const float l = __shfl_up_sync(0xffffffffu, c[3], 1), r = __shfl_down_sync(0xffffffffu, c[0], 1);
+                    s.v[1][0] = qx == 0 ? o.s : l;
+                    s.v[1][5] = qx == ES_Q - 1 ? o.s : r;
+                } else {
+                    s.load(plane + i0, ro, xl, xr, o.c);
+                }
+            };
             bool live = in;
             if constexpr (NP > 0) {
-                nc[0] = quad(pP + i0);
-                s0.load(pP + i0, ro, xl, xr, nc[0]);
-                if (q.gate) live = in && s0.any_above(eps_p);
+                fetch(pP, nx[0]);
+                if (q.gate) {
+                    if constexpr (RD == 1) {
+                        float m = fmaxf(fmaxf(nx[0].c.x, nx[0].c.y), fmaxf(nx[0].c.z, nx[0].c.w));
+                        if (rim_y) m = fmaxf(m, fmaxf(fmaxf(nx[0].e.x, nx[0].e.y), fmaxf(nx[0].e.z, nx[0].e.w)));
+                        if (rim_x) m = fmaxf(m, nx[0].s);
+                        live = m > eps_p;                   // (of the warp, below)
+                    } else {
+                        Stencil<RD> s;
+                        gather(nx[0], pP, s);
+                        live = s.any_above(eps_p);
+                    }
+                }
             }
             float acc[CT][4];
 #pragma unroll
             for (int c = 0; c < CT; c++)
 #pragma unroll
                 for (int i = 0; i < 4; i++) acc[c][i] = 0.f;
-            bool al[4] = {live, live, live, live};
+            bool al[4] = {in, in, in, in};
             float tsum[4] = {0.f, 0.f, 0.f, 0.f}, tband[4] = {0.f, 0.f, 0.f, 0.f};
             bool wrote = false;                     // a non-zero gene went out already
             int k = 0;
-            if (__any_sync(0xffffffffu, live)) {
-                const float* up = pU + i0;
-                const float* gp = pP + i0;          // kernel k's first plane at the quad
-                float* go = pPo + i0;
+            const bool warp_live = __any_sync(0xffffffffu, live);
+            if (NP > 0 && !warp_live) al[0] = al[1] = al[2] = al[3] = false;
+            if (warp_live) {
                 const size_t KN = (size_t)K * N;
-                bool want = live;               // something left to compute for this quad
-                if (want) {
-                    nu = quad(up);
+                const float* up = pU + i0;
+                const float* gp = pP;               // kernel k's first plane
+                float* go = pPo + i0;
+                bool want = in;                     // something left to compute for this quad
+                nu = quad(up);
 #pragma unroll
-                    for (int pp = 1; pp < NP; pp++) nc[pp] = quad(gp + pp * KN);
-                }
+                for (int pp = 1; pp < NP; pp++) fetch(gp + pp * KN, nx[pp]);
 #pragma unroll 1
                 for (; k < K; k++) {
                     float ph[NQ][4], u[4], gk[4], tk[4];
@@ -311,25 +349,25 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                     auto sg_of = [&](int c) { return PSG >= 0 ? ph[PSG >= 0 ? PSG : 0][c] : ks; };
                     auto h_of = [&](int c) { return PH >= 0 ? ph[PH >= 0 ? PH : 0][c] : kh; };
                     uint32_t near = 0;              // sites whose test is to be settled
+                    Pre cur[NQ];
+#pragma unroll
+                    for (int pp = 0; pp < NP; pp++) cur[pp] = nx[pp];
+                    u[0] = nu.x, u[1] = nu.y, u[2] = nu.z, u[3] = nu.w;
                     up += N;
+                    if (k + 1 < K) {
+                        nu = quad(up);
+#pragma unroll
+                        for (int pp = 0; pp < NP; pp++) fetch(gp + pp * KN + N, nx[pp]);
+                    }
+#pragma unroll
+                    for (int pp = 0; pp < NP; pp++) {
+                        Stencil<RD> s;
+                        gather(cur[pp], gp + pp * KN, s);
+                        s.diffused(eps_p, ph[pp]);
+#pragma unroll
+                        for (int c = 0; c < 4; c++) al[c] = al[c] & (ph[pp][c] > eps_p);
+                    }
                     if (want) {
-                        float4 cc4[NQ];
-                        u[0] = nu.x, u[1] = nu.y, u[2] = nu.z, u[3] = nu.w;
-#pragma unroll
-                        for (int pp = 0; pp < NP; pp++) cc4[pp] = nc[pp];
-                        if (k + 1 < K) {
-                            nu = quad(up);
-#pragma unroll
-                            for (int pp = 0; pp < NP; pp++) nc[pp] = quad(gp + pp * KN + N);
-                        }
-#pragma unroll
-                        for (int pp = 0; pp < NP; pp++) {
-                            Stencil<RD> s;
-                            s.load(gp + pp * KN, ro, xl, xr, cc4[pp]);
-                            s.diffused(eps_p, ph[pp]);
-#pragma unroll
-                            for (int c = 0; c < 4; c++) al[c] = al[c] & (ph[pp][c] > eps_p);
-                        }
 #pragma unroll
                         for (int c = 0; c < 4; c++) {
                             const float sg = sg_of(c);

@@ -102,7 +102,12 @@ __global__ void __launch_bounds__(T, 3) k_rows_r2c(FftParams p)
         auto ld_s = [&](int b, int i) { return sm[b * M + i]; };
         fft_run<M, NB, T, false, false, ROW_RMAX>(p.tw_M, ld_s, sld, sst, sst);
     } else {
-        auto ld_g = [&](int b, int i) { return __ldg(&src[(size_t)b * M + i]); };
+        // (rows that may start at any float: scalar loads)
+        const float* srcf = plane + (size_t)y0 * W;
+        auto ld_g = [&](int b, int i) {
+            const float* q = srcf + 2 * ((size_t)b * M + i);
+            return make_float2(__ldg(q), __ldg(q + 1));
+        };
         fft_run<M, NB, T, false, false, ROW_RMAX>(p.tw_M, ld_g, sld, sst, sst);
     }
 

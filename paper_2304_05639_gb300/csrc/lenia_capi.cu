@@ -37,8 +37,8 @@ struct lenia_ctx {
     // small worlds with global genes: rollouts in one cooperative launch
     bool small = false;
     unsigned* d_small_count = nullptr;
-    int2* d_small_taps = nullptr;
-    std::vector<int> small_tap_off;
+    int2* d_taps = nullptr;
+    std::vector<int> tap_off;
     // the smallest of them: rollouts in one thread-block cluster (cr_Q blocks)
     int cr_Q = 0;
     float* d_cr_w = nullptr;
@@ -587,11 +587,8 @@ lenia_status step_impl(lenia_ctx* c, const float* A_in, const float* P_in, float
             const bool fast = epilogue_rows_supported(ep) && !quads11;
             GuardParams g;
             if (settle) {
-                g.w = c->d_w;
-                g.w_off = c->d_w_off;
-                g.yr = c->d_yr;
-                g.yr_off = c->d_yr_off;
-                for (int k = 0; k < c->cfg.n_kernels; k++) g.R[k] = c->conv_R[k];
+                g.taps = c->d_taps;
+                for (int k = 0; k <= c->cfg.n_kernels; k++) g.off[k] = c->tap_off[k];
                 g.du = c->guard_du;
             }
             CUDA_OR_FAIL(c, launch_epilogue_sites(ep, fast, settle ? &g : nullptr, 1, kSitesBlocksPerSm * c->num_sms, s, &nb));
@@ -759,7 +756,7 @@ void lenia_destroy(lenia_ctx* c)
                     c->d_Ahat_t, c->d_Uhat_t, c->d_ticket, c->d_walls, c->d_alpha_e, c->d_empty,
                     c->d_Useg, c->d_hA_in1, c->d_hP_in1, c->d_hA_out1,
                     c->d_hP_out1, c->d_hstats, c->d_tc_hi, c->d_tc_lo, c->d_tc_B, c->d_tc_ks,
-                    c->d_tc_grp, c->d_tc_has, c->d_small_count, c->d_small_taps, c->d_cr_w, c->d_tS, c->d_tS0,
+                    c->d_tc_grp, c->d_tc_has, c->d_small_count, c->d_taps, c->d_cr_w, c->d_tS, c->d_tS0,
                     c->d_ttw};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -942,7 +939,7 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
          (!cfg->maintain_genes || (epilogue_sites_supported(epi_params(c)) &&
                                    !(cfg->alpha_on && fabsf(cfg->eps_u) < 1e-4f))))) {
         memset(&c->tl, 0, sizeof(c->tl));
-        const double t_tile = tile_choose(&c->tl, H, W, kcount, c->max_R);
+        const double t_tile = tile_choose(&c->tl, H, W, kcount, c->max_R, 1, cfg->maintain_genes != 0);
         const double t_else = path == LENIA_CONV_FFT ? fft_passes_cost(H, W, C + NC) : direct_cost(H, W, NC, c->max_R);
         c->tile = t_tile < t_else;
         // one-channel worlds of one window: whole rollouts in one block, so the
@@ -990,13 +987,15 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
         }
     }
 
-    // small worlds with global genes on the direct route: their rollouts run
-    // as one cooperative launch over every kernel's non-zero taps (in the
-    // direct route's order: tap columns dx, then rows dy)
-    if (c->n_p == 0 && !cfg->maintain_genes && c->cfg.n_rings == 0 && cfg->conv_path == LENIA_CONV_DIRECT &&
-        NC == K) {
+    // every kernel's non-zero taps in the direct route's order (tap columns dx, then
+    // rows dy): for small worlds with global genes on the direct route, whose
+    // rollouts run as one cooperative launch over them, and for the alpha
+    // decisions that windows leave to the direct sums
+    const bool small_rule = c->n_p == 0 && !cfg->maintain_genes && !n_rings && cfg->conv_path == LENIA_CONV_DIRECT;
+    const bool settles = c->tile && path == LENIA_CONV_DIRECT && cfg->maintain_genes;
+    if (small_rule || settles) {
         std::vector<int2> taps;
-        c->small_tap_off.assign(1, 0);
+        c->tap_off.assign(1, 0);
         for (int k = 0; k < NC; k++) {
             const int R = c->conv_R[k], n = 2 * R + 1;
             for (int dx = -R; dx <= R; dx++)
@@ -1008,14 +1007,16 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
                     memcpy(&bits, &f, 4);
                     taps.push_back(make_int2((dy + 1024) * 2048 + (dx + 1024), bits));
                 }
-            c->small_tap_off.push_back((int)taps.size());
+            c->tap_off.push_back((int)taps.size());
         }
-        c->small = small_rollout_supported(H, W, C, NC, c->max_R, (int)taps.size());
-        if (c->small) {
-            ALLOC(c->d_small_count, 1);
-            ALLOC(c->d_small_taps, taps.size());
-            CK_INIT(cudaMemcpy(c->d_small_taps, taps.data(), taps.size() * sizeof(int2), cudaMemcpyHostToDevice));
+        c->small = small_rule && small_rollout_supported(H, W, C, NC, c->max_R, (int)taps.size());
+        if (c->small || settles) {
+            ALLOC(c->d_taps, taps.size());
+            CK_INIT(cudaMemcpy(c->d_taps, taps.data(), taps.size() * sizeof(int2), cudaMemcpyHostToDevice));
         }
+        if (c->small) ALLOC(c->d_small_count, 1);
+    }
+    if (small_rule) {
         // dense (2 maxR + 1)^2 kernels, each centred, for the cluster rollout
         c->cr_Q = cluster_rollout_blocks(H, W, C, NC, c->max_R);
         if (c->cr_Q) {
@@ -1347,9 +1348,9 @@ lenia_status lenia_rollout(lenia_ctx* c, float* A, float* P, int32_t n_steps, fl
         memset(&sp, 0, sizeof(sp));
         sp.A = A;
         sp.buf = c->d_A2;
-        sp.taps = c->d_small_taps;
-        for (int k = 0; k <= c->cfg.n_kernels; k++) sp.tap_off[k] = c->small_tap_off[k];
-        sp.n_taps = c->small_tap_off.back();
+        sp.taps = c->d_taps;
+        for (int k = 0; k <= c->cfg.n_kernels; k++) sp.tap_off[k] = c->tap_off[k];
+        sp.n_taps = c->tap_off.back();
         sp.kt = c->kt;
         sp.H = c->cfg.height;
         sp.W = c->cfg.width;
@@ -1547,7 +1548,15 @@ lenia_status lenia_potentials(lenia_ctx* c, const float* A_in, float* U_out, voi
     if (ranges_overlap(A_in, c->N * c->cfg.n_channels * sizeof(float), U_out,
                        c->N * c->cfg.n_kernels * sizeof(float)))
         return fail(c, LENIA_EINVAL, "A_in and U_out overlap");
-    return potentials(c, A_in, U_out, (cudaStream_t)stream);
+    cudaStream_t s = (cudaStream_t)stream;
+    const bool tc = c->path == LENIA_CONV_DIRECT_BF16 || c->path == LENIA_CONV_DIRECT_BF16X3;
+    const uintptr_t unit = tc ? 15 : (c->path == LENIA_CONV_FFT && !c->tile ? 7 : 3);
+    if (((uintptr_t)U_out & unit) == 0) return potentials(c, A_in, U_out, s);
+    // these forms write pairs or quads: an output that starts between them is copied
+    const lenia_status st = potentials(c, A_in, c->d_U, s);
+    if (st != LENIA_OK) return st;
+    CUDA_OR_FAIL(c, cudaMemcpyAsync(U_out, c->d_U, c->N * c->conv_w.size() * sizeof(float), cudaMemcpyDeviceToDevice, s));
+    return LENIA_OK;
 }
 
 lenia_status lenia_update_from_potentials(lenia_ctx* c, const float* A_in, const float* P_in, const float* U_in,

@@ -311,7 +311,8 @@ bool tile_plan(TileParams* p, int N, int H, int W, int R);
 // The faster window size and kernels per block (in p; the model's time in us, or
 // infinity where no window serves R), and the models of the other routes.
 // (n_worlds: worlds of that shape in one launch)
-double tile_choose(TileParams* p, int H, int W, const int* kcount, int R, int n_worlds = 1);
+double tile_choose(TileParams* p, int H, int W, const int* kcount, int R, int n_worlds = 1,
+                   bool gated = false);
 // time models of the transposed convolution: summed per channel in the frequency
 // domain, or plane by plane
 double tile_adj_cost(const TileParams& p, const int* kcount);
@@ -412,10 +413,9 @@ bool epilogue_gated(const EpiParams& p);
 // where a potential within du of its value would change the test, that
 // potential is summed directly.
 struct GuardParams {
-    const float* w;            // as ConvParams
-    const int *w_off, *yr, *yr_off;
-    int R[kMaxKernels];
-    float du;                  // 0: no guard
+    const int2* taps;          // as SmallRolloutParams, kernel k's at off[k] .. off[k + 1] - 1
+    int off[kMaxKernels + 1];
+    float du;                  // 0: the potentials are the direct sums already
 };
 // fast: the streaming kernel's reciprocals and exponential, else divisions and expf
 cudaError_t launch_epilogue_sites(const EpiParams& p, bool fast, const GuardParams* guard, int n_worlds, int max_blocks,
