@@ -91,12 +91,12 @@ __device__ __forceinline__ float2 ctw(float2 a)
     }
 }
 
-template <int N>
+template <int N, int NT = 2 * N>
 struct TC {
     static constexpr int M = N / 2;            // complex values per row
     static constexpr int CA = N / 8;           // column transform: CA x 8
     static constexpr int RR = M / 8;           // row transform: RR x 8
-    static constexpr int T = 2 * N;            // threads
+    static constexpr int T = NT;               // threads: 2 N or 4 N (see launch_n)
     static constexpr int NW = T / 32;          // warps
     static constexpr int CH = M / 32;          // 32-column halves
     static constexpr int TMEM = N == 128 ? 128 : 32;      // TMEM columns of a block
@@ -253,11 +253,11 @@ struct Window {                     // the tile of a block
 };
 
 // Forward transform of one plane's window up to the last column pass.
-template <int N>
+template <int N, int NT>
 __device__ __forceinline__ void forward_start(const TileParams& p, const float* plane, const Window& w,
                                               unsigned char* buf)
 {
-    using X = TC<N>;
+    using X = TC<N, NT>;
     const int lane = w.lane, warp = w.warp;
     const bool inside = w.x0 >= w.g.halo_x && w.x0 - w.g.halo_x + N <= p.W && w.y0 >= w.g.halo_y &&
                         w.y0 - w.g.halo_y + N <= p.H;
@@ -338,12 +338,12 @@ __device__ __forceinline__ void cols_inv(unsigned char* buf, const float2* twc, 
 }
 
 // Forward transform; task i's CA spectrum values go to `sink(i, c, b, v)`.
-template <int N, int UNR, class Sink>
+template <int N, int NT, int UNR, class Sink>
 __device__ __forceinline__ void forward(const TileParams& p, const float* plane, const Window& w, unsigned char* buf,
                                         const float2* twc, Sink sink)
 {
-    using X = TC<N>;
-    forward_start<N>(p, plane, w, buf);
+    using X = TC<N, NT>;
+    forward_start<N, NT>(p, plane, w, buf);
     constexpr int TASKS = 8 * X::CH / X::NW;             // per warp
 #pragma unroll UNR
     for (int i = 0; i < TASKS; i++) {
@@ -358,10 +358,10 @@ __device__ __forceinline__ void forward(const TileParams& p, const float* plane,
 // Inverse transform after its first column pass; the real rows go to
 // `out(y, m, off, value)` (window row y < rows, sites 2m and 2m + 1; off: where the
 // value's element of the buffer was).
-template <int N, class Out>
+template <int N, int NT, class Out>
 __device__ __forceinline__ void inverse_end(const Window& w, int rows, unsigned char* buf, Out out)
 {
-    using X = TC<N>;
+    using X = TC<N, NT>;
     const int lane = w.lane, warp = w.warp;
     __syncthreads();
 #pragma unroll 1
@@ -437,11 +437,11 @@ __device__ __forceinline__ void spectral_product(const float* S, const float* S0
 }
 
 // Inverse transform of the spectrum that `source(i, c, b, v)` yields per task.
-template <int N, int UNR, class Source, class Out>
+template <int N, int NT, int UNR, class Source, class Out>
 __device__ __forceinline__ void inverse(const Window& w, int rows, unsigned char* buf, const float2* twc,
                                         Source source, Out out)
 {
-    using X = TC<N>;
+    using X = TC<N, NT>;
     constexpr int TASKS = 8 * X::CH / X::NW;
 #pragma unroll UNR
     for (int i = 0; i < TASKS; i++) {
@@ -451,15 +451,15 @@ __device__ __forceinline__ void inverse(const Window& w, int rows, unsigned char
         source(i, c, b, v);
         cols_inv<N>(buf, twc, c, b, v);
     }
-    inverse_end<N>(w, rows, buf, out);
+    inverse_end<N, NT>(w, rows, buf, out);
 }
 
 // Whether any value of the plane `gate` within gate_r of the output tile is above
 // gate_eps (whole quads of columns, so a few columns more on either side).
-template <int N>
+template <int N, int NT>
 __device__ __forceinline__ bool window_live(const float* gate, const TileParams& p, const Window& w, int rows, int xend)
 {
-    constexpr int NW = TC<N>::NW, RB = 7;
+    constexpr int NW = TC<N, NT>::NW, RB = 7;
     const int nr = rows + 2 * p.gate_r, ys = w.y0 - p.gate_r;
     const int q0 = (w.x0 - p.gate_r + 4) / 4 - 1, nq = (w.x0 + xend + p.gate_r + 3) / 4 - q0;   // quads, from q0 >= -1
     bool any = false;
@@ -492,11 +492,12 @@ __device__ __forceinline__ bool window_live(const float* gate, const TileParams&
 // whose output tile has no gene within the diffusion disk of any site does
 // nothing: alpha is false at all of its sites, so the step never reads
 // their potentials.
-template <int N, bool ADJ>
-__global__ void __launch_bounds__(2 * N, N == 128 ? 3 : (ADJ ? 6 : 8)) k_tile_conv(const __grid_constant__ TileParams p)
+template <int N, int NT, bool ADJ>
+__global__ void __launch_bounds__(NT, NT == 4 * N ? (N == 128 ? 2 : (ADJ ? 4 : 5)) : (N == 128 ? 3 : (ADJ ? 6 : 8)))
+k_tile_conv(const __grid_constant__ TileParams p)
 {
     pdl_enter();
-    using X = TC<N>;
+    using X = TC<N, NT>;
     extern __shared__ __align__(128) unsigned char buf[];
     float2* F0 = reinterpret_cast<float2*>(buf + (size_t)N * X::M * 8);     // spectrum column 0 (ADJ: its mirrored sum)
     float2* twc = F0 + N;                                                    // [b][n1] w_N^(n1 b)
@@ -523,7 +524,7 @@ __global__ void __launch_bounds__(2 * N, N == 128 ? 3 : (ADJ ? 6 : 8)) k_tile_co
     const int rows = min(w.g.vy, p.H - w.y0);
     const int xend = min(w.g.vx, p.W - w.x0);
     if constexpr (!ADJ) {
-        if (p.gate && !window_live<N>(p.gate, p, w, rows, xend)) return;
+        if (p.gate && !window_live<N, NT>(p.gate, p, w, rows, xend)) return;
     }
     if (w.warp == 0) {
         tmem_alloc<X::TMEM>(&tmem_base);
@@ -552,7 +553,7 @@ __global__ void __launch_bounds__(2 * N, N == 128 ? 3 : (ADJ ? 6 : 8)) k_tile_co
     };
     const size_t SP = (size_t)N * X::M;                                      // floats of one kernel spectrum
     if constexpr (!ADJ) {
-        forward<N, UNR>(p, gA + (size_t)w.c * HW, w, buf, twc, [&](int i, int c, int b, float2* v) {
+        forward<N, NT, UNR>(p, gA + (size_t)w.c * HW, w, buf, twc, [&](int i, int c, int b, float2* v) {
             tput(i, v);
             if (c == 0)
 #pragma unroll
@@ -563,7 +564,7 @@ __global__ void __launch_bounds__(2 * N, N == 128 ? 3 : (ADJ ? 6 : 8)) k_tile_co
         for (int t = t0; t < t1; t++) {
             const int k = p.per_plane ? w.c : p.klist[w.c][t];
             float* U = gU + (size_t)k * HW;
-            inverse<N, UNR>(
+            inverse<N, NT, UNR>(
                 w, rows, buf, twc,
                 [&](int i, int c, int b, float2* v) {
                     tget(i, v);
@@ -584,7 +585,7 @@ __global__ void __launch_bounds__(2 * N, N == 128 ? 3 : (ADJ ? 6 : 8)) k_tile_co
     } else {
         for (int t = 0; t < nk; t++) {
             const int k = p.klist[w.c][t];
-            forward<N, UNR>(p, gA + (size_t)k * HW, w, buf, twc, [&](int i, int c, int b, float2* v) {
+            forward<N, NT, UNR>(p, gA + (size_t)k * HW, w, buf, twc, [&](int i, int c, int b, float2* v) {
                 if (c == 0) {
                     // mirrored share of the packed column, at -ky (this thread's slots only)
                     const float* s2 = gS0 + (size_t)k * N;
@@ -611,7 +612,7 @@ __global__ void __launch_bounds__(2 * N, N == 128 ? 3 : (ADJ ? 6 : 8)) k_tile_co
         }
         float* O = gU + (size_t)w.c * HW;
         const float* add = p.add ? p.add + (size_t)w.c * HW : nullptr;
-        inverse<N, UNR>(
+        inverse<N, NT, UNR>(
             w, rows, buf, twc,
             [&](int i, int c, int b, float2* v) {
                 tget(i, v);
@@ -792,17 +793,53 @@ __global__ void k_tile_spectra(const float* S, float* out, float* out0)
     out[(((size_t)b * (CA / 4) + a / 4) * M + c) * 4 + a % 4] = 0.5f * v;
 }
 
+// Blocks of one window and one share of a channel's kernels.
+dim3 conv_grid(const TileParams& p, bool adj)
+{
+    int kmax = p.per_plane ? 1 : 0;
+    for (int c = 0; c < p.C && c < kMaxChannels && !p.per_plane; c++) kmax = p.kcount[c] > kmax ? p.kcount[c] : kmax;
+    return dim3(p.worlds ? p.tiles : p.g.tiles_x * p.g.tiles_y, p.worlds ? p.C * p.n_worlds : p.C,
+                adj ? (kmax > 0) : (kmax + p.kpb - 1) / p.kpb);
+}
+
+template <int N, int NT, bool ADJ>
+cudaError_t launch_nt(const TileParams& p, const dim3& grid, cudaStream_t s)
+{
+    cudaError_t e = smem_limit<k_tile_conv<N, NT, ADJ>>(TC<N, NT>::SMEM);
+    if (e != cudaSuccess) return e;
+    launch_pdl(k_tile_conv<N, NT, ADJ>, grid, NT, TC<N, NT>::SMEM, s, p);
+    return cudaGetLastError();
+}
+
+// Threads of a block.  Each pass has the same tasks with either count, so the
+// values do not depend on it.  With few blocks the SMs are short of warps and
+// 4 N threads are faster; with many, 2 N keep more windows in flight and spare
+// registers.  Measured (us, 2 N against 4 N threads; R = 18 unless stated):
+//   N = 64   one window 5.8 / 4.8, 300 x 404 6.5 / 5.5, 256^2 15 kernels in 147
+//            blocks 15.9 / 14.4, in 245 12.9 / 12.4, in 390 12.4 / 12.6, in 735
+//            13.6 / 14.6, 1080 x 1920 15 kernels 131 / 143
+//   N = 128  256^2 15 kernels in 135 blocks 12.6 / 11.0, 1024^2 one kernel (121
+//            blocks) 11.8 / 10.4, 2048^2 one kernel (441) 23.1 / 24.0, 15 kernels
+//            190 / 196
+// hence the line at two blocks an SM.  Where a gate skips windows the blocks
+// that work are few again (N = 128, 1080 x 1920 15 kernels, a quarter live:
+// 66 / 52; 2048^2, 28% live: 112 / 106).  The transposed sum of N = 128 would
+// spill at 4 N threads.
+bool wide_block(int N, double blocks, bool gated, bool adj)
+{
+    if (N == 128 && adj) return false;
+    return blocks <= 2 * 152 || (N == 128 && gated);
+}
+
 template <int N, bool ADJ>
 cudaError_t launch_n(const TileParams& p, cudaStream_t s)
 {
-    cudaError_t e = smem_limit<k_tile_conv<N, ADJ>>(TC<N>::SMEM);
-    if (e != cudaSuccess) return e;
-    int kmax = p.per_plane ? 1 : 0;
-    for (int c = 0; c < p.C && c < kMaxChannels && !p.per_plane; c++) kmax = p.kcount[c] > kmax ? p.kcount[c] : kmax;
-    if (kmax == 0) return cudaSuccess;
-    const dim3 grid(p.worlds ? p.tiles : p.g.tiles_x * p.g.tiles_y, p.worlds ? p.C * p.n_worlds : p.C, ADJ ? 1 : (kmax + p.kpb - 1) / p.kpb);
-    launch_pdl(k_tile_conv<N, ADJ>, grid, TC<N>::T, TC<N>::SMEM, s, p);
-    return cudaGetLastError();
+    const dim3 grid = conv_grid(p, ADJ);
+    if (grid.z == 0) return cudaSuccess;
+    if constexpr (!(N == 128 && ADJ)) {
+        if (wide_block(N, (double)grid.x * grid.y * grid.z, p.gate != nullptr, ADJ)) return launch_nt<N, 4 * N, ADJ>(p, grid, s);
+    }
+    return launch_nt<N, 2 * N, ADJ>(p, grid, s);
 }
 
 }  // namespace
@@ -840,10 +877,12 @@ bool tile_plan(TileParams* p, int N, int H, int W, int R)
 // Time model of one launch (us), fitted to measurements at 64^2 .. 2048^2: a
 // block's work is two units for the forward transform and one per kernel; a
 // unit takes t1 on an idle SM and tf with every block slot of the SM taken.
-static double tile_time(const TileParams& p, double blocks, double units)
+static double tile_time(const TileParams& p, double blocks, double units, bool adj)
 {
-    const double slots = 152.0 * (p.N == 128 ? 3 : 8);
-    const double t1 = p.N == 128 ? 2.3 : 0.9, tf = p.N == 128 ? 7.7 : 3.9;
+    const bool wide = wide_block(p.N, blocks, false, adj);
+    const double slots = 152.0 * (wide ? 2 : p.N == 128 ? 3 : 8);
+    const double t1 = p.N == 128 ? (wide ? 2.0 : 2.3) : wide ? 0.6 : 0.9;
+    const double tf = p.N == 128 ? (wide ? 3.8 : 7.7) : wide ? 2.2 : 4.2;
     const double waves = blocks / slots, whole = floor(waves), rest = waves - whole;
     return 3.0 + units * (whole * tf + (rest > 0 ? t1 + (tf - t1) * rest : 0));
 }
@@ -856,7 +895,7 @@ static double tile_cost(const TileParams& p, const int* kcount, int kpb, int n_w
         blocks += (double)n_worlds * p.g.tiles_x * p.g.tiles_y * ((kcount[c] + kpb - 1) / kpb);
         kmax = kcount[c] > kmax ? kcount[c] : kmax;
     }
-    return tile_time(p, blocks, 2 + (kpb < kmax ? kpb : kmax));
+    return tile_time(p, blocks, 2 + (kpb < kmax ? kpb : kmax), false);
 }
 
 double tile_adj_cost(const TileParams& p, const int* kcount)
@@ -866,12 +905,12 @@ double tile_adj_cost(const TileParams& p, const int* kcount)
         kmax = kcount[c] > kmax ? kcount[c] : kmax;
         chans += kcount[c] > 0;
     }
-    return tile_time(p, (double)p.g.tiles_x * p.g.tiles_y * chans, 1 + 2 * kmax);
+    return tile_time(p, (double)p.g.tiles_x * p.g.tiles_y * chans, 1 + 2 * kmax, true);
 }
 
 double tile_planes_cost(const TileParams& p, int K)
 {
-    return tile_time(p, (double)p.g.tiles_x * p.g.tiles_y * K, 3);
+    return tile_time(p, (double)p.g.tiles_x * p.g.tiles_y * K, 3, false);
 }
 
 double tile_choose(TileParams* p, int H, int W, const int* kcount, int R, int n_worlds, bool gated)

@@ -49,6 +49,16 @@ def test_window_potentials_match_oracle(shape):
     assert err <= TOL_U
 
 
+# grids below and above two blocks an SM, where a block's thread count changes
+@pytest.mark.parametrize("shape", [(900, 800, 5, 1), (1000, 1100, 5, 1), (300, 560, 20, 3), (600, 560, 20, 3)])
+def test_window_potentials_of_larger_grids_match_oracle(shape):
+    w = _global(*shape)
+    U, _ = gpu_potentials(w)
+    err = np.abs(U - _oracle_u(w)).max()
+    print(shape, "max |dU|", err)
+    assert err <= TOL_U
+
+
 @pytest.mark.parametrize("shape", SHAPES[2:8])
 def test_unaligned_state_equals_aligned(shape):
     """A caller's A that starts 4 bytes past an 8-byte boundary takes scalar loads: same bits."""
