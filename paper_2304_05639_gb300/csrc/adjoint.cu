@@ -166,7 +166,9 @@ cudaError_t launch_adjoint_epilogue(const AdjParams& p0, cudaStream_t s)
     AdjParams p = p0;
     for (int k = 0; k < p.kt.K; k++) p.inv_s2[k] = (float)(1.0 / ((double)p.kt.sigma[k] * p.kt.sigma[k]));
     const size_t smem = (size_t)(p.kt.K + 2 * p.kt.C + 3 * ADJ_KB) * ADJ_THREADS * sizeof(float);
-    cudaError_t e = smem_limit<k_adjoint_epilogue>(smem);
+    // one limit for every kernel count: threads with different worlds may come here at once
+    constexpr size_t most = (size_t)(kMaxKernels + 2 * kMaxChannels + 3 * ADJ_KB) * ADJ_THREADS * sizeof(float);
+    cudaError_t e = smem_limit<k_adjoint_epilogue>(most);
     if (e != cudaSuccess) return e;
     launch_pdl(k_adjoint_epilogue, adjoint_blocks(p.H, p.W), ADJ_THREADS, smem, s, p);
     return cudaGetLastError();
