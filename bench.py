@@ -566,7 +566,10 @@ def direct_leg(torch, lenia, inputs, stream, fp32_peak=None, bf16_peak=None, ste
              "ms_per_step": step_ms, "value": w.sites / (step_ms / 1e3), "unit": UNIT, "conv_ms": conv_ms,
              "kernels_ms": kern, "useful_conv_tflops": useful / (conv_ms / 1e3) / 1e12 if conv_ms else None}
         if used == lenia.CONV_DIRECT and fp32_peak:
-            r["fp32_frac"] = r["useful_conv_tflops"] / fp32_peak
+            if path == lenia.CONV_AUTO:
+                r["note"] = "AUTO may convolve in spectral windows; useful_conv_tflops counts the direct sums' operations"
+            else:
+                r["fp32_frac"] = r["useful_conv_tflops"] / fp32_peak
         if used in (lenia.CONV_DIRECT_BF16, lenia.CONV_DIRECT_BF16X3):
             terms = 1 if used == lenia.CONV_DIRECT_BF16 else 3
             issued = 2.0 * sum(ksteps) * 16 * 32 * 256 * terms * (w.sites / (32 * 256))
