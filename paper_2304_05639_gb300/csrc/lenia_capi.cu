@@ -150,9 +150,12 @@ static_assert(sizeof(kKindNames) / sizeof(kKindNames[0]) == KIND_COUNT, "one nam
 
 namespace {
 
-// blocks of the per-site kernel per SM: enough to even out live and empty parts of
-// a world, few enough for their statistics records
-constexpr int kSitesBlocksPerSm = 24;
+// Blocks of the per-site kernel per SM, four of which run at once: enough to even out
+// live and empty parts of a world, few enough for their statistics records.  Step
+// times (us) with 8 / 16 / 24 / 32: 1080 x 1920, 15 kernels, with 3, 16 or 60 patches
+// 143 / 138 / 149 / 152, 203 / 199 / 200 / 207, 281 / 268 / 278 / 273; 2048^2, R = 5,
+// 336 / 323 / 325 / 316, nearly all live 526 / 529 / 529 / 523.
+constexpr int kSitesBlocksPerSm = 16;
 
 const double kTwoPi = 6.283185307179586476925286766559;
 
