@@ -937,10 +937,7 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
     // where that would be every empty site, keeps the sums throughout, and so
     // do ring worlds and an explicit LENIA_CONV_DIRECT.
     const bool want_adj = cfg->max_rollout_steps > 0 && c->n_p == 0 && !cfg->maintain_genes;
-    // (A 64^2 world that is differentiated keeps the passes: a 64-point axis is one or two
-    // of their large radices, and their gradients are closer to 64 bits: 1.9e-7 against
-    // 2.7e-7 after 8 steps.  From 128 on the windows are the closer ones.)
-    if ((path == LENIA_CONV_FFT && !cfg->maintain_genes && !(want_adj && H == 64 && W == 64)) ||
+    if ((path == LENIA_CONV_FFT && !cfg->maintain_genes) ||
         (path == LENIA_CONV_DIRECT && cfg->conv_path == LENIA_CONV_AUTO && !n_rings &&
          (!cfg->maintain_genes || (epilogue_sites_supported(epi_params(c)) &&
                                    !(cfg->alpha_on && fabsf(cfg->eps_u) < 1e-4f))))) {
