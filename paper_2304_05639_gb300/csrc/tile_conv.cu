@@ -490,7 +490,7 @@ __device__ __forceinline__ bool window_live(const float* gate, const TileParams&
 // One block: a window of channel blockIdx.y, kernels blockIdx.z kpb .. of its
 // list.  ADJ: the transpose, out_c = add_c + sum_{k in list(c)} K~_k (x) plane k:
 // every listed plane is transformed forward, weighted and summed in TMEM, and
-// one inverse transform follows.
+// one inverse transform follows (a channel that no kernel reads gets add_c).
 // With a gate (the first gene plane of a world that maintains its genes) a block
 // whose output tile has no gene within the diffusion disk of any site does
 // nothing: alpha is false at all of its sites, so the step never reads
@@ -519,7 +519,7 @@ k_tile_conv(const __grid_constant__ TileParams p)
     const float* gS0 = tw ? tw->S0 : p.S0;
     const int nk = !ADJ && p.per_plane ? 1 : p.kcount[w.c];
     const int t0 = ADJ ? 0 : (int)blockIdx.z * p.kpb;
-    if (t0 >= nk) return;                                                    // uniform over the block
+    if (!ADJ && t0 >= nk) return;                                            // uniform over the block
     const int t1 = ADJ ? nk : min(nk, t0 + p.kpb);
     w.x0 = (int)(blockIdx.x % w.g.tiles_x) * w.g.vx;
     w.y0 = (int)(blockIdx.x / w.g.tiles_x) * w.g.vy;
@@ -528,6 +528,13 @@ k_tile_conv(const __grid_constant__ TileParams p)
     const int xend = min(w.g.vx, p.W - w.x0);
     if constexpr (!ADJ) {
         if (p.gate && !window_live<N, NT>(p.gate, p, w, rows, xend)) return;
+    } else if (nk == 0) {
+        // a channel that no kernel reads: its sum is empty
+        for (int i = threadIdx.x; i < rows * xend; i += X::T) {
+            const size_t o = (size_t)w.c * HW + (size_t)(w.y0 + i / xend) * p.W + w.x0 + i % xend;
+            gU[o] = p.add ? __ldg(p.add + o) : 0.f;
+        }
+        return;
     }
     if (w.warp == 0) {
         tmem_alloc<X::TMEM>(&tmem_base);
