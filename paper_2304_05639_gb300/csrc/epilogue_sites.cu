@@ -379,12 +379,14 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                             gk[c] = sg > 0.f ? e : 0.f;
                             tk[c] = p.alpha_on ? u[c] : h_of(c) * gk[c];
                             if (NP > 0) {
-                                // how far the test may be off: rounding, and the potential's du
-                                // through |d t / d u| = t |z| / s (doubled for its curvature); a
-                                // bump narrower than du's reach is always settled
-                                const float off = p.alpha_on
-                                                      ? q.g.du + 1e-7f * fabsf(u[c])
-                                                      : fabsf(tk[c]) * fmaf(2e-6f, z2, fmaf(2.f * q.g.du * rs, fabsf(z), 2e-6f));
+                                // how far the test may be off: rounding, and the potential's du.
+                                // With eta = du / s <= 1/64 the bump's ratio at z + d, |d| <= eta, is
+                                // exp(-z d - d^2 / 2): off by at most 2 |z| eta + eta^2 (|z| eta <= 5/4;
+                                // beyond it both bumps are zero).  A narrower one is always settled
+                                const float eta = q.g.du * rs;
+                                const float off =
+                                    p.alpha_on ? q.g.du + 1e-7f * fabsf(u[c])
+                                               : fabsf(tk[c]) * fmaf(2e-6f, z2, fmaf(eta, fmaf(2.f, fabsf(z), eta), 2e-6f));
                                 const bool narrow = sg < q.g.du * 64.f;
                                 if (p.empty_out) tband[c] += narrow ? fabsf(h_of(c)) : off;
                                 near |= (al[c] & (narrow | (fabsf(tk[c] - eps_u) <= off)) ? 1u : 0u) << c;

@@ -45,3 +45,58 @@ def test_gradient_of_channels_that_no_kernel_reads(shape, topology):
     for c in range(C):
         assert float((a[c] - b[c]).norm()) <= 1e-4 * float(b[c].norm())
     assert float((ga - gb).norm()) <= 1e-4 * float(gb.norm())
+
+
+def _potentials_of(w, path, A):
+    g = inputs.World(w.height, w.width, w.n_channels, w.kernels, w.dt, localized=0, maintain_genes=0)
+    return gpu_potentials(g, path, A)[0]
+
+
+def _decisions(w, path):
+    """(alpha, E_pen) of one evolution step without mutation or penalisation."""
+    torch = torch_mod()
+    ev = inputs.evolution_events(w, 0, gamma_mut=0.0, gamma_pen=0.0)
+    cfg, ks = lenia.config_from_world(w, path)
+    ctx = lenia.lenia_init(cfg, ks)
+    try:
+        A, P = to_dev(w.A), to_dev(w.P) if w.n_planes else None
+        A2, P2 = torch.empty_like(A), torch.empty_like(P) if w.n_planes else None
+        al = torch.zeros((w.height, w.width), dtype=torch.uint8, device="cuda")
+        ep = torch.zeros((w.height, w.width), dtype=torch.float32, device="cuda")
+        lenia.lenia_step_evolve(ctx, A, P, A2, P2, ev, None, al, ep)
+        torch.cuda.synchronize()
+        return al.cpu().numpy(), ep.cpu().numpy()
+    finally:
+        lenia.lenia_destroy(ctx)
+
+
+def _uniform_at_threshold(w, sigma, z, on_windows, n_levels=24):
+    """Makes a uniform world of w, at the level (of n_levels) where the direct sums'
+    one potential and the windows' are furthest apart.  Returns (mu, eps_u): a bump
+    of width sigma z widths above the windows' (or the sums') potential, and a
+    threshold half-way between the two routes' bumps."""
+    best = None
+    for level in np.linspace(0.3, 1.0, n_levels):
+        A = np.full(w.A.shape, level, np.float32)
+        d, t = (_potentials_of(w, p, A) for p in (lenia.CONV_DIRECT, lenia.CONV_AUTO))
+        assert (d == d.flat[0]).all() and (d != t).any()
+        ud, uw = float(d.flat[0]), float(t.mean(dtype=np.float64))
+        if best is None or abs(ud - uw) > abs(best[0] - best[1]):
+            best = ud, uw, A
+    ud, uw, w.A = best
+    mu = np.float32((uw if on_windows else ud) - z * sigma)
+    bump = lambda v: np.exp(-0.5 * ((v - float(mu)) / float(np.float32(sigma))) ** 2)
+    print("direct", ud, "windows", uw, "bumps", bump(ud), bump(uw))
+    return mu, 0.5 * (bump(ud) + bump(uw))
+
+
+@pytest.mark.parametrize("sigma", [2e-4, 3e-4, 6e-4, 2e-3])
+@pytest.mark.parametrize("z", [0.0, 0.01, 0.2, 2.0])
+@pytest.mark.parametrize("on_windows", [False, True])
+def test_narrow_bumps_decide_as_the_direct_sums(sigma, z, on_windows):
+    w = inputs.localized_single_channel(H=130, W=132, R=31, patch=64, n_geno=1, live=True)
+    w.P[0], w.eps_u = _uniform_at_threshold(w, sigma, z, on_windows)
+    w.P[1] = np.float32(sigma)
+    a, b = _decisions(w, lenia.CONV_AUTO), _decisions(w, lenia.CONV_DIRECT)
+    np.testing.assert_array_equal(a[0], b[0])
+    np.testing.assert_array_equal(a[1], b[1])
