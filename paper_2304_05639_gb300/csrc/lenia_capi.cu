@@ -385,6 +385,30 @@ std::vector<float2> twiddles(int n, int count)
     return t;
 }
 
+// How far the windows' and the direct sums' potentials may be apart, for states of
+// magnitude at most 1.  The direct route adds a kernel's n taps one after the
+// other, each addition off by at most 2^-24 of the partial sum, so tap i's weight
+// is rounded n - i times: the bound grows with the taps (1.5e-5 at R = 13, 3.7e-5
+// at R = 20, 2.9e-4 at R = 56; uniform states reach 6e-6 there).  The windows stay
+// below 2.5e-7 of the absolute weights' sum (measured); four times that is allowed.
+float window_guard(const lenia_ctx* c)
+{
+    double most = 0.0;
+    for (size_t k = 0; k < c->conv_w.size(); k++) {
+        const int R = c->conv_R[k], n = 2 * R + 1;
+        double passed = 0.0, total = 0.0;      // sum_i |w_i| (n - i): every prefix sum once
+        for (int dx = 0; dx < n; dx++)
+            for (int dy = 0; dy < n; dy++) {
+                const double w = fabs((double)(float)c->conv_w[k][(size_t)dy * n + dx]);
+                if (w == 0.0) continue;
+                total += w;
+                passed += total;
+            }
+        most = std::max(most, passed * 5.9604644775390625e-8 + 1e-6 * total);
+    }
+    return (float)(1.001 * most);
+}
+
 // Spectra and twiddles of the context's windows (c->tl.N).  Waits for the work.
 lenia_status build_tiles(lenia_ctx* c, cudaStream_t s)
 {
@@ -934,13 +958,15 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
     // direct sums that AUTO falls back to.  The transforms round differently
     // from the sums, so alpha tests that this could turn are decided by the sums
     // (GuardParams); a world whose alpha tests potentials against (nearly) zero,
-    // where that would be every empty site, keeps the sums throughout, and so
-    // do ring worlds and an explicit LENIA_CONV_DIRECT.
+    // where that would be every empty site (one kernel's, or the sum of all of
+    // them), keeps the sums throughout, and so do ring worlds and an explicit
+    // LENIA_CONV_DIRECT.
     const bool want_adj = cfg->max_rollout_steps > 0 && c->n_p == 0 && !cfg->maintain_genes;
+    c->guard_du = window_guard(c);
     if ((path == LENIA_CONV_FFT && !cfg->maintain_genes) ||
         (path == LENIA_CONV_DIRECT && cfg->conv_path == LENIA_CONV_AUTO && !n_rings &&
          (!cfg->maintain_genes || (epilogue_sites_supported(epi_params(c)) &&
-                                   !(cfg->alpha_on && fabsf(cfg->eps_u) < 1e-4f))))) {
+                                   !(cfg->alpha_on && fabsf(cfg->eps_u) < std::max(1e-4f, 2.f * K * c->guard_du)))))) {
         memset(&c->tl, 0, sizeof(c->tl));
         const double t_tile = tile_choose(&c->tl, H, W, kcount, c->max_R, 1, cfg->maintain_genes != 0);
         const double t_else = path == LENIA_CONV_FFT ? fft_passes_cost(H, W, C + NC) : direct_cost(H, W, NC, c->max_R);
@@ -967,15 +993,6 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
     ALLOC(c->d_partials, (size_t)c->n_part_blocks * C * 5);
 
     if (c->tile) {
-        // FP32 rounding of either form, for values in [0, 1] and the kernels' absolute
-        // weights (measured: at most 8e-7 direct, 2.5e-7 windows, for weights that sum to 1)
-        double wabs = 0.0;
-        for (const std::vector<double>& w : c->conv_w) {
-            double t = 0.0;
-            for (double v : w) t += fabs(v);
-            wabs = std::max(wabs, t);
-        }
-        c->guard_du = (float)(4e-6 * wabs);
         int blocks = 0;
         for (int ch = 0; ch < C; ch++) blocks += c->tl.g.tiles_x * c->tl.g.tiles_y * ((kcount[ch] + c->tl.kpb - 1) / c->tl.kpb);
         c->gate_pays = blocks > c->num_sms * (c->tl.N == 128 ? 3 : 8);

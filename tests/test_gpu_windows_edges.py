@@ -2,6 +2,8 @@
 no kernel reads, narrow bumps and large radii (every alpha decision is that of
 the direct sums), values outside [0, 1], infinite genes, long sums, and groups
 of worlds.  GPU only."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -95,6 +97,27 @@ def _uniform_at_threshold(w, sigma, z, on_windows, n_levels=24):
 @pytest.mark.parametrize("on_windows", [False, True])
 def test_narrow_bumps_decide_as_the_direct_sums(sigma, z, on_windows):
     w = inputs.localized_single_channel(H=130, W=132, R=31, patch=64, n_geno=1, live=True)
+    w.P[0], w.eps_u = _uniform_at_threshold(w, sigma, z, on_windows)
+    w.P[1] = np.float32(sigma)
+    a, b = _decisions(w, lenia.CONV_AUTO), _decisions(w, lenia.CONV_DIRECT)
+    np.testing.assert_array_equal(a[0], b[0])
+    np.testing.assert_array_equal(a[1], b[1])
+
+
+FLAT = inputs.KernelDesc(0, 0, 1, inputs.KERNEL_BUMPS, (1.0,), bump=(0.0, 1e5, 1.0, 0.5, 0.1, 0.0))
+SHELL = inputs.KernelDesc(0, 0, 1, inputs.KERNEL_SHELLS, (1.0,))
+
+
+@pytest.mark.parametrize("shape", [(130, 132, 12), (300, 404, 20), (300, 404, 31), (600, 900, 56)])
+@pytest.mark.parametrize("kernel", [FLAT, SHELL], ids=["flat", "shell"])
+@pytest.mark.parametrize("sigma,z", [(0.03, 1.0), (0.004, 0.0)])
+@pytest.mark.parametrize("on_windows", [False, True])
+def test_the_sums_rounding_at_any_radius(shape, kernel, sigma, z, on_windows):
+    """The direct sums' rounding grows with their taps, most with equal weights (a flat
+    disk: 1.5e-5 at R = 20, 1.4e-4 at R = 56): the decisions are still theirs."""
+    H, W, R = shape
+    w = inputs.localized_single_channel(H=H, W=W, R=R, patch=64, n_geno=1, live=True)
+    w.kernels = [dataclasses.replace(w.kernels[0], form=kernel.form, beta=kernel.beta, bump=kernel.bump)]
     w.P[0], w.eps_u = _uniform_at_threshold(w, sigma, z, on_windows)
     w.P[1] = np.float32(sigma)
     a, b = _decisions(w, lenia.CONV_AUTO), _decisions(w, lenia.CONV_DIRECT)
