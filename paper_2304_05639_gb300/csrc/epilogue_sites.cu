@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                                 const float off =
                                     p.alpha_on ? q.g.du + 1e-7f * fabsf(u[c])
                                                : fabsf(tk[c]) * fmaf(2e-6f, z2, fmaf(eta, fmaf(2.f, fabsf(z), eta), 2e-6f));
-                                const bool narrow = sg < q.g.du * 64.f;
+                                const bool narrow = sg > 0.f && sg < q.g.du * 64.f;     // (sigma 0: no bump, on either route)
                                 if (p.empty_out) tband[c] += narrow ? fabsf(h_of(c)) : off;
                                 near |= (al[c] & (narrow | (fabsf(tk[c] - eps_u) <= off)) ? 1u : 0u) << c;
                             }
@@ -493,10 +493,12 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
             if (in && p.alpha_out)
                 *reinterpret_cast<uchar4*>(p.alpha_out + i0) =
                     NP == 0 ? make_uchar4(1, 1, 1, 1) : make_uchar4(al[0], al[1], al[2], al[3]);
+            // (no band: every test is exactly the direct route's, and so is their sum)
             if (NP > 0 && in && p.empty_out)
 #pragma unroll
                 for (int c = 0; c < 4; c++)
-                    if (fabsf(tsum[c] - eps_u) <= tband[c] + 1e-6f) tsum[c] = tests_at(q, pA, pP, pU, y, x + c);
+                    if (tband[c] > 0.f && fabsf(tsum[c] - eps_u) <= tband[c] + 1e-6f)
+                        tsum[c] = tests_at(q, pA, pP, pU, y, x + c);
             if (in && p.empty_out)
                 *reinterpret_cast<uchar4*>(p.empty_out + i0) =
                     make_uchar4(!(tsum[0] > eps_u), !(tsum[1] > eps_u), !(tsum[2] > eps_u), !(tsum[3] > eps_u));

@@ -123,3 +123,33 @@ def test_the_sums_rounding_at_any_radius(shape, kernel, sigma, z, on_windows):
     a, b = _decisions(w, lenia.CONV_AUTO), _decisions(w, lenia.CONV_DIRECT)
     np.testing.assert_array_equal(a[0], b[0])
     np.testing.assert_array_equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("eps_u", [0.0, 0.01])
+def test_evolution_on_a_mostly_empty_world_costs_no_more_than_direct_sums(eps_u):
+    """Sites without genes need no settling: their tests are zero on both routes."""
+    torch = torch_mod()
+    w = inputs.multi_channel(H=540, W=960, R=13, patch=64, n_geno=3, matched=True)
+    w.eps_u = eps_u
+    a, b = _decisions(w, lenia.CONV_AUTO), _decisions(w, lenia.CONV_DIRECT)
+    np.testing.assert_array_equal(a[0], b[0])
+    np.testing.assert_array_equal(a[1], b[1])
+    ev = inputs.evolution_events(w, 0)
+    us = []
+    for path in (lenia.CONV_AUTO, lenia.CONV_DIRECT):
+        cfg, ks = lenia.config_from_world(w, path)
+        ctx = lenia.lenia_init(cfg, ks)
+        A, P = to_dev(w.A), to_dev(w.P)
+        A2, P2 = torch.empty_like(A), torch.empty_like(P)
+        t = []
+        for i in range(8):
+            e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            e0.record()
+            lenia.lenia_step_evolve(ctx, A, P, A2, P2, ev)
+            e1.record()
+            torch.cuda.synchronize()
+            t.append(e0.elapsed_time(e1) * 1e3)
+        lenia.lenia_destroy(ctx)
+        us.append(float(np.median(t[3:])))
+    print("evolution step us, windows and direct sums:", us)
+    assert us[0] <= us[1]
