@@ -26,6 +26,7 @@
 // the issue slots used).  1080 x 1920, 15 kernels, 43% live: 121 us (533 with
 // the general kernel; 146 with every lane loading its own stencils); 2048^2 all live
 // 333 us; 512^2, 8 kernels, three genes, radius 2: 23 us (230).
+#include <math.h>
 #include <string.h>
 
 #include "lenia_internal.cuh"
@@ -42,6 +43,7 @@ struct SitesParams {
     int n_worlds;              // worlds of a batched launch (lists in e), else 1
     int tx, ty;                // blocks of 32 x 16 sites per world
     int gate;
+    int tiny_eps;              // the threshold lies where bumps underflow
     int fast;                  // settle with reciprocals and the hardware exponential, else divisions and expf
     GuardParams g;
 };
@@ -379,17 +381,32 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                             gk[c] = sg > 0.f ? e : 0.f;
                             tk[c] = p.alpha_on ? u[c] : h_of(c) * gk[c];
                             if (NP > 0) {
-                                // how far the test may be off: rounding, and the potential's du.
-                                // With eta = du / s <= 1/64 the bump's ratio at z + d, |d| <= eta, is
-                                // exp(-z d - d^2 / 2): off by at most 2 |z| eta + eta^2 (|z| eta <= 5/4;
-                                // beyond it both bumps are zero).  A narrower one is always settled
-                                const float eta = q.g.du * rs;
-                                const float off =
-                                    p.alpha_on ? q.g.du + 1e-7f * fabsf(u[c])
-                                               : fabsf(tk[c]) * fmaf(2e-6f, z2, fmaf(eta, fmaf(2.f, fabsf(z), eta), 2e-6f));
-                                const bool narrow = sg > 0.f && sg < q.g.du * 64.f;     // (sigma 0: no bump, on either route)
-                                if (p.empty_out) tband[c] += narrow ? fabsf(h_of(c)) : off;
-                                near |= (al[c] & (narrow | (fabsf(tk[c] - eps_u) <= off)) ? 1u : 0u) << c;
+                                // the test's range: rounding, and the potential's du.  With eta = du / s
+                                // <= 1/64 the bump's ratio at z + d, |d| <= eta, is exp(-z d - d^2 / 2):
+                                // off by at most 2 |z| eta + eta^2 (|z| eta <= 5/4; beyond it both
+                                // bumps are zero).  A narrower bump's range is formed at z -+ eta.
+                                const float eta = q.g.du * rs, az = fabsf(z);
+                                float lo, hi;
+                                if (p.alpha_on) {
+                                    const float off = fmaf(1e-7f, fabsf(u[c]), q.g.du);
+                                    lo = tk[c] - off;
+                                    hi = tk[c] + off;
+                                } else if (sg > 0.f && eta > 1.f / 64.f) {
+                                    const float hh = h_of(c), z0 = fmaxf(az - eta, 0.f), z1 = az + eta;
+                                    const float t0 = hh * ex2_approx(-0.721347520444481703680f * (z0 * z0));
+                                    const float t1 = hh * ex2_approx(-0.721347520444481703680f * (z1 * z1));
+                                    const float r = fabsf(t0) * fmaf(2e-6f, fminf(z0 * z0, 225.f), 2e-6f);
+                                    lo = fminf(t0, t1) - r;
+                                    hi = fmaxf(t0, t1) + r;
+                                } else {
+                                    float off = fabsf(tk[c]) * fmaf(2e-6f, z2, fmaf(eta, fmaf(2.f, az, eta), 2e-6f));
+                                    // thresholds at zero: where the bump underflows
+                                    if (q.tiny_eps && sg > 0.f && z2 < 225.f && fabsf(tk[c]) < 1e-36f) off = 1e-36f;
+                                    lo = tk[c] - off;
+                                    hi = tk[c] + off;
+                                }
+                                if (p.empty_out) tband[c] += hi - lo;
+                                near |= (al[c] & (lo <= eps_u) & (eps_u <= hi) ? 1u : 0u) << c;
                             }
                         }
                     }
@@ -562,6 +579,7 @@ cudaError_t launch_epilogue_sites(const EpiParams& p, bool fast, const GuardPara
     q.tx = (p.W + 4 * ES_Q - 1) / (4 * ES_Q);
     q.ty = (p.H + ES_Y - 1) / ES_Y;
     q.gate = epilogue_gated(p);
+    q.tiny_eps = fabsf(p.eps_u) < 1e-30f;
     q.fast = fast;
     if (p.n_p == 0) return launch_sites_c<0, 0>(q, max_blocks, s, n_blocks);
     if (p.r_diff == 1)

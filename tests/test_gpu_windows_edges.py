@@ -153,3 +153,16 @@ def test_evolution_on_a_mostly_empty_world_costs_no_more_than_direct_sums(eps_u)
         us.append(float(np.median(t[3:])))
     print("evolution step us, windows and direct sums:", us)
     assert us[0] <= us[1]
+
+
+@pytest.mark.parametrize("z", [14.0, 14.35, 14.4, 15.5])
+def test_thresholds_at_zero_decide_as_the_direct_sums(z):
+    """eps_u = 0: the decision lies where a bump underflows."""
+    w = inputs.localized_single_channel(H=130, W=132, R=31, patch=64, n_geno=1, live=True)
+    rng = np.random.default_rng(3)
+    w.A = (0.5 + 0.02 * rng.standard_normal(w.A.shape)).clip(0, 1).astype(np.float32)
+    w.P[0], w.P[1], w.eps_u = np.float32(0.5 - z * 0.03), np.float32(0.03), 0.0
+    a, b = _decisions(w, lenia.CONV_AUTO), _decisions(w, lenia.CONV_DIRECT)
+    print("alpha", b[0].mean())
+    np.testing.assert_array_equal(a[0], b[0])
+    np.testing.assert_array_equal(a[1], b[1])
