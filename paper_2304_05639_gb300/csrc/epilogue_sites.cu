@@ -406,7 +406,7 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                                     hi = tk[c] + off;
                                 }
                                 if (p.empty_out) tband[c] += hi - lo;
-                                near |= (al[c] & (lo <= eps_u) & (eps_u <= hi) ? 1u : 0u) << c;
+                                near |= (al[c] & (lo < eps_u) & (eps_u < hi) ? 1u : 0u) << c;   // (lo = hi: exact)
                             }
                         }
                     }
