@@ -107,6 +107,9 @@ struct Stencil {
                         s = first ? v[j][RD + c + d] : s + v[j][RD + c + d];
                         n = first ? one[j][RD + c + d] : n + one[j][RD + c + d];
                     }
+            // (a sum above the count gives 1, an infinite one too, where the quotient's
+            // correction would be infinity less infinity)
+            s = s > n ? n : s;
             const float rn = rcp_approx(n), t = s * rn;
             const float r = fmaf(fmaf(-t, n, s), rn, t);
             out[c] = n > 0.f ? __saturatef(r) : 0.f;

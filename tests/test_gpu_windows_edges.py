@@ -166,3 +166,35 @@ def test_thresholds_at_zero_decide_as_the_direct_sums(z):
     print("alpha", b[0].mean())
     np.testing.assert_array_equal(a[0], b[0])
     np.testing.assert_array_equal(a[1], b[1])
+
+
+def _near(H, W, y, x, R):
+    """Sites of a torus within |d| < R of (y, x)."""
+    dy = np.minimum((np.arange(H) - y) % H, (y - np.arange(H)) % H)
+    dx = np.minimum((np.arange(W) - x) % W, (x - np.arange(W)) % W)
+    return dy[:, None] ** 2 + dx[None, :] ** 2 < R * R
+
+
+@pytest.mark.parametrize("localized", [3, 7])
+@pytest.mark.parametrize("r_diff", [1, 2])
+@pytest.mark.parametrize("value", [np.inf, 3e38, 40.0])
+def test_diffused_genes_saturate(localized, r_diff, value):
+    """A gene above the disk's count diffuses to 1, an infinite one too."""
+    torch = torch_mod()
+    w = inputs.multi_channel(H=72, W=100, R=9, patch=40, n_geno=4, matched=True, localized=localized, seed_index=31,
+                             n_channels=2)
+    w.r_diff = r_diff
+    ys, xs = np.nonzero(w.P[0, 0] != 0)
+    y, x = ys[len(ys) // 2], xs[len(xs) // 2]
+    w.P[1, 2, y, x] = value
+    cfg, ks = lenia.config_from_world(w)
+    ctx = lenia.lenia_init(cfg, ks)
+    A, P = to_dev(w.A), to_dev(w.P)
+    A2, P2 = torch.empty_like(A), torch.empty_like(P)
+    lenia.lenia_step(ctx, A, P, A2, P2)
+    torch.cuda.synchronize()
+    lenia.lenia_destroy(ctx)
+    alpha = (P2.cpu().numpy() != 0).all(axis=(0, 1))
+    g = oracle.diffuse(w.P[1, 2], r_diff)
+    assert g[y, x] == 1.0 and alpha[_near(72, 100, y, x, r_diff + 1e-3)].any()
+    np.testing.assert_allclose(P2[1, 2].cpu().numpy()[alpha], g[alpha], atol=4e-7)
