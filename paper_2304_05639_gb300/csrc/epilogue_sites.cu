@@ -11,15 +11,19 @@
 //
 // Where the genes are maintained, a site whose disk holds no first gene above
 // eps_p has alpha = 0 whatever the rest says: its genes are zero and its update
-// is the per-channel constant.  Such sites (the empty part of a world, most
-// of it in the worlds of the paper) read one gene plane instead of all of
-// them and no potential.
+// is the per-channel constant.  A warp (32 columns x 4 rows) of such sites (the
+// empty part of a world, most of it in the worlds of the paper) reads one gene
+// plane instead of all of them and no potential.
 //
 // The arithmetic is the hardware reciprocal (with one correction for the genes)
 // and exponential.  Alpha tests that its rounding, or the rounding of the
-// windows' potentials, could turn are settled by the other update kernels'
-// arithmetic on the direct sums (`settle`), so that a world's decisions do
-// not depend on the kernel or the convolution it takes.
+// windows' potentials, could turn count as passed until the kernels are done; the
+// sites that hang on them are then dealt to the warp's lanes and settled by the
+// other update kernels' arithmetic on the direct sums, so that a world's
+// decisions do not depend on the kernel or the convolution it takes.  (Settled
+// inside the kernels' loop, or with a site of each lane at a time, the guard that
+// large radii need makes a step of 600 x 900 at R = 45 / 56 1.15 / 2.25 ms; 0.44 /
+// 0.72 so, 0.56 / 0.93 with the direct sums throughout.)
 //
 // What bounds it: on a mostly empty world the writes of the gene planes, on a
 // full one its loads and instruction issue (16 warps an SM at 128 registers, half of
@@ -127,37 +131,31 @@ __device__ __forceinline__ int tap_site(int2 tap, int y, int x, int H, int W)
 }
 
 // Kernel k's direct sum at (y, x): its non-zero taps in k_direct_conv's order (a zero
-// weight adds nothing there), so the same bits.
-__device__ __forceinline__ float direct_at(const SitesParams& q, const float* A, int k, int y, int x)
-{
-    const int H = q.e.H, W = q.e.W;
-    const float* plane = A + (size_t)q.e.kt.src[k] * H * W;
-    float acc = 0.f;
-    for (int t = q.g.off[k]; t < q.g.off[k + 1]; t++) {
-        const int2 tap = __ldg(&q.g.taps[t]);
-        acc = fmaf(__int_as_float(tap.y), __ldg(&plane[tap_site(tap, y, x, H, W)]), acc);
-    }
-    return acc;
-}
-
-// The same sum by a whole warp: the lanes load 8 x 32 taps at once and every lane
-// adds them in order.
+// weight adds nothing there), so the same bits.  By a whole warp: the lanes load
+// 4 x 32 taps at once, the next ones while every lane adds these in order.
 __device__ __forceinline__ float direct_warp(const SitesParams& q, const float* A, int k, int y, int x)
 {
-    constexpr int B = 8;
+    constexpr int B = 4;
     const int H = q.e.H, W = q.e.W, lane = threadIdx.x & 31;
     const float* plane = A + (size_t)q.e.kt.src[k] * H * W;
     const int t1 = q.g.off[k + 1];
-    float acc = 0.f;
-    for (int t0 = q.g.off[k]; t0 < t1; t0 += 32 * B) {
-        float v[B], w[B];
+    float vn[B], wn[B];
+    auto fetch = [&](int t0) {
 #pragma unroll
         for (int j = 0; j < B; j++) {
             const int t = t0 + 32 * j + lane;
             const int2 tap = t < t1 ? __ldg(&q.g.taps[t]) : make_int2((1024 << 11) + 1024, 0);
-            w[j] = __int_as_float(tap.y);
-            v[j] = __ldg(&plane[tap_site(tap, y, x, H, W)]);
+            wn[j] = __int_as_float(tap.y);
+            vn[j] = __ldg(&plane[tap_site(tap, y, x, H, W)]);
         }
+    };
+    float acc = 0.f;
+    fetch(q.g.off[k]);
+    for (int t0 = q.g.off[k]; t0 < t1; t0 += 32 * B) {
+        float v[B], w[B];
+#pragma unroll
+        for (int j = 0; j < B; j++) v[j] = vn[j], w[j] = wn[j];
+        if (t0 + 32 * B < t1) fetch(t0 + 32 * B);
 #pragma unroll
         for (int j = 0; j < B; j++) {
             const int n = min(32, t1 - (t0 + 32 * j));
@@ -167,6 +165,78 @@ __device__ __forceinline__ float direct_warp(const SitesParams& q, const float* 
         }
     }
     return acc;
+}
+
+// The direct sums of the lanes that want one (the whole warp calls it).  A sum's
+// additions are one chain, so several sites go side by side, a lane each, 32 taps
+// in flight; up to four take the whole warp each (R = 56, 9648 taps: about 35 us
+// a site against 135 for up to 32).
+__device__ __forceinline__ float direct_sums(const SitesParams& q, const float* A, int k, int y, int x, bool want)
+{
+    const int H = q.e.H, W = q.e.W, lane = threadIdx.x & 31;
+    uint32_t m = __ballot_sync(0xffffffffu, want);
+    float acc = 0.f;
+    if (__popc(m) <= 4) {
+        for (; m; m &= m - 1) {
+            const int L = __ffs(m) - 1;
+            const float s = direct_warp(q, A, k, __shfl_sync(0xffffffffu, y, L), __shfl_sync(0xffffffffu, x, L));
+            if (lane == L) acc = s;
+        }
+        return acc;
+    }
+    const float* plane = A + (size_t)q.e.kt.src[k] * H * W;
+    const int t1 = q.g.off[k + 1];
+    if (q.g.off[k] == t1) return 0.f;
+    int2 next = __ldg(&q.g.taps[min(q.g.off[k] + lane, t1 - 1)]);
+    for (int t0 = q.g.off[k]; t0 < t1; t0 += 32) {
+        const int2 tap = next;
+        next = __ldg(&q.g.taps[min(t0 + 32 + lane, t1 - 1)]);
+        float v[32];
+#pragma unroll
+        for (int j = 0; j < 32; j++) {
+            const int at = __shfl_sync(0xffffffffu, tap.x, j);
+            v[j] = want ? __ldg(&plane[tap_site(make_int2(at, 0), y, x, H, W)]) : 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < 32; j++) {
+            const float w = __int_as_float(__shfl_sync(0xffffffffu, tap.y, j));
+            if (t0 + j < t1) acc = fmaf(w, v[j], acc);
+        }
+    }
+    return acc;
+}
+
+// The warp's marked sites (bit c of a lane's marks: its column c), dealt to the lanes 32
+// at a time: `one(y, x, owner, c, valid)` handles a lane's site, for the whole warp, and
+// its result goes back to the owner's `take(c, result)`.
+template <class One, class Take>
+__device__ __forceinline__ void deal_sites(uint32_t marks, int y, int x, One one, Take take)
+{
+    const int lane = threadIdx.x & 31;
+    uint32_t b[4];
+    int n[5] = {0, 0, 0, 0, 0};
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+        b[c] = __ballot_sync(0xffffffffu, (marks >> c) & 1);
+        n[c + 1] = n[c] + __popc(b[c]);
+    }
+    for (int base = 0; base < n[4]; base += 32) {
+        const int j = base + lane;
+        int c = 0, owner = 0;
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+            if (j >= n[i] && j < n[i + 1]) {
+                c = i;
+                owner = (int)__fns(b[i], 0, j - n[i] + 1);
+            }
+        const float r = one(__shfl_sync(0xffffffffu, y, owner), __shfl_sync(0xffffffffu, x, owner) + c, owner, c, j < n[4]);
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const int rank = n[i] + __popc(b[i] & ((1u << lane) - 1)) - base;
+            const float v = __shfl_sync(0xffffffffu, r, rank & 31);
+            if (((marks >> i) & 1) && rank >= 0 && rank < 32) take(i, v);
+        }
+    }
 }
 
 // (growth bump, alpha test) at one site as the other update kernels compute them from
@@ -186,37 +256,110 @@ __device__ __forceinline__ float2 settled(const SitesParams& q, float u, float m
     return make_float2(gk, q.e.alpha_on ? u : hh * gk);
 }
 
-// sum_k of the alpha tests at one site, settled, for a Delta_sum(U) decision near
-// its threshold.
-__device__ __noinline__ float tests_at(const SitesParams& q, const float* A, const float* P, const float* U, int y, int x)
+__device__ __forceinline__ bool passes(const SitesParams& q, float t) { return t > q.e.eps_u; }
+
+// The range (low, high) that a test t = h g (or u) may lie in: rounding, and the
+// potential's du.  With eta = du / s <= 1/64 the bump's ratio at z + d, |d| <= eta, is
+// exp(-z d - d^2 / 2): off by at most 2 |z| eta + eta^2 (|z| eta <= 5/4; beyond it both
+// bumps are zero).  A narrower bump's range is formed at z -+ eta.
+__device__ __forceinline__ float2 test_range(const SitesParams& q, float u, float t, float az, float sg, float hh)
+{
+    const float du = fminf(q.g.du, fmaf(q.g.slope, fmaxf(u, 0.f), q.g.floor));
+    if (q.e.alpha_on) {
+        const float off = fmaf(1e-7f, fabsf(u), du);
+        return make_float2(t - off, t + off);
+    }
+    const float eta = du * rcp_approx(sg), z2 = az * az;
+    if (sg > 0.f && eta > 1.f / 64.f) {
+        const float z0 = fmaxf(az - eta, 0.f), z1 = az + eta;
+        const float t0 = hh * ex2_approx(-0.721347520444481703680f * (z0 * z0));
+        const float t1 = hh * ex2_approx(-0.721347520444481703680f * (z1 * z1));
+        const float r = fabsf(t0) * fmaf(2e-6f, fminf(z0 * z0, 225.f), 2e-6f);
+        return make_float2(fminf(t0, t1) - r, fmaxf(t0, t1) + r);
+    }
+    float off = fabsf(t) * fmaf(2e-6f, z2, fmaf(eta, fmaf(2.f, az, eta), 2e-6f));
+    // thresholds at zero: where the bump underflows
+    if (q.tiny_eps && sg > 0.f && z2 < 225.f && fabsf(t) < 1e-36f) off = 1e-36f;
+    return make_float2(t - off, t + off);
+}
+
+// Kernel k's diffused genes at one site as the kernel divides them that the shape
+// otherwise takes (the streaming kernel by the hardware reciprocal).
+__device__ __forceinline__ void genes_at(const SitesParams& q, const float* P, int k, int y, int x, float* g)
 {
     const EpiParams& p = q.e;
-    const int H = p.H, W = p.W, K = p.kt.K, RD = p.r_diff;
-    const size_t N = (size_t)H * W;
+    const int H = p.H, W = p.W, RD = p.r_diff;
+    for (int pp = 0; pp < p.n_p; pp++) {
+        const float* pl = P + (size_t)(pp * p.kt.K + k) * H * W;
+        float s = 0.f, n = 0.f;
+        for (int dy = -RD; dy <= RD; dy++)
+            for (int dx = -RD; dx <= RD; dx++) {
+                if (dy * dy + dx * dx > RD * RD) continue;
+                int yy = y + dy, xx = x + dx;
+                yy = yy < 0 ? yy + H : (yy >= H ? yy - H : yy);
+                xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
+                const float v = __ldg(&pl[(size_t)yy * W + xx]);
+                s += v;
+                n += v > p.eps_p ? 1.f : 0.f;
+            }
+        const float r = q.fast ? s * rcp_approx(n) : s / n;
+        g[pp] = n > 0.f ? __saturatef(r) : 0.f;
+    }
+}
+
+// alpha's undecided tests, settled, at the sites of the lanes that want it: kernel
+// `first`'s, and the later kernels' where it was not the only one (the whole warp calls it).
+__device__ __forceinline__ bool alpha_at(const SitesParams& q, const float* A, const float* P, const float* U, int y, int x,
+                                         bool want, int first, bool more)
+{
+    const EpiParams& p = q.e;
+    const int W = p.W, K = p.kt.K;
+    const size_t N = (size_t)p.H * W;
+    bool ok = want;
+    int k = first;                             // (a lane's own; K: done)
+    while (__any_sync(0xffffffffu, ok && k < K)) {
+        // the lanes at the warp's lowest kernel go on
+        const int kk = __reduce_min_sync(0xffffffffu, ok && k < K ? k : K);
+        const bool on = ok && k == kk;
+        float g[3] = {0.f, 0.f, 0.f};
+        if (on) genes_at(q, P, kk, y, x, g);
+        const float m = p.p_mu >= 0 ? g[p.p_mu] : p.kt.mu[kk];
+        const float sg = p.p_sigma >= 0 ? g[p.p_sigma] : p.kt.sigma[kk];
+        const float hh = p.p_h >= 0 ? g[p.p_h] : p.kt.h[kk];
+        float u = on ? __ldg(&U[(size_t)kk * N + (size_t)y * W + x]) : 0.f;
+        float t = settled(q, u, m, sg, hh).y;
+        const float2 r = test_range(q, u, t, fabsf((u - m) * rcp_approx(sg)), sg, hh);
+        const bool open = on && r.x < p.eps_u && p.eps_u < r.y;
+        if (q.g.du > 0.f && __any_sync(0xffffffffu, open)) {
+            u = direct_sums(q, A, kk, y, x, open);
+            if (open) t = settled(q, u, m, sg, hh).y;
+        }
+        if (on) {
+            ok = passes(q, t);
+            k = more ? kk + 1 : K;
+        }
+    }
+    return ok;
+}
+
+// sum_k of the alpha tests, settled, at the sites of the lanes that want it (a
+// Delta_sum(U) decision near its threshold; the whole warp calls it).
+__device__ __forceinline__ float tests_at(const SitesParams& q, const float* A, const float* P, const float* U, int y, int x,
+                                       bool want)
+{
+    const EpiParams& p = q.e;
+    const int W = p.W, K = p.kt.K;
+    const size_t N = (size_t)p.H * W;
     float sum = 0.f;
     for (int k = 0; k < K; k++) {
         float g[3] = {0.f, 0.f, 0.f};
-        for (int pp = 0; pp < p.n_p; pp++) {
-            const float* pl = P + (size_t)(pp * K + k) * N;
-            float s = 0.f, n = 0.f;
-            for (int dy = -RD; dy <= RD; dy++)
-                for (int dx = -RD; dx <= RD; dx++) {
-                    if (dy * dy + dx * dx > RD * RD) continue;
-                    int yy = y + dy, xx = x + dx;
-                    yy = yy < 0 ? yy + H : (yy >= H ? yy - H : yy);
-                    xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
-                    const float v = __ldg(&pl[(size_t)yy * W + xx]);
-                    s += v;
-                    n += v > p.eps_p ? 1.f : 0.f;
-                }
-            const float r = q.fast ? s * rcp_approx(n) : s / n;
-            g[pp] = n > 0.f ? __saturatef(r) : 0.f;
-        }
+        if (want) genes_at(q, P, k, y, x, g);
         const float m = p.p_mu >= 0 ? g[p.p_mu] : p.kt.mu[k];
         const float sg = p.p_sigma >= 0 ? g[p.p_sigma] : p.kt.sigma[k];
         const float hh = p.p_h >= 0 ? g[p.p_h] : p.kt.h[k];
-        const float u = q.g.du > 0.f ? direct_at(q, A, k, y, x) : __ldg(&U[(size_t)k * N + (size_t)y * W + x]);
-        sum += settled(q, u, m, sg, hh).y;
+        const float u = q.g.du > 0.f ? direct_sums(q, A, k, y, x, want && (sg > 0.f || p.alpha_on))
+                                     : (want ? __ldg(&U[(size_t)k * N + (size_t)y * W + x]) : 0.f);
+        if (want) sum += settled(q, u, m, sg, hh).y;
     }
     return sum;
 }
@@ -337,6 +480,7 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
             bool al[4] = {in, in, in, in};
             float tsum[4] = {0.f, 0.f, 0.f, 0.f}, tband[4] = {0.f, 0.f, 0.f, 0.f};
             bool wrote = false;                     // a non-zero gene went out already
+            uint32_t undecided = 0, many = 0, first = 0;    // sites with tests to be settled; with several; their first kernels
             int k = 0;
             const bool warp_live = __any_sync(0xffffffffu, live);
             if (NP > 0 && !warp_live) al[0] = al[1] = al[2] = al[3] = false;
@@ -356,7 +500,7 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                     auto mu_of = [&](int c) { return PMU >= 0 ? ph[PMU >= 0 ? PMU : 0][c] : km; };
                     auto sg_of = [&](int c) { return PSG >= 0 ? ph[PSG >= 0 ? PSG : 0][c] : ks; };
                     auto h_of = [&](int c) { return PH >= 0 ? ph[PH >= 0 ? PH : 0][c] : kh; };
-                    uint32_t near = 0;              // sites whose test is to be settled
+                    bool pass[4] = {false, false, false, false};    // undecided tests pass for now
                     Pre cur[NQ];
 #pragma unroll
                     for (int pp = 0; pp < NP; pp++) cur[pp] = nx[pp];
@@ -384,53 +528,16 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                             gk[c] = sg > 0.f ? e : 0.f;
                             tk[c] = p.alpha_on ? u[c] : h_of(c) * gk[c];
                             if (NP > 0) {
-                                // the test's range: rounding, and the potential's du.  With eta = du / s
-                                // <= 1/64 the bump's ratio at z + d, |d| <= eta, is exp(-z d - d^2 / 2):
-                                // off by at most 2 |z| eta + eta^2 (|z| eta <= 5/4; beyond it both
-                                // bumps are zero).  A narrower bump's range is formed at z -+ eta.
-                                const float eta = q.g.du * rs, az = fabsf(z);
-                                float lo, hi;
-                                if (p.alpha_on) {
-                                    const float off = fmaf(1e-7f, fabsf(u[c]), q.g.du);
-                                    lo = tk[c] - off;
-                                    hi = tk[c] + off;
-                                } else if (sg > 0.f && eta > 1.f / 64.f) {
-                                    const float hh = h_of(c), z0 = fmaxf(az - eta, 0.f), z1 = az + eta;
-                                    const float t0 = hh * ex2_approx(-0.721347520444481703680f * (z0 * z0));
-                                    const float t1 = hh * ex2_approx(-0.721347520444481703680f * (z1 * z1));
-                                    const float r = fabsf(t0) * fmaf(2e-6f, fminf(z0 * z0, 225.f), 2e-6f);
-                                    lo = fminf(t0, t1) - r;
-                                    hi = fmaxf(t0, t1) + r;
-                                } else {
-                                    float off = fabsf(tk[c]) * fmaf(2e-6f, z2, fmaf(eta, fmaf(2.f, az, eta), 2e-6f));
-                                    // thresholds at zero: where the bump underflows
-                                    if (q.tiny_eps && sg > 0.f && z2 < 225.f && fabsf(tk[c]) < 1e-36f) off = 1e-36f;
-                                    lo = tk[c] - off;
-                                    hi = tk[c] + off;
+                                const float2 r = test_range(q, u[c], tk[c], fabsf(z), sg, h_of(c));
+                                if (p.empty_out) tband[c] += fmaxf(r.y - tk[c], tk[c] - r.x);
+                                // (an exact test's range is one value)
+                                const bool open = (r.x < eps_u) & (eps_u < r.y);
+                                if (al[c] & open) {
+                                    many |= undecided & (1u << c);
+                                    if (!((undecided >> c) & 1)) first |= (uint32_t)k << (8 * c);
+                                    undecided |= 1u << c;
+                                    pass[c] = true;
                                 }
-                                if (p.empty_out) tband[c] += hi - lo;
-                                near |= (al[c] & (lo < eps_u) & (eps_u < hi) ? 1u : 0u) << c;   // (lo = hi: exact)
-                            }
-                        }
-                    }
-                    if (NP > 0) {
-                        // one site after the other, the warp summing its potential together
-                        for (uint32_t nm = __ballot_sync(0xffffffffu, near != 0); nm;
-                             nm = __ballot_sync(0xffffffffu, near != 0)) {
-                            const int L = __ffs(nm) - 1;
-                            const int i = __ffs(__shfl_sync(0xffffffffu, near, L)) - 1;
-                            const int ys = __shfl_sync(0xffffffffu, y, L), xs = __shfl_sync(0xffffffffu, x, L) + i;
-                            float ud = 0.f;
-                            if (q.g.du > 0.f) ud = direct_warp(q, pA, k, ys, xs);
-                            if (lane == L) {
-#pragma unroll
-                                for (int c = 0; c < 4; c++)
-                                    if (c == i) {
-                                        const float2 r = settled(q, q.g.du > 0.f ? ud : u[c], mu_of(c), sg_of(c), h_of(c));
-                                        gk[c] = r.x;
-                                        tk[c] = r.y;
-                                    }
-                                near &= near - 1;
                             }
                         }
                     }
@@ -438,7 +545,7 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                     if (want) {
 #pragma unroll
                         for (int c = 0; c < 4; c++) {
-                            if (NP > 0) al[c] = al[c] & (tk[c] > eps_u);
+                            if (NP > 0) al[c] = al[c] & (pass[c] | passes(q, tk[c]));
                             tsum[c] += tk[c];
                             G[c] = p.growth_form == 0 ? fmaf(2.f * gk[c], h_of(c), -h_of(c)) : h_of(c) * gk[c];
                         }
@@ -468,6 +575,23 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                             break;
                         }
                     }
+                }
+            }
+            if (NP > 0) {
+                // sites that hang on undecided tests
+                const uint32_t open = undecided & (al[0] | (al[1] << 1) | (al[2] << 2) | (al[3] << 3));
+                if (__any_sync(0xffffffffu, open != 0)) {
+                    uint32_t lost = 0;
+                    deal_sites(
+                        open, y, x,
+                        [&](int ys, int xs, int owner, int c, bool valid) {
+                            const int k0 = (__shfl_sync(0xffffffffu, first, owner) >> (8 * c)) & 255;
+                            const bool more = (__shfl_sync(0xffffffffu, many, owner) >> c) & 1;
+                            return alpha_at(q, pA, pP, pU, ys, xs, valid, k0, more) ? 1.f : 0.f;
+                        },
+                        [&](int c, float ok) { lost |= (ok == 0.f ? 1u : 0u) << c; });
+#pragma unroll
+                    for (int c = 0; c < 4; c++) al[c] = al[c] & !((lost >> c) & 1);
                 }
             }
             if (NP > 0 && in) {
@@ -514,11 +638,21 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                 *reinterpret_cast<uchar4*>(p.alpha_out + i0) =
                     NP == 0 ? make_uchar4(1, 1, 1, 1) : make_uchar4(al[0], al[1], al[2], al[3]);
             // (no band: every test is exactly the direct route's, and so is their sum)
-            if (NP > 0 && in && p.empty_out)
+            if (NP > 0 && p.empty_out) {
+                uint32_t close = 0;
 #pragma unroll
                 for (int c = 0; c < 4; c++)
-                    if (tband[c] > 0.f && fabsf(tsum[c] - eps_u) <= tband[c] + 1e-6f)
-                        tsum[c] = tests_at(q, pA, pP, pU, y, x + c);
+                    close |= (in && tband[c] > 0.f && fabsf(tsum[c] - eps_u) <= tband[c] + 1e-6f ? 1u : 0u) << c;
+                if (__any_sync(0xffffffffu, close != 0))
+                    deal_sites(
+                        close, y, x,
+                        [&](int ys, int xs, int, int, bool valid) { return tests_at(q, pA, pP, pU, ys, xs, valid); },
+                        [&](int c, float t) {
+#pragma unroll
+                            for (int i = 0; i < 4; i++)
+                                if (c == i) tsum[i] = t;
+                        });
+            }
             if (in && p.empty_out)
                 *reinterpret_cast<uchar4*>(p.empty_out + i0) =
                     make_uchar4(!(tsum[0] > eps_u), !(tsum[1] > eps_u), !(tsum[2] > eps_u), !(tsum[3] > eps_u));

@@ -58,7 +58,7 @@ struct lenia_ctx {
     TileParams tl;
     bool block = false;                    // rollouts in one block (the torus is one window)
     bool gate_pays = false;                // more windows than run at once: skipping some saves time
-    float guard_du = 0.f;                  // how far the windows' and the direct sums' potentials may be apart
+    GuardParams guard = {};                // how far the windows' and the direct sums' potentials may be apart
     float* d_tS = nullptr;
     float* d_tS0 = nullptr;
     float2* d_ttw = nullptr;
@@ -385,28 +385,41 @@ std::vector<float2> twiddles(int n, int count)
     return t;
 }
 
-// How far the windows' and the direct sums' potentials may be apart, for states of
-// magnitude at most 1.  The direct route adds a kernel's n taps one after the
-// other, each addition off by at most 2^-24 of the partial sum, so tap i's weight
-// is rounded n - i times: the bound grows with the taps (1.5e-5 at R = 13, 3.7e-5
-// at R = 20, 2.9e-4 at R = 56; uniform states reach 6e-6 there).  The windows stay
-// below 2.5e-7 of the absolute weights' sum (measured); four times that is allowed.
-float window_guard(const lenia_ctx* c)
+// How far the windows' and the direct sums' potentials may be apart, for states in
+// [0, 1].  The direct route adds a kernel's n taps one after the other, each
+// addition off by at most 2^-24 of the partial sum, so tap i's weight is rounded
+// n - i times: the bound grows with the taps (1.5e-5 at R = 13, 3.7e-5 at R = 20,
+// 2.9e-4 at R = 56, of which a uniform state on a flat disk reaches half).  Where no
+// weight is negative a partial sum is at most the potential itself, and n 2^-24 of
+// it the bound.  The windows stay below 2.5e-7 of the absolute weights' sum
+// (measured); four times that is allowed.
+GuardParams window_guard(const lenia_ctx* c)
 {
-    double most = 0.0;
+    GuardParams g;
+    memset(&g, 0, sizeof(g));
+    bool negative = false;
+    double du = 0.0, floor = 0.0, slope = 0.0;
     for (size_t k = 0; k < c->conv_w.size(); k++) {
-        const int R = c->conv_R[k], n = 2 * R + 1;
-        double passed = 0.0, total = 0.0;      // sum_i |w_i| (n - i): every prefix sum once
+        double passed = 0.0, total = 0.0, taps = 0.0;      // passed: sum_i |w_i| (n - i), every prefix sum once
+        const int n = 2 * c->conv_R[k] + 1;
         for (int dx = 0; dx < n; dx++)
             for (int dy = 0; dy < n; dy++) {
-                const double w = fabs((double)(float)c->conv_w[k][(size_t)dy * n + dx]);
+                const double w = (double)(float)c->conv_w[k][(size_t)dy * n + dx];
                 if (w == 0.0) continue;
-                total += w;
+                negative = negative || w < 0.0;
+                total += fabs(w);
                 passed += total;
+                taps += 1.0;
             }
-        most = std::max(most, passed * 5.9604644775390625e-8 + 1e-6 * total);
+        const double u = 5.9604644775390625e-8;            // 2^-24
+        slope = std::max(slope, u * taps);
+        floor = std::max(floor, 1e-6 * total * (1.0 + u * taps));
+        du = std::max(du, u * passed + 1e-6 * total);
     }
-    return (float)(1.001 * most);
+    g.du = (float)(1.001 * du);
+    g.slope = negative ? 0.f : (float)(1.001 * slope);
+    g.floor = negative ? g.du : (float)(1.001 * floor);
+    return g;
 }
 
 // Spectra and twiddles of the context's windows (c->tl.N).  Waits for the work.
@@ -612,13 +625,7 @@ lenia_status step_impl(lenia_ctx* c, const float* A_in, const float* P_in, float
         if (sites) {
             // the arithmetic of the kernel that the shape otherwise takes
             const bool fast = epilogue_rows_supported(ep) && !quads11;
-            GuardParams g;
-            if (settle) {
-                g.taps = c->d_taps;
-                for (int k = 0; k <= c->cfg.n_kernels; k++) g.off[k] = c->tap_off[k];
-                g.du = c->guard_du;
-            }
-            CUDA_OR_FAIL(c, launch_epilogue_sites(ep, fast, settle ? &g : nullptr, 1, kSitesBlocksPerSm * c->num_sms, s, &nb));
+            CUDA_OR_FAIL(c, launch_epilogue_sites(ep, fast, settle ? &c->guard : nullptr, 1, kSitesBlocksPerSm * c->num_sms, s, &nb));
         } else if (quads11 && aligned && aligned_out) {
             CUDA_OR_FAIL(c, launch_epilogue_batch(ep, 1, s, -1));
         } else if (aligned && epilogue_rows_supported(ep)) {
@@ -962,11 +969,11 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
     // them), keeps the sums throughout, and so do ring worlds and an explicit
     // LENIA_CONV_DIRECT.
     const bool want_adj = cfg->max_rollout_steps > 0 && c->n_p == 0 && !cfg->maintain_genes;
-    c->guard_du = window_guard(c);
+    c->guard = window_guard(c);
     if ((path == LENIA_CONV_FFT && !cfg->maintain_genes) ||
         (path == LENIA_CONV_DIRECT && cfg->conv_path == LENIA_CONV_AUTO && !n_rings &&
          (!cfg->maintain_genes || (epilogue_sites_supported(epi_params(c)) &&
-                                   !(cfg->alpha_on && fabsf(cfg->eps_u) < std::max(1e-4f, 2.f * K * c->guard_du)))))) {
+                                   !(cfg->alpha_on && fabsf(cfg->eps_u) < std::max(1e-4f, 2.f * K * c->guard.du)))))) {
         memset(&c->tl, 0, sizeof(c->tl));
         const double t_tile = tile_choose(&c->tl, H, W, kcount, c->max_R, 1, cfg->maintain_genes != 0);
         const double t_else = path == LENIA_CONV_FFT ? fft_passes_cost(H, W, C + NC) : direct_cost(H, W, NC, c->max_R);
@@ -1033,6 +1040,10 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
         if (c->small || settles) {
             ALLOC(c->d_taps, taps.size());
             CK_INIT(cudaMemcpy(c->d_taps, taps.data(), taps.size() * sizeof(int2), cudaMemcpyHostToDevice));
+        }
+        if (settles) {
+            c->guard.taps = c->d_taps;
+            for (int k = 0; k <= K; k++) c->guard.off[k] = c->tap_off[k];
         }
         if (c->small) ALLOC(c->d_small_count, 1);
     }

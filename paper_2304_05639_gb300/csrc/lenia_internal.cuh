@@ -416,6 +416,7 @@ struct GuardParams {
     const int2* taps;          // as SmallRolloutParams, kernel k's at off[k] .. off[k + 1] - 1
     int off[kMaxKernels + 1];
     float du;                  // 0: the potentials are the direct sums already
+    float slope, floor;        // at a potential u: the smaller of du and slope u + floor
 };
 // fast: the streaming kernel's reciprocals and exponential, else divisions and expf
 cudaError_t launch_epilogue_sites(const EpiParams& p, bool fast, const GuardParams* guard, int n_worlds, int max_blocks,
