@@ -41,8 +41,10 @@ def test_gradient_of_channels_that_no_kernel_reads(shape, topology):
     H, W, R = shape
     C = max(max(t) for t in topology) + 1
     ks = [inputs.KernelDesc(s, d, R, inputs.KERNEL_SHELLS, (1.0,), h=0.7, mu=0.5, sigma=0.08) for s, d in topology]
-    w = inputs.World(H, W, C, ks, 0.1, localized=0, maintain_genes=0)
-    w.A = inputs.random_field(H + W, (C, H, W))
+    # (three updates of at most 0.02 x 0.7 x 3: no site comes near a clip, whose two
+    # sides differ by a whole gradient)
+    w = inputs.World(H, W, C, ks, 0.02, localized=0, maintain_genes=0)
+    w.A = (0.3 + 0.4 * inputs.random_field(H + W, (C, H, W))).astype(np.float32)
     (a, ga), (b, gb) = (_gradients(w, 3, p) for p in (lenia.CONV_AUTO, lenia.CONV_DIRECT))
     for c in range(C):
         assert float((a[c] - b[c]).norm()) <= 1e-4 * float(b[c].norm())
