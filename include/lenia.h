@@ -74,7 +74,8 @@ enum { LENIA_LOC_MU = 1, LENIA_LOC_SIGMA = 2, LENIA_LOC_H = 4, LENIA_LOC_KERNEL 
  * direct worlds convolve in overlapping 64 x 64 or 128 x 128 windows of
  * spectral transforms instead (lenia_conv_path still reports DIRECT; alpha and
  * Delta_sum decisions that the rounding could turn are settled by the direct
- * sums at those sites, values of A outside [0, 1] excepted), and so do FFT
+ * sums at those sites, and a window that holds a value of A outside [0, 1] is
+ * summed directly, so that the value reaches no further than R), and so do FFT
  * worlds without gene maintenance; an explicit LENIA_CONV_DIRECT always
  * sums.  DIRECT_BF16 and DIRECT_BF16X3 run the direct
  * convolution on the tensor cores as banded Toeplitz products (tcgen05,

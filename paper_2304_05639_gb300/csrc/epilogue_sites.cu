@@ -256,7 +256,11 @@ __device__ __forceinline__ float2 settled(const SitesParams& q, float u, float m
     return make_float2(gk, q.e.alpha_on ? u : hh * gk);
 }
 
-__device__ __forceinline__ bool passes(const SitesParams& q, float t) { return t > q.e.eps_u; }
+// (the streaming kernel's minimum of the tests passes NaN over, the others' do not)
+__device__ __forceinline__ bool passes(const SitesParams& q, float t)
+{
+    return q.fast ? !(t <= q.e.eps_u) : t > q.e.eps_u;
+}
 
 // The range (low, high) that a test t = h g (or u) may lie in: rounding, and the
 // potential's du.  With eta = du / s <= 1/64 the bump's ratio at z + d, |d| <= eta, is

@@ -658,6 +658,8 @@ lenia_status transposed_conv(lenia_ctx* c, const float* gU, float* V, cudaStream
     const int K = c->cfg.n_kernels;
     if (c->adj_form != lenia_ctx::ADJ_PASSES) {
         TileParams tl = c->tl;
+        tl.centre = 0.f;
+        tl.reach = 1e30f;
         tl.A = gU;
         if (c->adj_form == lenia_ctx::ADJ_PLANES) {
             tl.U = V;
@@ -1093,6 +1095,16 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
         CK_INIT(cudaMemcpy(c->d_yr, yr.data(), yr.size() * sizeof(int), cudaMemcpyHostToDevice));
         CK_INIT(cudaMemcpy(c->d_yr_off, yroff.data(), NC * sizeof(int), cudaMemcpyHostToDevice));
         memset(&c->cp, 0, sizeof(c->cp));
+        // windows: states that cannot be summed in the frequency domain without reaching
+        // further than R
+        if (c->tile) {
+            c->tl.dw = c->d_w;
+            c->tl.dw_off = c->d_w_off;
+            c->tl.yr = c->d_yr;
+            c->tl.yr_off = c->d_yr_off;
+            c->tl.centre = c->tl.reach = 0.5f;
+            for (int k = 0; k < K; k++) c->tl.dR[k] = c->conv_R[k];
+        }
         c->cp.w = c->d_w;
         c->cp.w_off = c->d_w_off;
         c->cp.yr = c->d_yr;

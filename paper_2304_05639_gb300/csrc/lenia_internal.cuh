@@ -300,6 +300,15 @@ struct TileParams {
     const float* gate;
     float gate_eps;
     int gate_r;
+    // A window holding a value further than `reach` from `centre` is summed directly, so
+    // that no value reaches further than R: states outside [0, 1], gradients above
+    // 1e30 (the dense kernels of ConvParams, or null: no limit)
+    float centre, reach;
+    const float* dw;
+    const int* dw_off;
+    const int* yr;
+    const int* yr_off;
+    int dR[kMaxKernels];
     int kpb;                   // kernels per block
     int per_plane;             // K planes of A, plane k convolved with kernel k (C = K)
     int vec2, vec2o;           // input / output 8-byte aligned (set by the launcher)

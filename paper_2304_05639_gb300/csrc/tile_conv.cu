@@ -243,6 +243,14 @@ __device__ __forceinline__ void cols8(unsigned char* buf, int n1, int c)
     for (int q = 0; q < 8; q++) st2(buf, ((q & 1) ? o1 : o0) + q * CA * TC<N>::PITCH, v[q]);
 }
 
+// The largest magnitude of three, NaN if one is NaN.
+__device__ __forceinline__ float max_abs(float a, float b, float c)
+{
+    float d;
+    asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
 __device__ __forceinline__ int wrap_any(int i, int n)
 {
     i %= n;
@@ -255,9 +263,10 @@ struct Window {                     // the tile of a block
     int c, lane, warp;
 };
 
-// Forward transform of one plane's window up to the last column pass.
+// Forward transform of one plane's window up to the last column pass; stops and
+// returns true if the window holds a value beyond the limit.
 template <int N, int NT>
-__device__ __forceinline__ void forward_start(const TileParams& p, const float* plane, const Window& w,
+__device__ __forceinline__ bool forward_start(const TileParams& p, const float* plane, const Window& w,
                                               unsigned char* buf)
 {
     using X = TC<N, NT>;
@@ -265,6 +274,7 @@ __device__ __forceinline__ void forward_start(const TileParams& p, const float* 
     const bool inside = w.x0 >= w.g.halo_x && w.x0 - w.g.halo_x + N <= p.W && w.y0 >= w.g.halo_y &&
                         w.y0 - w.g.halo_y + N <= p.H;
     const int m1 = lane % X::RR;
+    float largest = 0.f;
     {
         // rows: radix 8 over m2 of the pairs m1 + RR m2, straight from global
         // memory; window index i stands for site x0 + i, or x0 + i - N beyond the cut
@@ -290,13 +300,16 @@ __device__ __forceinline__ void forward_start(const TileParams& p, const float* 
 #pragma unroll
                 for (int m2 = 0; m2 < 8; m2++) v[m2] = make_float2(__ldg(row + gx[m2]), __ldg(row + gx[m2] + 1));
             }
+#pragma unroll
+            for (int m2 = 0; m2 < 8; m2++)
+                largest = max_abs(largest, v[m2].x - p.centre, v[m2].y - p.centre);
             DFT<8, false, true>::run(v);
             const int base = y * X::PITCH + ((m1 * 8 + (m1 & 7)) ^ row_sw(y)) * 8;
 #pragma unroll
             for (int j = 0; j < 8; j++) st2(buf, base ^ (j * 8), v[j]);
         }
     }
-    __syncthreads();
+    if (__syncthreads_or(p.dw && !(largest <= p.reach))) return true;
     // rows: radix RR over m1 and the real split; warp-uniform t
 #pragma unroll 1
     for (int u = warp; u < 4 * (N / 32); u += X::NW) {
@@ -313,6 +326,48 @@ __device__ __forceinline__ void forward_start(const TileParams& p, const float* 
 #pragma unroll 1
     for (int u = warp; u < X::CA * X::CH; u += X::NW) cols8<N, false>(buf, u % X::CA, (u / X::CA) * 32 + lane);
     __syncthreads();
+    return false;
+}
+
+// Kernel k's direct sum over the plane at (y, x), in k_direct_conv's order.
+__device__ __forceinline__ float window_sum(const TileParams& p, const float* plane, int k, int y, int x)
+{
+    const int R = p.dR[k];
+    const float* w = p.dw + p.dw_off[k];       // [dx + R][dy + R]
+    const int* yr = p.yr + p.yr_off[k];
+    float acc = 0.f;
+#pragma unroll 1
+    for (int dx = -R; dx <= R; dx++) {
+        const int r = __ldg(&yr[dx + R]);
+        const float* wc = w + (dx + R) * (2 * R + 1) + R;
+        const float* col = plane + wrap_any(x + dx, p.W);
+#pragma unroll 1
+        for (int dy = -r; dy <= r; dy++) acc = fmaf(__ldg(&wc[dy]), __ldg(col + (size_t)wrap_any(y + dy, p.H) * p.W), acc);
+    }
+    return acc;
+}
+
+// The output tile by direct sums, for a window that holds a value beyond the limit.
+// (Inline: as a call it cost the 64^2 windows' passes spills, 2048^2 with R = 5
+// 340 against 330 us a step.)
+// Kernels t0 .. t1 - 1 of channel c; ADJ: their sum added to the channel's plane.
+template <bool ADJ>
+__device__ __forceinline__ void window_direct(const TileParams& p, int c, int t0, int t1, int x0, int y0, int rows, int xend)
+{
+    const size_t HW = (size_t)p.H * p.W;
+#pragma unroll 1
+    for (int i = threadIdx.x; i < rows * xend; i += blockDim.x) {
+        const int y = y0 + i / xend, x = x0 + i % xend;
+        const size_t o = (size_t)y * p.W + x;
+        float sum = 0.f;
+        for (int t = t0; t < t1; t++) {
+            const int k = p.per_plane ? c : p.klist[c][t];
+            const float u = window_sum(p, p.A + (ADJ ? k : c) * HW, k, y, x);
+            if (ADJ) sum += u;
+            else p.U[k * HW + o] = u;
+        }
+        if (ADJ) p.U[c * HW + o] = p.add ? __ldg(p.add + c * HW + o) + sum : sum;
+    }
 }
 
 // Last forward column pass of (column c, residue b): twiddle w_N^(n1 b), radix CA over
@@ -340,13 +395,14 @@ __device__ __forceinline__ void cols_inv(unsigned char* buf, const float2* twc, 
         st2(buf, at<N>(n1 + X::CA * b, c), n1 ? cmulc(v[n1], twc[b * X::CA + n1]) : v[n1]);
 }
 
-// Forward transform; task i's CA spectrum values go to `sink(i, c, b, v)`.
+// Forward transform; task i's CA spectrum values go to `sink(i, c, b, v)`.  Returns
+// false, without having called it, if the window holds a value beyond the limit.
 template <int N, int NT, int UNR, class Sink>
-__device__ __forceinline__ void forward(const TileParams& p, const float* plane, const Window& w, unsigned char* buf,
+__device__ __forceinline__ bool forward(const TileParams& p, const float* plane, const Window& w, unsigned char* buf,
                                         const float2* twc, Sink sink)
 {
     using X = TC<N, NT>;
-    forward_start<N, NT>(p, plane, w, buf);
+    if (forward_start<N, NT>(p, plane, w, buf)) return false;
     constexpr int TASKS = 8 * X::CH / X::NW;             // per warp
 #pragma unroll UNR
     for (int i = 0; i < TASKS; i++) {
@@ -356,6 +412,7 @@ __device__ __forceinline__ void forward(const TileParams& p, const float* plane,
         cols_fwd<N>(buf, twc, c, b, v);
         sink(i, c, b, v);
     }
+    return true;
 }
 
 // Inverse transform after its first column pass; the real rows go to
@@ -563,7 +620,8 @@ k_tile_conv(const __grid_constant__ TileParams p)
     };
     const size_t SP = (size_t)N * X::M;                                      // floats of one kernel spectrum
     if constexpr (!ADJ) {
-        forward<N, NT, UNR>(p, gA + (size_t)w.c * HW, w, buf, twc, [&](int i, int c, int b, float2* v) {
+        const float* plane = gA + (size_t)w.c * HW;
+        const bool usual = forward<N, NT, UNR>(p, plane, w, buf, twc, [&](int i, int c, int b, float2* v) {
             tput(i, v);
             if (c == 0)
 #pragma unroll
@@ -571,6 +629,8 @@ k_tile_conv(const __grid_constant__ TileParams p)
         });
         tmem_wait_st();
         __syncthreads();
+        if (!usual) window_direct<false>(p, w.c, t0, t1, w.x0, w.y0, rows, xend);
+        else
         for (int t = t0; t < t1; t++) {
             const int k = p.per_plane ? w.c : p.klist[w.c][t];
             float* U = gU + (size_t)k * HW;
@@ -593,9 +653,10 @@ k_tile_conv(const __grid_constant__ TileParams p)
             __syncthreads();
         }
     } else {
-        for (int t = 0; t < nk; t++) {
+        bool usual = true;
+        for (int t = 0; usual && t < nk; t++) {
             const int k = p.klist[w.c][t];
-            forward<N, NT, UNR>(p, gA + (size_t)k * HW, w, buf, twc, [&](int i, int c, int b, float2* v) {
+            usual = forward<N, NT, UNR>(p, gA + (size_t)k * HW, w, buf, twc, [&](int i, int c, int b, float2* v) {
                 if (c == 0) {
                     // mirrored share of the packed column, at -ky (this thread's slots only)
                     const float* s2 = gS0 + (size_t)k * N;
@@ -622,6 +683,8 @@ k_tile_conv(const __grid_constant__ TileParams p)
         }
         float* O = gU + (size_t)w.c * HW;
         const float* add = p.add ? p.add + (size_t)w.c * HW : nullptr;
+        if (!usual) window_direct<true>(p, w.c, 0, nk, w.x0, w.y0, rows, xend);
+        else
         inverse<N, NT, UNR>(
             w, rows, buf, twc,
             [&](int i, int c, int b, float2* v) {

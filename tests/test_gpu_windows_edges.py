@@ -201,3 +201,71 @@ def test_diffused_genes_saturate(localized, r_diff, value):
     g = oracle.diffuse(w.P[1, 2], r_diff)
     assert g[y, x] == 1.0 and alpha[_near(72, 100, y, x, r_diff + 1e-3)].any()
     np.testing.assert_allclose(P2[1, 2].cpu().numpy()[alpha], g[alpha], atol=4e-7)
+
+
+BAD = [np.nan, np.inf, -np.inf, 3e38, 1e4, -2.0]
+
+
+@pytest.mark.parametrize("bad", BAD)
+@pytest.mark.parametrize("shape", [(300, 404, 12), (90, 100, 9), (61, 132, 6)])
+def test_values_outside_the_unit_interval_stay_within_the_radius(shape, bad):
+    """A value the state cannot hold reaches the potentials within R of it and no others,
+    and there gives what the direct sums give."""
+    H, W, R = shape
+    w = inputs.single_kernel_global(H=H, W=W, R=R, patch=min(H, W) // 2)
+    A = inputs.random_field(5, w.A.shape)
+    clean = gpu_potentials(w, lenia.CONV_DIRECT, A)[0]
+    A[0, H // 3, W // 2] = bad
+    t, d = (gpu_potentials(w, p, A)[0] for p in (lenia.CONV_AUTO, lenia.CONV_DIRECT))
+    far = ~_near(H, W, H // 3, W // 2, R)
+    assert np.abs(t[0] - clean[0])[far].max() <= TOL_U
+    np.testing.assert_array_equal(np.isfinite(t), np.isfinite(d))
+    with np.errstate(invalid="ignore"):
+        np.testing.assert_allclose(t, d, rtol=1e-5, atol=TOL_U)
+
+
+@pytest.mark.parametrize("bad", BAD)
+@pytest.mark.parametrize("kw", [dict(H=130, W=92, R=13, n_channels=3), dict(H=130, W=256, R=13, n_channels=3),
+                                dict(H=105, W=100, R=9, n_channels=1)])
+def test_steps_from_states_outside_the_unit_interval_equal_direct(kw, bad):
+    torch = torch_mod()
+    w = inputs.multi_channel(patch=40, n_geno=4, matched=True, seed_index=31, **kw)
+    ys, xs = np.nonzero(w.P[0, 0] != 0)
+    w.A[0, ys[len(ys) // 2], xs[len(xs) // 2]] = bad
+    out = []
+    for path in (lenia.CONV_AUTO, lenia.CONV_DIRECT):
+        cfg, ks = lenia.config_from_world(w, path)
+        ctx = lenia.lenia_init(cfg, ks)
+        A, P = to_dev(w.A), to_dev(w.P)
+        A2, P2 = torch.empty_like(A), torch.empty_like(P)
+        lenia.lenia_step(ctx, A, P, A2, P2)
+        torch.cuda.synchronize()
+        out.append((A2.cpu().numpy(), P2.cpu().numpy()))
+        lenia.lenia_destroy(ctx)
+    np.testing.assert_array_equal(out[0][1] != 0, out[1][1] != 0)
+    assert np.abs(out[0][0] - out[1][0]).max() <= 1e-5
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, 1e38])
+@pytest.mark.parametrize("shape", [(130, 140, 13, 1), (100, 72, 9, 3), (48, 60, 13, 3)])
+def test_gradients_outside_the_usual_range_stay_within_the_radius(shape, bad):
+    """One reversed step: the carried gradient's one bad site reaches dL/dA_0 within R."""
+    torch = torch_mod()
+    H, W, R, C = shape
+    ks = [inputs.KernelDesc(s, d, R, inputs.KERNEL_SHELLS, (1.0,), h=0.7, mu=0.5, sigma=0.08)
+          for s, d in inputs.paper_topology(C)]
+    w = inputs.World(H, W, C, ks, 0.01, localized=0, maintain_genes=0)
+    A0 = (0.3 + 0.4 * inputs.random_field(7, (C, H, W))).astype(np.float32)
+    out = []
+    for path in (lenia.CONV_AUTO, lenia.CONV_DIRECT):
+        f = lenia.LeniaRollout(w, 1, conv_path=path)
+        A = to_dev(A0).requires_grad_(True)
+        genes = torch.from_numpy(lenia.genes_of(w)).cuda()
+        g = torch.ones(A0.shape, device="cuda")
+        g[0, H // 2, W // 2] = bad
+        f(A, genes).backward(g)
+        out.append(A.grad.cpu().numpy())
+        f.close()
+    np.testing.assert_array_equal(np.isfinite(out[0]), np.isfinite(out[1]))
+    far = ~_near(H, W, H // 2, W // 2, R)
+    assert np.abs(out[0] - out[1])[:, far].max() <= 1e-5
