@@ -379,15 +379,16 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
     constexpr int PSG = (LOC & 2) ? ((LOC & 1) ? 1 : 0) : -1;
     constexpr int PH = (LOC & 4) ? NP - 1 : -1;
     const EpiParams& p = q.e;
-    // statistics: each thread's own sums over its tiles
-    __shared__ float ssum[CT * 5][ES_T];
+    // statistics: each thread's own sums over its tiles, in compensated pairs (their number
+    // grows with the world)
+    __shared__ float2 ssum[CT * 5][ES_T];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int H = p.H, W = p.W, K = p.kt.K, C = p.kt.C;
     const size_t N = (size_t)H * W;
     const float eps_p = p.eps_p, eps_u = p.eps_u;
     if (p.partials) {
 #pragma unroll
-        for (int v = 0; v < CT * 5; v++) ssum[v][threadIdx.x] = 0.f;
+        for (int v = 0; v < CT * 5; v++) ssum[v][threadIdx.x] = make_float2(0.f, 0.f);
     }
     const int per_world = q.tx * q.ty;
     for (int t = blockIdx.x; t < per_world * q.n_worlds; t += gridDim.x) {
@@ -630,12 +631,13 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                     const float* sx = p.sin_x + x;
                     const float* cx = p.cos_x + x;
                     const float m = (o[0] + o[1]) + (o[2] + o[3]);
-                    float* a5 = &ssum[c * 5][threadIdx.x];
-                    a5[0] += m;
-                    a5[ES_T] += m * __ldg(&p.sin_y[y]);
-                    a5[2 * ES_T] += m * __ldg(&p.cos_y[y]);
-                    a5[3 * ES_T] += (o[0] * __ldg(sx) + o[1] * __ldg(sx + 1)) + (o[2] * __ldg(sx + 2) + o[3] * __ldg(sx + 3));
-                    a5[4 * ES_T] += (o[0] * __ldg(cx) + o[1] * __ldg(cx + 1)) + (o[2] * __ldg(cx + 2) + o[3] * __ldg(cx + 3));
+                    float2* a5 = &ssum[c * 5][threadIdx.x];
+                    auto add = [&](int v, float t) { a5[v * ES_T] = ff_add(a5[v * ES_T], make_float2(t, 0.f)); };
+                    add(0, m);
+                    add(1, m * __ldg(&p.sin_y[y]));
+                    add(2, m * __ldg(&p.cos_y[y]));
+                    add(3, (o[0] * __ldg(sx) + o[1] * __ldg(sx + 1)) + (o[2] * __ldg(sx + 2) + o[3] * __ldg(sx + 3)));
+                    add(4, (o[0] * __ldg(cx) + o[1] * __ldg(cx + 1)) + (o[2] * __ldg(cx + 2) + o[3] * __ldg(cx + 3)));
                 }
             }
             if (in && p.alpha_out)
@@ -667,7 +669,7 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
         __syncthreads();
         for (int v = warp; v < C * 5; v += ES_NW) {
             float2 s = make_float2(0.f, 0.f);
-            for (int i = lane; i < ES_T; i += 32) s = ff_add(s, make_float2(ssum[v][i], 0.f));
+            for (int i = lane; i < ES_T; i += 32) s = ff_add(s, ssum[v][i]);
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) s = ff_add(s, ff_shfl_down(s, off));
             if (lane == 0) p.partials[(size_t)blockIdx.x * C * 5 + v] = s;

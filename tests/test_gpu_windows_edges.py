@@ -269,3 +269,27 @@ def test_gradients_outside_the_usual_range_stay_within_the_radius(shape, bad):
     np.testing.assert_array_equal(np.isfinite(out[0]), np.isfinite(out[1]))
     far = ~_near(H, W, H // 2, W // 2, R)
     assert np.abs(out[0] - out[1])[:, far].max() <= 1e-5
+
+
+def test_statistics_of_a_large_world_do_not_collect_rounding():
+    """A uniform world of 4096^2 sites: a thread's plain sum over its tiles would round
+    alike everywhere.  Tolerance: the result's own rounding, twice."""
+    torch = torch_mod()
+    ks = [inputs.KernelDesc(0, 0, 4, inputs.KERNEL_SHELLS, (1.0,), h=0.5, mu=0.5, sigma=0.1),
+          inputs.KernelDesc(1, 1, 4, inputs.KERNEL_SHELLS, (1.0,), h=0.5, mu=0.5, sigma=0.1)]
+    w = inputs.World(4092, 4096, 2, ks, 0.0, localized=0, maintain_genes=0)
+    cfg, kk = lenia.config_from_world(w)
+    ctx = lenia.lenia_init(cfg, kk)
+    try:
+        A = torch.empty((2, 4092, 4096), device="cuda")
+        out = torch.empty_like(A)
+        st = torch.zeros((2, 3), device="cuda")
+        for a, b in ((0.1, 0.7), (0.3, 0.9), (1.0 / 3.0, 0.6)):
+            A[0], A[1] = a, b
+            lenia.lenia_step(ctx, A, None, out, None, st)
+            torch.cuda.synchronize()
+            for c in range(2):
+                exact = float(A[c, 0, 0].double()) * 4092 * 4096
+                assert abs(float(st[c, 0].double()) - exact) <= 1.2e-7 * exact
+    finally:
+        lenia.lenia_destroy(ctx)
