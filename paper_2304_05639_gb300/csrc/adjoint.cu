@@ -28,9 +28,9 @@ constexpr float ADJ_HALF_LOG2E = 0.721347520444481703680f;   // 0.5 log2(e)
 // the forward streaming epilogue so that clip decisions match.  A site's bumps
 // and channel sums sit in its thread's column of shared memory (kernel counts
 // and routing are run-time values), and the gene terms of ADJ_KB kernels at a
-// time are summed over the block from there: a warp per value, four loads and
-// one shuffle tree, instead of a tree per warp and value (256^2, 15 kernels:
-// 17 -> 8 us with the gather).
+// time are summed over the block from there in compensated pairs: a warp per
+// value, four loads and one shuffle tree, instead of a tree per warp and value
+// (256^2, 15 kernels: 17 -> 8 us with the gather).
 __global__ void __launch_bounds__(ADJ_THREADS) k_adjoint_epilogue(const __grid_constant__ AdjParams p)
 {
     pdl_enter();
@@ -88,19 +88,20 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adjoint_epilogue(const __grid_c
             const float wd = w * d * p.inv_s2[k];
             if (valid) p.gU[(size_t)k * N + i] = -wd;
             red[(3 * j) * ADJ_THREADS + tid] = wd;
-            red[(3 * j + 1) * ADJ_THREADS + tid] = wd * d * rcp_approx(sg);
+            red[(3 * j + 1) * ADJ_THREADS + tid] = wd * d / sg;
             red[(3 * j + 2) * ADJ_THREADS + tid] = gp * (p.growth_form == 0 ? 2.f * g - 1.f : g);
         }
         __syncthreads();
         // value-major partials [K * 3][blocks]: the reduction kernel reads them coalesced
         for (int v = warp; v < 3 * kn; v += ADJ_THREADS / 32) {
             const float* r = red + v * ADJ_THREADS + lane;
-            float t = (r[0] + r[32]) + (r[64] + r[96]);
+            float2 t = ff_add(ff_add(make_float2(r[0], 0.f), make_float2(r[32], 0.f)),
+                              ff_add(make_float2(r[64], 0.f), make_float2(r[96], 0.f)));
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
+            for (int off = 16; off > 0; off >>= 1) t = ff_add(t, ff_shfl_down(t, off));
             if (lane == 0) {
                 float2* o = p.gene_partials + (size_t)(3 * k0 + v) * gridDim.x + blockIdx.x;
-                *o = ff_add(p.first ? make_float2(0.f, 0.f) : *o, make_float2(t, 0.f));
+                *o = p.first ? t : ff_add(*o, t);
             }
         }
         __syncthreads();
