@@ -272,7 +272,9 @@ LENIA_API lenia_status lenia_set_walls(lenia_ctx* ctx, const uint8_t* mask);
  * of P_out as `ev` (host) describes.  stats_out (C*3 floats), alpha_out
  * ([H][W] bytes) and epen_out ([H][W] floats, E_pen) are nullable device
  * outputs.  Without gene maps both operators must be off.  The first call
- * allocates 4 bytes of scratch per site (synchronously). */
+ * allocates 4 bytes of scratch per site (synchronously), and on FFT worlds
+ * without gene maintenance that convolve in windows the FFT passes' spectra and
+ * planes, which these steps take (Delta_sum as the passes round it). */
 LENIA_API lenia_status lenia_step_evolve(lenia_ctx* ctx, float* A, float* P, float* A_out, float* P_out,
                                          const lenia_events* ev, float* stats_out, uint8_t* alpha_out,
                                          float* epen_out, void* stream);

@@ -456,6 +456,52 @@ lenia_status build_tiles(lenia_ctx* c, cudaStream_t s)
     return LENIA_OK;
 }
 
+// The FFT path's three passes: spectra, twiddles and intermediate planes, unless the
+// context has them.  Waits for the work.
+lenia_status build_passes(lenia_ctx* c, cudaStream_t s)
+{
+    const int H = c->cfg.height, W = c->cfg.width, C = c->cfg.n_channels, NC = (int)c->conv_w.size();
+    const int M = W / 2, HS = H / 2 + 1;
+    if (c->d_S) return LENIA_OK;
+    const std::vector<float2> twM = pass_twiddles(M, ROW_RMAX), twW = twiddles(W, M + 1), twH = pass_twiddles(H, 16);
+    lenia_status st = c->d_Ahat ? LENIA_OK : dalloc(c, &c->d_Ahat, (size_t)C * H * M);
+    if (st == LENIA_OK && !c->d_Uhat) st = dalloc(c, &c->d_Uhat, (size_t)NC * H * M);
+    if (st == LENIA_OK && !c->d_twM) st = dalloc(c, &c->d_twM, twM.size());
+    if (st == LENIA_OK && !c->d_twW) st = dalloc(c, &c->d_twW, twW.size());
+    if (st == LENIA_OK && !c->d_twH) st = dalloc(c, &c->d_twH, twH.size());
+    float* S = nullptr;                        // (kept only once it is complete)
+    if (st == LENIA_OK) st = dalloc(c, &S, (size_t)NC * (M + 1) * HS);
+    if (st != LENIA_OK) return st;
+    cudaError_t e = cudaMemcpy(c->d_twM, twM.data(), twM.size() * sizeof(float2), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(c->d_twW, twW.data(), twW.size() * sizeof(float2), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(c->d_twH, twH.data(), twH.size() * sizeof(float2), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = build_spectra(c, H, W, S, s);
+    if (e != cudaSuccess) {
+        cudaFree(S);
+        return fail(c, LENIA_ECUDA, std::string("spectra: ") + cudaGetErrorString(e));
+    }
+    c->d_S = S;
+    memset(&c->fp, 0, sizeof(c->fp));
+    c->fp.Ahat = c->d_Ahat;
+    c->fp.Uhat = c->d_Uhat;
+    c->fp.S = c->d_S;
+    c->fp.tw_M = c->d_twM;
+    c->fp.tw_W = c->d_twW;
+    c->fp.tw_H = c->d_twH;
+    c->fp.H = H;
+    c->fp.W = W;
+    c->fp.C = C;
+    c->fp.K = NC;
+    c->fp.status = c->d_status;
+    c->fp.cw = C;
+    c->fp.kpw = NC;
+    for (int k = 0; k < NC; k++) {
+        const int sc = c->conv_src[k];
+        c->fp.klist[sc][c->fp.kcount[sc]++] = k;
+    }
+    return LENIA_OK;
+}
+
 // Records an event pair around each launch while profiling is on.
 struct ProfScope {
     lenia_ctx* c;
@@ -598,8 +644,8 @@ lenia_status step_impl(lenia_ctx* c, const float* A_in, const float* P_in, float
     const bool quads11 = !stats_out && !alpha_out && !empty_out && ep.kt.K == 1 && ep.kt.C == 1 && ep.W % 128 == 0 &&
                          ep.H % 8 == 0 && epilogue_batch_supported(ep);
     // worlds with alpha decisions take the windows only where the per-site kernel
-    // settles them
-    const bool windows = c->tile && (!c->cfg.maintain_genes || sites_ok);
+    // settles them; Delta_sum decisions without alpha's take the path's own form
+    const bool windows = c->tile && (c->cfg.maintain_genes ? sites_ok : !empty_out);
     const bool settle = windows && c->cfg.maintain_genes && !U_given;
     const bool sites = sites_ok && (settle || !((ep.kt.K == 1 && ep.kt.C == 1) || epilogue_rows_supported(ep)));
     if (!U_given) {
@@ -1200,34 +1246,12 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
         c->tp.n_groups = (int)grp.size() / (2 + TC_NG);
         c->tp.terms = path == LENIA_CONV_DIRECT_BF16X3 ? 3 : 1;
     } else if (path == LENIA_CONV_FFT && (!c->tile || (want_adj && c->adj_form == lenia_ctx::ADJ_PASSES))) {
-        const int M = W / 2, HS = H / 2 + 1;
-        ALLOC(c->d_Ahat, (size_t)C * H * M);
-        ALLOC(c->d_Uhat, (size_t)NC * H * M);
-        ALLOC(c->d_S, (size_t)NC * (M + 1) * HS);
-        std::vector<float2> twM = pass_twiddles(M, ROW_RMAX), twW = twiddles(W, M + 1), twH = pass_twiddles(H, 16);
-        ALLOC(c->d_twM, twM.size());
-        ALLOC(c->d_twW, twW.size());
-        ALLOC(c->d_twH, twH.size());
-        CK_INIT(cudaMemcpy(c->d_twM, twM.data(), twM.size() * sizeof(float2), cudaMemcpyHostToDevice));
-        CK_INIT(cudaMemcpy(c->d_twW, twW.data(), twW.size() * sizeof(float2), cudaMemcpyHostToDevice));
-        CK_INIT(cudaMemcpy(c->d_twH, twH.data(), twH.size() * sizeof(float2), cudaMemcpyHostToDevice));
-        CK_INIT(build_spectra(c, H, W, c->d_S, s));
-        memset(&c->fp, 0, sizeof(c->fp));
-        c->fp.Ahat = c->d_Ahat;
-        c->fp.Uhat = c->d_Uhat;
-        c->fp.S = c->d_S;
-        c->fp.tw_M = c->d_twM;
-        c->fp.tw_W = c->d_twW;
-        c->fp.tw_H = c->d_twH;
-        c->fp.H = H;
-        c->fp.W = W;
-        c->fp.C = C;
-        c->fp.K = NC;
-        c->fp.status = c->d_status;
-        c->fp.cw = C;
-        c->fp.kpw = NC;
-        memcpy(c->fp.kcount, kcount, sizeof(kcount));
-        memcpy(c->fp.klist, klist, sizeof(klist));
+        const lenia_status ps = build_passes(c, s);
+        if (ps != LENIA_OK) {
+            fprintf(stderr, "lenia_init: %s\n", c->err.c_str());
+            lenia_destroy(c);
+            return ps;
+        }
     }
     // adjoint buffers (global genes only; gene maps make alpha decisions)
     if (want_adj) {
@@ -1658,6 +1682,10 @@ lenia_status lenia_step_evolve(lenia_ctx* c, float* A, float* P, float* A_out, f
         if (st != LENIA_OK) return st;
     }
     cudaStream_t s = (cudaStream_t)stream;
+    if (c->tile && c->path == LENIA_CONV_FFT) {
+        st = build_passes(c, s);
+        if (st != LENIA_OK) return st;
+    }
     // (1) environment: walls remove material from the current state
     if (c->n_walls > 0) {
         ProfScope ps(c, KIND_WALLS, s);

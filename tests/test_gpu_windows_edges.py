@@ -293,3 +293,53 @@ def test_statistics_of_a_large_world_do_not_collect_rounding():
                 assert abs(float(st[c, 0].double()) - exact) <= 1.2e-7 * exact
     finally:
         lenia.lenia_destroy(ctx)
+
+
+@pytest.mark.parametrize("n_channels", [1, 2])
+@pytest.mark.parametrize("z", [1.0, 3.0])
+@pytest.mark.parametrize("on_windows", [False, True])
+def test_delta_sum_without_gene_maps_decides_as_the_direct_sums(n_channels, z, on_windows):
+    """Global genes: E_pen of a uniform world whose sum of growths lies between the routes'."""
+    k = inputs.KernelDesc(0, 0, 12, inputs.KERNEL_BUMPS, (1.0,), bump=FLAT.bump, h=1.0, mu=0.5, sigma=0.03)
+    ks = [dataclasses.replace(k, src=c, dst=c) for c in range(n_channels)]
+    w = inputs.World(300, 404, n_channels, ks, 0.1, localized=0, maintain_genes=0)
+    w.A = np.zeros((n_channels, 300, 404), np.float32)
+    mu, eps_u = _uniform_at_threshold(w, 0.03, z, on_windows)
+    for k in w.kernels:
+        k.mu = float(mu)
+    w.eps_u = n_channels * eps_u
+    a, b = _decisions(w, lenia.CONV_AUTO), _decisions(w, lenia.CONV_DIRECT)
+    np.testing.assert_array_equal(a[1], b[1])
+
+
+def test_delta_sum_on_fft_worlds_in_windows():
+    """A power-of-two world with global genes: evolution steps (on the passes) between
+    ordinary ones (in windows).  The threshold lies in the widest gap between the
+    sums of two neighbouring sites, so that every route decides alike."""
+    torch = torch_mod()
+    w = inputs.global_multi_channel(H=256, W=128, R=13, patch=64)
+    w.A = inputs.random_field(5, w.A.shape)
+    for k in w.kernels:
+        k.mu, k.sigma = 0.47, 0.05
+    U = np.stack([oracle.potential(w.A[k.src], K) for k, K in zip(w.kernels, oracle.world_kernels(w))])
+    t = np.sort(sum(k.h * np.exp(-0.5 * ((u - k.mu) / k.sigma) ** 2) for k, u in zip(w.kernels, U)).ravel())
+    mid = len(t) // 2
+    i = mid - 500 + int(np.argmax(np.diff(t[mid - 500:mid + 500])))
+    w.eps_u = 0.5 * (t[i] + t[i + 1])
+    assert t[i + 1] - t[i] > 4e-5
+    _, d = _decisions(w, lenia.CONV_DIRECT)
+    cfg, ks = lenia.config_from_world(w)
+    ctx = lenia.lenia_init(cfg, ks)
+    try:
+        ev = inputs.evolution_events(w, 0, gamma_mut=0.0, gamma_pen=0.0)
+        A = to_dev(w.A)
+        B, E = torch.empty_like(A), torch.empty_like(A)
+        ep = torch.zeros((w.height, w.width), device="cuda")
+        lenia.lenia_step(ctx, A, None, B, None)
+        lenia.lenia_step_evolve(ctx, A, None, E, None, ev, None, None, ep)
+        lenia.lenia_step(ctx, A, None, B, None)
+        torch.cuda.synchronize()
+        np.testing.assert_array_equal(ep.cpu().numpy(), d)
+        assert float((E - B).abs().max()) <= 1e-5
+    finally:
+        lenia.lenia_destroy(ctx)
