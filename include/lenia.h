@@ -226,7 +226,9 @@ LENIA_API lenia_status lenia_stats(lenia_ctx* ctx, const float* A, float* out, v
 
 /* Potentials U_k = K~_k * A_src(k) for every kernel (Algorithm 2, convolve
  * and normalised sum; note after Algorithm 2 for the FFT route) into U_out
- * [K][H][W], through the context's convolution path.  With n_rings > 0 the
+ * [K][H][W], through the context's convolution path (worlds with gene
+ * maintenance never in windows: lenia_update_from_potentials then decides as
+ * lenia_step does).  With n_rings > 0 the
  * ring potentials K_r * A_c instead, [C][n_rings][H][W] (Section 2.4). */
 LENIA_API lenia_status lenia_potentials(lenia_ctx* ctx, const float* A_in, float* U_out, void* stream);
 

@@ -1618,9 +1618,12 @@ lenia_status lenia_potentials(lenia_ctx* c, const float* A_in, float* U_out, voi
     cudaStream_t s = (cudaStream_t)stream;
     const bool tc = c->path == LENIA_CONV_DIRECT_BF16 || c->path == LENIA_CONV_DIRECT_BF16X3;
     const uintptr_t unit = tc ? 15 : (c->path == LENIA_CONV_FFT && !c->tile ? 7 : 3);
-    if (((uintptr_t)U_out & unit) == 0) return potentials(c, A_in, U_out, s);
+    // alpha's tests of these potentials are the caller's: where lenia_step settles its
+    // own on the direct sums, these are the direct sums
+    const bool windows = !c->cfg.maintain_genes;
+    if (((uintptr_t)U_out & unit) == 0) return potentials(c, A_in, U_out, s, nullptr, windows);
     // these forms write pairs or quads: an output that starts between them is copied
-    const lenia_status st = potentials(c, A_in, c->d_U, s);
+    const lenia_status st = potentials(c, A_in, c->d_U, s, nullptr, windows);
     if (st != LENIA_OK) return st;
     CUDA_OR_FAIL(c, cudaMemcpyAsync(U_out, c->d_U, c->N * c->conv_w.size() * sizeof(float), cudaMemcpyDeviceToDevice, s));
     return LENIA_OK;

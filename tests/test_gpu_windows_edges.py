@@ -343,3 +343,32 @@ def test_delta_sum_on_fft_worlds_in_windows():
         assert float((E - B).abs().max()) <= 1e-5
     finally:
         lenia.lenia_destroy(ctx)
+
+
+@pytest.mark.parametrize("z", [1.0, 3.0])
+@pytest.mark.parametrize("on_windows", [False, True])
+@pytest.mark.parametrize("n_channels", [1, 2])
+def test_split_step_decides_as_the_step(z, on_windows, n_channels):
+    """lenia_potentials then lenia_update_from_potentials: the alpha decisions of
+    lenia_step on a uniform world between the two routes' bumps."""
+    torch = torch_mod()
+    k = inputs.KernelDesc(0, 0, 20, inputs.KERNEL_BUMPS, (1.0,), bump=FLAT.bump, h=1.0, mu=0.5, sigma=0.03)
+    ks = [dataclasses.replace(k, src=c, dst=c) for c in range(n_channels)]
+    w = inputs.World(300, 404, n_channels, ks, 0.1, localized=3, maintain_genes=1)
+    w.A = np.zeros((n_channels, 300, 404), np.float32)
+    w.P = np.zeros((2, n_channels, 300, 404), np.float32)
+    w.P[0], w.eps_u = _uniform_at_threshold(w, 0.03, z, on_windows)
+    w.P[1] = np.float32(0.03)
+    cfg, kk = lenia.config_from_world(w)
+    ctx = lenia.lenia_init(cfg, kk)
+    try:
+        A, P = to_dev(w.A), to_dev(w.P)
+        (A1, P1), (A2, P2) = ((torch.empty_like(A), torch.empty_like(P)) for _ in range(2))
+        U = torch.empty((w.n_kernels, w.height, w.width), device="cuda")
+        lenia.lenia_potentials(ctx, A, U)
+        lenia.lenia_update_from_potentials(ctx, A, P, U, A1, P1)
+        lenia.lenia_step(ctx, A, P, A2, P2)
+        torch.cuda.synchronize()
+        assert torch.equal(P1 != 0, P2 != 0)
+    finally:
+        lenia.lenia_destroy(ctx)
