@@ -532,12 +532,12 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                             const float e = ex2_approx(-0.721347520444481703680f * z2);      // -log2(e) / 2
                             gk[c] = sg > 0.f ? e : 0.f;
                             tk[c] = p.alpha_on ? u[c] : h_of(c) * gk[c];
-                            if (NP > 0 || p.empty_out) {
+                            if (NP > 0) {
                                 const float2 r = test_range(q, u[c], tk[c], fabsf(z), sg, h_of(c));
                                 if (p.empty_out) tband[c] += fmaxf(r.y - tk[c], tk[c] - r.x);
                                 // (an exact test's range is one value)
                                 const bool open = (r.x < eps_u) & (eps_u < r.y);
-                                if (NP > 0 && (al[c] & open)) {
+                                if (al[c] & open) {
                                     many |= undecided & (1u << c);
                                     if (!((undecided >> c) & 1)) first |= (uint32_t)k << (8 * c);
                                     undecided |= 1u << c;
@@ -644,7 +644,7 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                 *reinterpret_cast<uchar4*>(p.alpha_out + i0) =
                     NP == 0 ? make_uchar4(1, 1, 1, 1) : make_uchar4(al[0], al[1], al[2], al[3]);
             // (no band: every test is exactly the direct route's, and so is their sum)
-            if (p.empty_out) {
+            if (NP > 0 && p.empty_out) {
                 uint32_t close = 0;
 #pragma unroll
                 for (int c = 0; c < 4; c++)
@@ -702,7 +702,7 @@ bool epilogue_sites_supported(const EpiParams& p)
 {
     if (p.n_rings || p.p_kern >= 0 || (size_t)p.H * p.W >= (1u << 30)) return false;
     const int loc = (p.p_mu >= 0 ? 1 : 0) | (p.p_sigma >= 0 ? 2 : 0) | (p.p_h >= 0 ? 4 : 0);
-    return loc == 0 || ((loc == 3 || loc == 7) && p.maintain && p.eps_p == 0.f && (p.r_diff == 1 || p.r_diff == 2));
+    return (loc == 0 && !p.empty_out) || ((loc == 3 || loc == 7) && p.maintain && p.eps_p == 0.f && (p.r_diff == 1 || p.r_diff == 2));
 }
 
 bool epilogue_gated(const EpiParams& p)

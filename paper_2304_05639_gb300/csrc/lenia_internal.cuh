@@ -413,7 +413,7 @@ cudaError_t launch_epilogue_queue(const EpiParams& p, const QueueWorld* worlds, 
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 cudaError_t launch_epilogue_rows(const EpiParams& p, int num_sms, int* status, cudaStream_t s, int* n_blocks);
 // The per-site rule for any kernel and channel count (mu and sigma, or mu, sigma and h
-// per site with diffusion radius 1 or 2 and eps_p = 0, or global genes;
+// per site with diffusion radius 1 or 2 and eps_p = 0, or global genes without Delta_sum;
 // epilogue_sites.cu).  A, P, U and the outputs 16-byte aligned.
 bool epilogue_sites_supported(const EpiParams& p);
 // whether sites without a first gene around them are known to have alpha = 0
