@@ -28,9 +28,9 @@ constexpr float ADJ_HALF_LOG2E = 0.721347520444481703680f;   // 0.5 log2(e)
 // the forward streaming epilogue so that clip decisions match.  A site's bumps
 // and channel sums sit in its thread's column of shared memory (kernel counts
 // and routing are run-time values), and the gene terms of ADJ_KB kernels at a
-// time are summed over the block from there in compensated pairs: a warp per
-// value, four loads and one shuffle tree, instead of a tree per warp and value
-// (256^2, 15 kernels: 17 -> 8 us with the gather).
+// time are summed over the block from there in compensated pairs, four values a
+// warp (256^2, 15 kernels: 17 -> 8 us with the gather; a pass of 12 steps 1.05 ms
+// with a shuffle tree of pairs per value).
 __global__ void __launch_bounds__(ADJ_THREADS) k_adjoint_epilogue(const __grid_constant__ AdjParams p)
 {
     pdl_enter();
@@ -81,27 +81,43 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adjoint_epilogue(const __grid_c
         for (int j = 0; j < kn; j++) {
             const int k = k0 + j;
             const float d = __ldg(&p.U[(size_t)k * N + ic]) - p.kt.mu[k];
-            const float sg = p.kt.sigma[k], h = p.kt.h[k];
+            const float h = p.kt.h[k];
             const float g = bump[k * ADJ_THREADS + tid];
             const float gp = chan[p.kt.dst[k] * ADJ_THREADS + tid] * p.dt;
             const float w = gp * h * fp * g;                // dL/d(exp term)
             const float wd = w * d * p.inv_s2[k];
             if (valid) p.gU[(size_t)k * N + i] = -wd;
             red[(3 * j) * ADJ_THREADS + tid] = wd;
-            red[(3 * j + 1) * ADJ_THREADS + tid] = wd * d / sg;
+            red[(3 * j + 1) * ADJ_THREADS + tid] = wd * d;
             red[(3 * j + 2) * ADJ_THREADS + tid] = gp * (p.growth_form == 0 ? 2.f * g - 1.f : g);
         }
         __syncthreads();
-        // value-major partials [K * 3][blocks]: the reduction kernel reads them coalesced
-        for (int v = warp; v < 3 * kn; v += ADJ_THREADS / 32) {
-            const float* r = red + v * ADJ_THREADS + lane;
-            float2 t = ff_add(ff_add(make_float2(r[0], 0.f), make_float2(r[32], 0.f)),
-                              ff_add(make_float2(r[64], 0.f), make_float2(r[96], 0.f)));
+        // value-major partials [K * 3][blocks]: the reduction kernel reads them coalesced.
+        // Four values a warp: the lanes halve twice over the values, then three times
+        // over the sites, and lanes 0, 8, 16 and 24 end with a value each.
+        for (int v0 = 4 * warp; v0 < 3 * kn; v0 += ADJ_THREADS / 8) {
+            float2 t[4];
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) t = ff_add(t, ff_shfl_down(t, off));
-            if (lane == 0) {
+            for (int j = 0; j < 4; j++) {
+                const float* r = red + min(v0 + j, 3 * kn - 1) * ADJ_THREADS + lane;
+                t[j] = ff_add(ff_add(make_float2(r[0], 0.f), make_float2(r[32], 0.f)),
+                              ff_add(make_float2(r[64], 0.f), make_float2(r[96], 0.f)));
+            }
+            const bool hi = lane & 16, mid = lane & 8;
+            const float2 s0 = ff_shfl_xor(hi ? t[0] : t[2], 16), s1 = ff_shfl_xor(hi ? t[1] : t[3], 16);
+            const float2 h0 = ff_add(hi ? t[2] : t[0], s0), h1 = ff_add(hi ? t[3] : t[1], s1);
+            float2 u = ff_add(mid ? h1 : h0, ff_shfl_xor(mid ? h0 : h1, 8));
+#pragma unroll
+            for (int off = 4; off > 0; off >>= 1) u = ff_add(u, ff_shfl_xor(u, off));
+            const int v = v0 + (hi ? 2 : 0) + (mid ? 1 : 0);
+            if ((lane & 7) == 0 && v < 3 * kn) {
+                if (v % 3 == 1) {
+                    // dL/dsigma: the sum's sites share the division by sigma
+                    const float sg = p.kt.sigma[k0 + v / 3], q = u.x / sg;
+                    u = make_float2(q, (fmaf(-q, sg, u.x) + u.y) / sg);
+                }
                 float2* o = p.gene_partials + (size_t)(3 * k0 + v) * gridDim.x + blockIdx.x;
-                *o = p.first ? t : ff_add(*o, t);
+                *o = p.first ? u : ff_add(*o, u);
             }
         }
         __syncthreads();

@@ -87,6 +87,11 @@ __device__ __forceinline__ float2 ff_shfl_down(float2 v, int off)
     return make_float2(__shfl_down_sync(0xffffffffu, v.x, off), __shfl_down_sync(0xffffffffu, v.y, off));
 }
 
+__device__ __forceinline__ float2 ff_shfl_xor(float2 v, int mask)
+{
+    return make_float2(__shfl_xor_sync(0xffffffffu, v.x, mask), __shfl_xor_sync(0xffffffffu, v.y, mask));
+}
+
 // One channel's outputs from its five reduced sums tot[c * 5 + (M, S_y,
 // C_y, S_x, C_x)]: axis 0 (y) also writes the mass; each axis writes the
 // circular-mean centre atan2(S, C) n / (2 pi) wrapped to [0, n), in FP64 on
