@@ -332,8 +332,12 @@ __device__ __forceinline__ bool alpha_at(const SitesParams& q, const float* A, c
         const float hh = p.p_h >= 0 ? g[p.p_h] : p.kt.h[kk];
         float u = on ? __ldg(&U[(size_t)kk * N + (size_t)y * W + x]) : 0.f;
         float t = settled(q, u, m, sg, hh).y;
-        const float2 r = test_range(q, u, t, fabsf((u - m) * rcp_approx(sg)), sg, hh);
-        const bool open = on && r.x < p.eps_u && p.eps_u < r.y;
+        // a lane's first kernel is known to be undecided
+        bool open = on;
+        if (__any_sync(0xffffffffu, on && kk != first)) {
+            const float2 r = test_range(q, u, t, fabsf((u - m) * rcp_approx(sg)), sg, hh);
+            open = on && (kk == first || (r.x < p.eps_u && p.eps_u < r.y));
+        }
         if (q.g.du > 0.f && __any_sync(0xffffffffu, open)) {
             u = direct_sums(q, A, kk, y, x, open);
             if (open) t = settled(q, u, m, sg, hh).y;
