@@ -22,8 +22,10 @@
 // other update kernels' arithmetic on the direct sums, so that a world's
 // decisions do not depend on the kernel or the convolution it takes.  (Settled
 // inside the kernels' loop, or with a site of each lane at a time, the guard that
-// large radii need makes a step of 600 x 900 at R = 45 / 56 1.15 / 2.25 ms; 0.44 /
-// 0.72 so, 0.56 / 0.93 with the direct sums throughout.)
+// large radii need makes a step of 600 x 900 at R = 45 / 56 1.15 / 2.25 ms; 0.31 /
+// 0.57 so, 0.56 / 0.93 with the direct sums throughout.  At R = 12, 13 a step has
+// one such site or none at 300 x 404, some 25 at 1080 x 1920, and they cost its
+// latency: 104 us for six steps of 300 x 404 where two have one, 79 without any.)
 //
 // What bounds it: on a mostly empty world the writes of the gene planes, on a
 // full one its loads and instruction issue (16 warps an SM at 128 registers, half of
@@ -132,7 +134,9 @@ __device__ __forceinline__ int tap_site(int2 tap, int y, int x, int H, int W)
 
 // Kernel k's direct sum at (y, x): its non-zero taps in k_direct_conv's order (a zero
 // weight adds nothing there), so the same bits.  By a whole warp: the lanes load
-// 4 x 32 taps at once, the next ones while every lane adds these in order.
+// 4 x 32 taps at once, the next ones while every lane adds these in order.  (This and
+// the code around it runs at a few sites a step, so it is kept small: what it costs
+// there is its latency, instruction fetches among it.)
 __device__ __forceinline__ float direct_warp(const SitesParams& q, const float* A, int k, int y, int x)
 {
     constexpr int B = 4;
@@ -146,37 +150,40 @@ __device__ __forceinline__ float direct_warp(const SitesParams& q, const float* 
             const int t = t0 + 32 * j + lane;
             const int2 tap = t < t1 ? __ldg(&q.g.taps[t]) : make_int2((1024 << 11) + 1024, 0);
             wn[j] = __int_as_float(tap.y);
-            vn[j] = __ldg(&plane[tap_site(tap, y, x, H, W)]);
+            vn[j] = t < t1 ? __ldg(&plane[tap_site(tap, y, x, H, W)]) : 0.f;
         }
     };
     float acc = 0.f;
     fetch(q.g.off[k]);
+#pragma unroll 1
     for (int t0 = q.g.off[k]; t0 < t1; t0 += 32 * B) {
         float v[B], w[B];
 #pragma unroll
         for (int j = 0; j < B; j++) v[j] = vn[j], w[j] = wn[j];
-        if (t0 + 32 * B < t1) fetch(t0 + 32 * B);
+        fetch(t0 + 32 * B);
 #pragma unroll
         for (int j = 0; j < B; j++) {
-            const int n = min(32, t1 - (t0 + 32 * j));
+            if (t0 + 32 * j >= t1) break;
 #pragma unroll 8
-            for (int i = 0; i < n; i++)
+            for (int i = 0; i < 32; i++)       // (beyond t1: 0 x 0)
                 acc = fmaf(__shfl_sync(0xffffffffu, w[j], i), __shfl_sync(0xffffffffu, v[j], i), acc);
         }
     }
     return acc;
 }
 
-// The direct sums of the lanes that want one (the whole warp calls it).  A sum's
-// additions are one chain, so several sites go side by side, a lane each, 32 taps
-// in flight; up to four take the whole warp each (R = 56, 9648 taps: about 35 us
-// a site against 135 for up to 32).
+// The direct sums of the lanes that want one (the whole warp calls it).  Up to four
+// sites take the warp one after the other; more go side by side, a lane each
+// (a sum's additions are one chain), the lanes passing the taps round.
 __device__ __forceinline__ float direct_sums(const SitesParams& q, const float* A, int k, int y, int x, bool want)
 {
-    const int H = q.e.H, W = q.e.W, lane = threadIdx.x & 31;
+    constexpr int B = 8;
+    const int H = q.e.H, W = q.e.W, lane = threadIdx.x & 31, R = q.g.R;
     uint32_t m = __ballot_sync(0xffffffffu, want);
+    const int t1 = q.g.off[k + 1];
     float acc = 0.f;
     if (__popc(m) <= 4) {
+#pragma unroll 1
         for (; m; m &= m - 1) {
             const int L = __ffs(m) - 1;
             const float s = direct_warp(q, A, k, __shfl_sync(0xffffffffu, y, L), __shfl_sync(0xffffffffu, x, L));
@@ -184,23 +191,39 @@ __device__ __forceinline__ float direct_sums(const SitesParams& q, const float* 
         }
         return acc;
     }
-    const float* plane = A + (size_t)q.e.kt.src[k] * H * W;
-    const int t1 = q.g.off[k + 1];
     if (q.g.off[k] == t1) return 0.f;
-    int2 next = __ldg(&q.g.taps[min(q.g.off[k] + lane, t1 - 1)]);
+    // the other lanes read along at the first site
+    const int L = __ffs(m) - 1, y0 = __shfl_sync(0xffffffffu, y, L), x0 = __shfl_sync(0xffffffffu, x, L);
+    if (!want) {
+        y = y0;
+        x = x0;
+    }
+    const bool inner = __all_sync(0xffffffffu, y >= R && y < H - R && x >= R && x < W - R);
+    const float* plane = A + (size_t)q.e.kt.src[k] * H * W;
+    const float* at = plane + (size_t)y * W + x;
+    auto fetch = [&](int t) { return __ldg(&q.g.taps[min(t + lane, t1 - 1)]); };
+    int2 next = fetch(q.g.off[k]);
+#pragma unroll 1
     for (int t0 = q.g.off[k]; t0 < t1; t0 += 32) {
         const int2 tap = next;
-        next = __ldg(&q.g.taps[min(t0 + 32 + lane, t1 - 1)]);
-        float v[32];
+        next = fetch(t0 + 32);
+        const int off = ((tap.x >> 11) - 1024) * W + (tap.x & 2047) - 1024;
+#pragma unroll 1
+        for (int h = 0; h < 32; h += B) {
+            float v[B];
+            if (inner) {
 #pragma unroll
-        for (int j = 0; j < 32; j++) {
-            const int at = __shfl_sync(0xffffffffu, tap.x, j);
-            v[j] = want ? __ldg(&plane[tap_site(make_int2(at, 0), y, x, H, W)]) : 0.f;
-        }
+                for (int j = 0; j < B; j++) v[j] = __ldg(at + __shfl_sync(0xffffffffu, off, h + j));
+            } else {
 #pragma unroll
-        for (int j = 0; j < 32; j++) {
-            const float w = __int_as_float(__shfl_sync(0xffffffffu, tap.y, j));
-            if (t0 + j < t1) acc = fmaf(w, v[j], acc);
+                for (int j = 0; j < B; j++)
+                    v[j] = __ldg(plane + tap_site(make_int2(__shfl_sync(0xffffffffu, tap.x, h + j), 0), y, x, H, W));
+            }
+#pragma unroll
+            for (int j = 0; j < B; j++) {
+                const float w = __int_as_float(__shfl_sync(0xffffffffu, tap.y, h + j));
+                if (t0 + h + j < t1) acc = fmaf(w, v[j], acc);
+            }
         }
     }
     return acc;
@@ -208,34 +231,41 @@ __device__ __forceinline__ float direct_sums(const SitesParams& q, const float* 
 
 // The warp's marked sites (bit c of a lane's marks: its column c), dealt to the lanes 32
 // at a time: `one(y, x, owner, c, valid)` handles a lane's site, for the whole warp, and
-// its result goes back to the owner's `take(c, result)`.
+// its result goes back to the owner's `take(c, result)`.  slot: the warp's 32 bytes.
 template <class One, class Take>
-__device__ __forceinline__ void deal_sites(uint32_t marks, int y, int x, One one, Take take)
+__device__ __forceinline__ void deal_sites(uint8_t* slot, uint32_t marks, int y, int x, One one, Take take)
 {
     const int lane = threadIdx.x & 31;
-    uint32_t b[4];
-    int n[5] = {0, 0, 0, 0, 0};
+    int before = 0, total = 0;                 // marks of the lanes below, of all
 #pragma unroll
     for (int c = 0; c < 4; c++) {
-        b[c] = __ballot_sync(0xffffffffu, (marks >> c) & 1);
-        n[c + 1] = n[c] + __popc(b[c]);
+        const uint32_t b = __ballot_sync(0xffffffffu, (marks >> c) & 1);
+        before += __popc(b & ((1u << lane) - 1));
+        total += __popc(b);
     }
-    for (int base = 0; base < n[4]; base += 32) {
-        const int j = base + lane;
-        int c = 0, owner = 0;
+#pragma unroll 1
+    for (int base = 0; base < total; base += 32) {
+        int r = before - base;
 #pragma unroll
-        for (int i = 0; i < 4; i++)
-            if (j >= n[i] && j < n[i + 1]) {
-                c = i;
-                owner = (int)__fns(b[i], 0, j - n[i] + 1);
+        for (int c = 0; c < 4; c++)
+            if ((marks >> c) & 1) {
+                if (r >= 0 && r < 32) slot[r] = (uint8_t)(4 * lane + c);
+                r++;
             }
-        const float r = one(__shfl_sync(0xffffffffu, y, owner), __shfl_sync(0xffffffffu, x, owner) + c, owner, c, j < n[4]);
+        __syncwarp();
+        const bool valid = base + lane < total;
+        const int s = valid ? slot[lane] : 0, owner = s >> 2, c = s & 3;
+        const float res = one(__shfl_sync(0xffffffffu, y, owner), __shfl_sync(0xffffffffu, x, owner) + c, owner, c, valid);
+        r = before - base;
 #pragma unroll
         for (int i = 0; i < 4; i++) {
-            const int rank = n[i] + __popc(b[i] & ((1u << lane) - 1)) - base;
-            const float v = __shfl_sync(0xffffffffu, r, rank & 31);
-            if (((marks >> i) & 1) && rank >= 0 && rank < 32) take(i, v);
+            const float v = __shfl_sync(0xffffffffu, res, r & 31);
+            if ((marks >> i) & 1) {
+                if (r >= 0 && r < 32) take(i, v);
+                r++;
+            }
         }
+        __syncwarp();
     }
 }
 
@@ -321,6 +351,7 @@ __device__ __forceinline__ bool alpha_at(const SitesParams& q, const float* A, c
     const size_t N = (size_t)p.H * W;
     bool ok = want;
     int k = first;                             // (a lane's own; K: done)
+#pragma unroll 1
     while (__any_sync(0xffffffffu, ok && k < K)) {
         // the lanes at the warp's lowest kernel go on
         const int kk = __reduce_min_sync(0xffffffffu, ok && k < K ? k : K);
@@ -386,6 +417,7 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
     // statistics: each thread's own sums over its tiles, in compensated pairs (their number
     // grows with the world)
     __shared__ float2 ssum[CT * 5][ES_T];
+    __shared__ uint8_t slot[ES_NW][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int H = p.H, W = p.W, K = p.kt.K, C = p.kt.C;
     const size_t N = (size_t)H * W;
@@ -592,7 +624,7 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                 if (__any_sync(0xffffffffu, open != 0)) {
                     uint32_t lost = 0;
                     deal_sites(
-                        open, y, x,
+                        slot[warp], open, y, x,
                         [&](int ys, int xs, int owner, int c, bool valid) {
                             const int k0 = (__shfl_sync(0xffffffffu, first, owner) >> (8 * c)) & 255;
                             const bool more = (__shfl_sync(0xffffffffu, many, owner) >> c) & 1;
@@ -655,7 +687,7 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                     close |= (in && tband[c] > 0.f && fabsf(tsum[c] - eps_u) <= tband[c] + 1e-6f ? 1u : 0u) << c;
                 if (__any_sync(0xffffffffu, close != 0))
                     deal_sites(
-                        close, y, x,
+                        slot[warp], close, y, x,
                         [&](int ys, int xs, int, int, bool valid) { return tests_at(q, pA, pP, pU, ys, xs, valid); },
                         [&](int c, float t) {
 #pragma unroll

@@ -397,6 +397,7 @@ GuardParams window_guard(const lenia_ctx* c)
 {
     GuardParams g;
     memset(&g, 0, sizeof(g));
+    g.R = c->max_R;
     bool negative = false;
     double du = 0.0, floor = 0.0, slope = 0.0;
     for (size_t k = 0; k < c->conv_w.size(); k++) {

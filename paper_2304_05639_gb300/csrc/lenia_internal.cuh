@@ -431,6 +431,7 @@ struct GuardParams {
     int off[kMaxKernels + 1];
     float du;                  // 0: the potentials are the direct sums already
     float slope, floor;        // at a potential u: the smaller of du and slope u + floor
+    int R;                     // the largest radius
 };
 // fast: the streaming kernel's reciprocals and exponential, else divisions and expf
 cudaError_t launch_epilogue_sites(const EpiParams& p, bool fast, const GuardParams* guard, int n_worlds, int max_blocks,
