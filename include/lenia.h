@@ -436,14 +436,18 @@ LENIA_API lenia_status lenia_batch_rollout(lenia_batch* batch, float* const* A, 
  * kernel topology are identical - kernel shapes may differ, and global genes
  * that the gene maps replace are ignored - step together:
  * one launch per stage for the whole group, the worlds along the launch's
- * planes or grid z), or -1 when it steps on its own (or w is out of range).
- * A grouped world's epilogue is the tiled kernel (FP32 division and expf),
- * which can differ in the last bits from the streaming kernel a world of
- * width 256 k uses on its own when that kernel is chosen (steps with
- * statistics, several kernels or channels). */
+ * planes or grid z; worlds without gene maintenance may convolve in windows,
+ * one launch per window size), or -1 when it steps on its own (or w is out of
+ * range).  At widths of 64 and 128 a grouped world gives the bits it gives on
+ * its own.  At widths of 256 k it can differ in the last bits: the
+ * convolution's form is chosen for the group, and its epilogue is the tiled
+ * kernel (FP32 division and expf; one kernel) or the per-site kernel (several)
+ * where a world on its own may take the streaming one. */
 LENIA_API int32_t lenia_batch_group_of(const lenia_batch* batch, int32_t world);
 /* Epilogue shape of world w's group: 0 = the tiled kernel, *param = rows per
- * thread (1, 2 or 4); 2 = the tiled kernel with four adjacent columns per
+ * thread (1, 2 or 4; for worlds of several kernels, one site or quad of sites
+ * per thread whatever param says, by the per-site kernel where every state
+ * buffer is 16-byte aligned); 2 = the tiled kernel with four adjacent columns per
  * thread (float4 loads; one-kernel worlds of width 128 k with 16-byte aligned
  * state buffers), *param = rows per thread (1 or 2); 1 = the streaming kernel
  * in one persistent launch over

@@ -43,12 +43,14 @@ struct ShapeKey {
 struct Group {
     std::vector<int> worlds;
     lenia::lenia_ctx_view v;               // the first world's parameters
-    float2* Ahat = nullptr;                // [n][C][M][H]
-    float2* Uhat = nullptr;                // [n][K][M][H]
+    float2* Ahat = nullptr;                // [n_pass][C][M][H]
+    float2* Uhat = nullptr;                // [n_pass][K][M][H]
     float* U = nullptr;                    // [n][K][H][W]
-    const float** S = nullptr;             // per-world kernel spectra (worlds may differ in kernels)
-    // worlds that convolve in windows: one launch per window size (their radii,
-    // and so their window sizes, may differ), the worlds' buffers per direction
+    const float** S = nullptr;             // [n_pass] kernel spectra (worlds may differ in kernels)
+    // The first n_pass worlds take the three passes, the others convolve in windows: one
+    // launch per window size (their radii, and so their window sizes, may
+    // differ), the worlds' buffers per direction
+    int n_pass = 0;
     struct TileSet {
         lenia::TileParams p;
         std::vector<int> member;           // positions in `worlds`
@@ -164,7 +166,10 @@ cudaError_t group_epilogue(const Group& g, int dir, cudaStream_t s)
 {
     const lenia::EpiParams ep = group_epi(g, dir);
     const int n = (int)g.worlds.size();
-    // several kernels: the per-site kernel, as a world takes on its own
+    // several kernels: the per-site kernel, as a world takes on its own (15 kernels, us
+    // per 4 steps against the tiled kernel: global genes 64^2 x 64 98 / 121, 256^2 x 4
+    // 142 / 165, 512^2 x 16 1166 / 1621; gene maps 64^2 x 64 267 / 411, 128^2 x 4 92 /
+    // 138, 512^2 x 16 1.32 / 4.54 ms)
     if (g.epi == 0 && ep.kt.K > 1 && g.aligned_all && lenia::epilogue_sites_supported(ep))
         return lenia::launch_epilogue_sites(ep, false, nullptr, n, 1 << 20, s, nullptr);
     if (g.epi == 1) return lenia::launch_epilogue_queue(ep, g.qw[dir], n, g.bands, 0, g.counter, g.v.fp.status, s);
@@ -175,14 +180,13 @@ cudaError_t group_epilogue(const Group& g, int dir, cudaStream_t s)
 // One step of every world of a group: A/P lists of direction `dir`.
 lenia_status group_step(const Group& g, int dir, cudaStream_t s)
 {
-    const int n = (int)g.worlds.size();
     for (const Group::TileSet& t : g.tiles) {
         lenia::TileParams tp = t.p;
         tp.worlds = t.list[dir];
         tp.aligned = g.aligned ? 1 : 0;
         if (lenia::launch_tile_conv(tp, s) != cudaSuccess) return LENIA_ECUDA;
     }
-    if (!g.tiles.empty()) return group_epilogue(g, dir, s) == cudaSuccess ? LENIA_OK : LENIA_ECUDA;
+    if (!g.n_pass) return group_epilogue(g, dir, s) == cudaSuccess ? LENIA_OK : LENIA_ECUDA;
     lenia::FftParams fp = g.v.fp;
     fp.A = nullptr;
     fp.A_list = g.Ain[dir];
@@ -193,8 +197,8 @@ lenia_status group_step(const Group& g, int dir, cudaStream_t s)
     fp.U = g.U;
     fp.cw = g.v.C;
     fp.kpw = g.v.K;
-    fp.C = n * g.v.C;                      // planes of the row and column passes
-    fp.K = n * g.v.K;                      // planes of the inverse row pass
+    fp.C = g.n_pass * g.v.C;               // planes of the row and column passes
+    fp.K = g.n_pass * g.v.K;               // planes of the inverse row pass
     if (lenia::launch_fft_rows_r2c(fp, s) != cudaSuccess) return LENIA_ECUDA;
     if (lenia::launch_fft_cols(fp, s) != cudaSuccess) return LENIA_ECUDA;
     if (lenia::launch_fft_rows_c2r(fp, s) != cudaSuccess) return LENIA_ECUDA;
@@ -212,7 +216,8 @@ lenia_status tune_epilogue(Group& g, cudaStream_t s)
     struct Cand {
         int epi, br, bands;
     };
-    std::vector<Cand> cands = {{0, 1, 1}, {0, 2, 1}, {0, 4, 1}};
+    std::vector<Cand> cands = {{0, 1, 1}};
+    if (g.v.K == 1) cands.insert(cands.end(), {{0, 2, 1}, {0, 4, 1}});     // (rows per thread: one-kernel worlds only)
     // four columns per thread (float4 loads; widths of 128 k, every listed pointer 16-byte aligned)
     if (g.v.K == 1 && g.v.C == 1 && g.v.fp.W % 128 == 0 && g.aligned_all)
         for (int b : {-1, -2})
@@ -478,7 +483,7 @@ lenia_status lenia_batch_init(int32_t n_worlds, const lenia_config* cfgs, const 
             std::vector<double> key = {(double)c0.height, (double)c0.width, (double)c0.n_channels,
                                        (double)c0.n_kernels, c0.dt, (double)c0.growth_form, (double)c0.localized,
                                        (double)c0.maintain_genes, c0.eps_u, c0.eps_p, (double)c0.r_diff,
-                                       (double)c0.alpha_on, (double)c0.n_rings, (double)v.tile};
+                                       (double)c0.alpha_on, (double)c0.n_rings};
             // kernel shapes may differ (each world's spectra are read through a list)
             for (int k = 0; k < c0.n_kernels; k++) {
                 const lenia_kernel_desc& d = ks[k];
@@ -495,51 +500,68 @@ lenia_status lenia_batch_init(int32_t n_worlds, const lenia_config* cfgs, const 
             if (kv.second.size() < 2) continue;
             Group g;
             g.worlds = kv.second;
-            lenia::ctx_view(b->ctx[g.worlds[0]], &g.v);
             const size_t n = g.worlds.size();
             const size_t H = cfgs[g.worlds[0]].height, W = cfgs[g.worlds[0]].width, M = W / 2;
-            bool okg = cudaMalloc(&g.U, n * g.v.K * g.v.N * sizeof(float)) == cudaSuccess;
-            if (g.v.tile) {
-                std::map<int, std::vector<int>> by_size;
-                for (size_t j = 0; okg && j < n; j++) {
-                    lenia_ctx* c = b->ctx[g.worlds[j]];
-                    // widths of 256 k: the window size that suits the whole group.  At
-                    // others a grouped world keeps the window size it has on its
-                    // own, and with it its results bit for bit
-                    if (W % 256 == 0) okg = lenia::ctx_group_tiles(c, (int)n, s) == cudaSuccess;
-                    lenia::lenia_ctx_view vj;
-                    lenia::ctx_view(c, &vj);
-                    by_size[vj.tl.N].push_back((int)j);
-                }
-                for (auto& bs : by_size) {
-                    Group::TileSet t;
-                    t.member = bs.second;
-                    lenia::lenia_ctx_view vj;
-                    lenia::ctx_view(b->ctx[g.worlds[t.member[0]]], &vj);
-                    t.p = vj.tl;
-                    t.p.n_worlds = (int)t.member.size();
-                    t.p.kpb = 64;                       // every kernel of a channel in one block
-                    t.p.tiles = 0;
-                    for (int j : t.member) {
-                        lenia::ctx_view(b->ctx[g.worlds[j]], &vj);
-                        t.p.tiles = std::max(t.p.tiles, vj.tl.g.tiles_x * vj.tl.g.tiles_y);
+            const int C = cfgs[g.worlds[0]].n_channels, K = cfgs[g.worlds[0]].n_kernels;
+            // Passes or windows: at widths of 256 k, where a world on its own may take
+            // another update kernel anyway, what suits the whole group; at others (64 and
+            // 128) what each world takes on its own, and with it its results bit for bit
+            bool okg = true;
+            if (W % 256 == 0) {
+                double t_win = 0.0;
+                for (int i : g.worlds) t_win = std::max(t_win, lenia::ctx_group_cost(b->ctx[i], (int)n));
+                const bool windows = t_win < lenia::fft_passes_cost((int)H, (int)W, (int)n * (C + K));
+                for (int i : g.worlds) okg = okg && lenia::ctx_group_form(b->ctx[i], (int)n, windows, s) == cudaSuccess;
+            }
+            auto tiled = [&](int i) {
+                lenia::lenia_ctx_view vi;
+                lenia::ctx_view(b->ctx[i], &vi);
+                return vi.tile;
+            };
+            std::stable_partition(g.worlds.begin(), g.worlds.end(), [&](int i) { return !tiled(i); });
+            for (int i : g.worlds) g.n_pass += !tiled(i);
+            lenia::ctx_view(b->ctx[g.worlds[0]], &g.v);
+            okg = okg && cudaMalloc(&g.U, n * g.v.K * g.v.N * sizeof(float)) == cudaSuccess;
+            std::map<int, std::vector<int>> by_size;
+            for (size_t j = g.n_pass; j < n; j++) {
+                lenia::lenia_ctx_view vj;
+                lenia::ctx_view(b->ctx[g.worlds[j]], &vj);
+                by_size[vj.tl.N].push_back((int)j);
+            }
+            for (auto& bs : by_size) {
+                Group::TileSet t;
+                t.member = bs.second;
+                lenia::lenia_ctx_view vj;
+                lenia::ctx_view(b->ctx[g.worlds[t.member[0]]], &vj);
+                t.p = vj.tl;
+                t.p.n_worlds = (int)t.member.size();
+                t.p.tiles = 0;
+                for (int j : t.member) {
+                    lenia::ctx_view(b->ctx[g.worlds[j]], &vj);
+                    const int tiles = vj.tl.g.tiles_x * vj.tl.g.tiles_y;
+                    if (tiles > t.p.tiles) {
+                        t.p.tiles = tiles;
+                        t.p.g = vj.tl.g;
                     }
-                    for (int d = 0; okg && d < 2; d++)
-                        okg = cudaMalloc(&t.list[d], t.member.size() * sizeof(lenia::TileWorld)) == cudaSuccess;
-                    g.tiles.push_back(t);
                 }
-            } else {
-                okg = okg && cudaMalloc(&g.Ahat, n * g.v.C * M * H * sizeof(float2)) == cudaSuccess &&
-                      cudaMalloc(&g.Uhat, n * g.v.K * M * H * sizeof(float2)) == cudaSuccess &&
-                      cudaMalloc(&g.S, n * sizeof(float*)) == cudaSuccess;
+                lenia::tile_choose_kpb(&t.p, t.p.kcount, t.p.n_worlds);
+                for (int d = 0; okg && d < 2; d++)
+                    okg = cudaMalloc(&t.list[d], t.member.size() * sizeof(lenia::TileWorld)) == cudaSuccess;
+                g.tiles.push_back(t);
+            }
+            if (okg && g.n_pass) {
+                const size_t m = g.n_pass;
+                okg = cudaMalloc(&g.Ahat, m * g.v.C * M * H * sizeof(float2)) == cudaSuccess &&
+                      cudaMalloc(&g.Uhat, m * g.v.K * M * H * sizeof(float2)) == cudaSuccess &&
+                      cudaMalloc(&g.S, m * sizeof(float*)) == cudaSuccess;
                 if (okg) {
-                    std::vector<const float*> spec(n);
-                    for (size_t j = 0; j < n; j++) {
+                    std::vector<const float*> spec(m);
+                    for (size_t j = 0; j < m; j++) {
                         lenia::lenia_ctx_view vj;
                         lenia::ctx_view(b->ctx[g.worlds[j]], &vj);
                         spec[j] = vj.fp.S;
                     }
-                    okg = cudaMemcpy(g.S, spec.data(), n * sizeof(float*), cudaMemcpyHostToDevice) == cudaSuccess;
+                    okg = cudaMemcpy(g.S, spec.data(), m * sizeof(float*), cudaMemcpyHostToDevice) == cudaSuccess;
                 }
             }
             for (int d = 0; okg && d < 2; d++)

@@ -777,10 +777,32 @@ bool ctx_view(lenia_ctx* c, lenia_ctx_view* v)
     return true;
 }
 
-cudaError_t ctx_group_tiles(lenia_ctx* c, int n_worlds, cudaStream_t s)
+double ctx_group_cost(const lenia_ctx* c, int n_worlds)
 {
-    if (!c || !c->tile) return cudaErrorInvalidValue;
-    const int n = c->tl.N;
+    if (!c || c->path != LENIA_CONV_FFT || c->cfg.maintain_genes) return INFINITY;
+    int kcount[kMaxChannels] = {0};
+    for (int src : c->conv_src) kcount[src]++;
+    TileParams tl;
+    memset(&tl, 0, sizeof(tl));
+    return tile_choose(&tl, c->cfg.height, c->cfg.width, kcount, c->max_R, n_worlds);
+}
+
+cudaError_t ctx_group_form(lenia_ctx* c, int n_worlds, bool windows, cudaStream_t s)
+{
+    if (!c || c->path != LENIA_CONV_FFT) return cudaErrorInvalidValue;
+    if (!windows) {
+        c->tile = false;
+        return build_passes(c, s) == LENIA_OK ? cudaSuccess : cudaErrorUnknown;
+    }
+    const int n = c->tile ? c->tl.N : 0;
+    if (!c->tile) memset(&c->tl, 0, sizeof(c->tl));
+    c->tile = true;
+    c->tl.C = c->cfg.n_channels;
+    memset(c->tl.kcount, 0, sizeof(c->tl.kcount));
+    for (int k = 0; k < (int)c->conv_src.size(); k++) {
+        const int sc = c->conv_src[k];
+        c->tl.klist[sc][c->tl.kcount[sc]++] = k;
+    }
     tile_choose(&c->tl, c->cfg.height, c->cfg.width, c->tl.kcount, c->max_R, n_worlds);
     return c->tl.N == n || build_tiles(c, s) == LENIA_OK ? cudaSuccess : cudaErrorUnknown;
 }

@@ -327,6 +327,8 @@ bool tile_plan(TileParams* p, int N, int H, int W, int R);
 // (n_worlds: worlds of that shape in one launch)
 double tile_choose(TileParams* p, int H, int W, const int* kcount, int R, int n_worlds = 1,
                    bool gated = false);
+// The faster number of kernels per block for p's window size, n_worlds in one launch.
+void tile_choose_kpb(TileParams* p, const int* kcount, int n_worlds);
 // time models of the transposed convolution: summed per channel in the frequency
 // domain, or plane by plane
 double tile_adj_cost(const TileParams& p, const int* kcount);
@@ -452,8 +454,11 @@ struct lenia_ctx_view {
 struct lenia_ctx;
 namespace lenia {
 bool ctx_view(lenia_ctx* c, lenia_ctx_view* v);
-// Window size for a world of a group of n_worlds (rebuilds its spectra); waits for the work.
-cudaError_t ctx_group_tiles(lenia_ctx* c, int n_worlds, cudaStream_t s);
+// The convolution of a world in a group of n_worlds: the windows' time by the model
+// (infinite where the world may not take them), and the choice carried out (windows
+// of the size that suits the group, or the three passes; waits for the work).
+double ctx_group_cost(const lenia_ctx* c, int n_worlds);
+cudaError_t ctx_group_form(lenia_ctx* c, int n_worlds, bool windows, cudaStream_t s);
 // batched worlds: one tiled-epilogue launch over n_worlds (grid z), pointer lists in EpiParams
 bool epilogue_batch_supported(const EpiParams& p);
 // br: rows per thread of the one-kernel tiled epilogue (1, 2 or 4)

@@ -1008,6 +1008,19 @@ double tile_choose(TileParams* p, int H, int W, const int* kcount, int R, int n_
     return best;
 }
 
+void tile_choose_kpb(TileParams* p, const int* kcount, int n_worlds)
+{
+    int kmax = 0;
+    for (int c = 0; c < kMaxChannels; c++) kmax = kcount[c] > kmax ? kcount[c] : kmax;
+    double best = INFINITY;
+    for (int kpb = 1; kpb <= kmax; kpb++) {
+        const double t = tile_cost(*p, kcount, kpb, n_worlds);
+        if (t >= best) continue;
+        best = t;
+        p->kpb = kpb;
+    }
+}
+
 double fft_passes_cost(int H, int W, int planes) { return 9.0 + 2.6e-6 * H * W * planes; }
 
 double direct_cost(int H, int W, int planes, int R)

@@ -397,3 +397,55 @@ def test_split_step_decides_as_the_step(z, on_windows, n_channels):
         assert torch.equal(P1 != 0, P2 != 0)
     finally:
         lenia.lenia_destroy(ctx)
+
+
+def _alone(w, n_steps):
+    torch = torch_mod()
+    cfg, ks = lenia.config_from_world(w)
+    ctx = lenia.lenia_init(cfg, ks)
+    A, P = to_dev(w.A), to_dev(w.P) if w.n_planes else None
+    for _ in range(n_steps):
+        A2, P2 = torch.empty_like(A), torch.empty_like(P) if w.n_planes else None
+        lenia.lenia_step(ctx, A, P, A2, P2)
+        A, P = A2, P2
+    torch.cuda.synchronize()
+    lenia.lenia_destroy(ctx)
+    return A, P
+
+
+@pytest.mark.parametrize("side,radii", [(64, (9, 13, 18)), (128, (9, 13, 20, 25)), (256, (9, 13)), (256, (18, 25, 13))])
+@pytest.mark.parametrize("kind", ["one", "global", "local"])
+@pytest.mark.parametrize("autotune", [0, 1])
+def test_groups_of_worlds_equal_single_steps(side, radii, kind, autotune):
+    """Grouped worlds of one size and several radii (so of several window sizes): bit for
+    bit what each is on its own, and to the step's tolerance at widths of 256 k."""
+    torch = torch_mod()
+    ws = []
+    for i, R in enumerate(radii):
+        if kind == "one":
+            w = inputs.single_kernel_global(H=side, W=side, R=R, patch=side // 2, sigma=0.05, mu=0.42)
+            w.A = inputs.random_field(100 * side + i, w.A.shape)
+        elif kind == "global":
+            w = inputs.global_multi_channel(H=side, W=side, R=R, patch=side // 2)
+            w.A = inputs.random_field(100 * side + i, w.A.shape)
+        else:
+            w = inputs.multi_channel(H=side, W=side, R=R, patch=side // 4, n_geno=3, matched=True, seed_index=60 + i)
+        ws.append(w)
+    if kind != "one":        # one topology and one set of global genes, so that they group
+        for w in ws[1:]:
+            for k, k0 in zip(w.kernels, ws[0].kernels):
+                k.h, k.mu, k.sigma = k0.h, k0.mu, k0.sigma
+    b = lenia.lenia_batch_init(ws, autotune=bool(autotune))
+    try:
+        assert all(lenia.lenia_batch_group_of(b, i) == 0 for i in range(len(ws)))
+        A = [to_dev(w.A) for w in ws]
+        P = [to_dev(w.P) if w.n_planes else None for w in ws]
+        lenia.lenia_batch_rollout(b, A, P, 3)
+        lenia.lenia_batch_check(b)
+        for i, w in enumerate(ws):
+            A1, P1 = _alone(w, 3)
+            if side % 256:
+                assert torch.equal(A[i], A1) and (P1 is None or torch.equal(P[i], P1))
+            assert float((A[i] - A1).abs().max()) <= 3e-5
+    finally:
+        lenia.lenia_batch_destroy(b)
