@@ -188,8 +188,9 @@ LENIA_API lenia_status lenia_step(lenia_ctx* ctx, const float* A_in, const float
  * in one thread-block cluster of 16 (or 8) blocks that keep the world in
  * shared memory and meet at the cluster barrier: dense (2R+1)^2 sums in
  * another order, equal to repeated lenia_step calls to FP32 rounding.
- * One-channel worlds of 64^2 or 128^2 sites with global genes and at most four
- * kernels on the FFT path run such a rollout in one thread block that keeps the
+ * One-channel worlds with global genes on the FFT path, of 64^2 sites with at
+ * most four kernels or 128^2 with at most three, run such a rollout (128^2 with
+ * several kernels: from four steps on) in one thread block that keeps the
  * world in registers and transforms it in shared memory; equal to repeated
  * lenia_step calls to FP32 rounding.
  * lenia_rollout_route tells which form a context uses. */

@@ -56,12 +56,16 @@ struct lenia_ctx {
     // faster than the path's other form
     bool tile = false;
     TileParams tl;
-    bool block = false;                    // rollouts in one block (the torus is one window)
+    bool block = false;                    // rollouts in one block (the torus is one window: bt)
+    TileParams bt;
     bool gate_pays = false;                // more windows than run at once: skipping some saves time
     GuardParams guard = {};                // how far the windows' and the direct sums' potentials may be apart
     float* d_tS = nullptr;
     float* d_tS0 = nullptr;
     float2* d_ttw = nullptr;
+    float* d_bS = nullptr;
+    float* d_bS0 = nullptr;
+    float2* d_btw = nullptr;
     float* d_S = nullptr;
     float2* d_twM = nullptr;
     float2* d_twW = nullptr;
@@ -423,18 +427,19 @@ GuardParams window_guard(const lenia_ctx* c)
     return g;
 }
 
-// Spectra and twiddles of the context's windows (c->tl.N).  Waits for the work.
-lenia_status build_tiles(lenia_ctx* c, cudaStream_t s)
+// Spectra and twiddles of windows of tl's size, in buffers of the context (replaced).
+// Waits for the work.
+lenia_status build_tiles(lenia_ctx* c, TileParams* tl, float** S, float** S0, float2** tws, cudaStream_t s)
 {
-    const int n = c->tl.N, ca = n / 8, NC = (int)c->conv_w.size();
+    const int n = tl->N, ca = n / 8, NC = (int)c->conv_w.size();
     const size_t ns = tile_spectrum_floats(n), hs = (size_t)(n / 2 + 1) * (n / 2 + 1);
-    for (void* q : {(void*)c->d_tS, (void*)c->d_tS0, (void*)c->d_ttw})
+    for (void* q : {(void*)*S, (void*)*S0, (void*)*tws})
         if (q) cudaFree(q);
-    c->d_tS = c->d_tS0 = nullptr;
-    c->d_ttw = nullptr;
-    lenia_status st = dalloc(c, &c->d_tS, ns * NC);
-    if (st == LENIA_OK) st = dalloc(c, &c->d_tS0, (size_t)n * NC);
-    if (st == LENIA_OK) st = dalloc(c, &c->d_ttw, (size_t)n);
+    *S = *S0 = nullptr;
+    *tws = nullptr;
+    lenia_status st = dalloc(c, S, ns * NC);
+    if (st == LENIA_OK) st = dalloc(c, S0, (size_t)n * NC);
+    if (st == LENIA_OK) st = dalloc(c, tws, (size_t)n);
     float* d_tmp = nullptr;
     if (st == LENIA_OK) st = dalloc(c, &d_tmp, hs * NC);
     if (st != LENIA_OK) return st;
@@ -444,17 +449,21 @@ lenia_status build_tiles(lenia_ctx* c, cudaStream_t s)
             const double a = kTwoPi * n1 * b / n;
             tw[b * ca + n1] = make_float2((float)cos(a), (float)-sin(a));
         }
-    cudaError_t e = cudaMemcpy(c->d_ttw, tw.data(), n * sizeof(float2), cudaMemcpyHostToDevice);
+    cudaError_t e = cudaMemcpy(*tws, tw.data(), n * sizeof(float2), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = build_spectra(c, n, n, d_tmp, s);
     for (int k = 0; k < NC && e == cudaSuccess; k++)
-        e = launch_tile_spectra(n, d_tmp + hs * k, c->d_tS + ns * k, c->d_tS0 + (size_t)n * k, s);
+        e = launch_tile_spectra(n, d_tmp + hs * k, *S + ns * k, *S0 + (size_t)n * k, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     cudaFree(d_tmp);
     if (e != cudaSuccess) return fail(c, LENIA_ECUDA, std::string("window spectra: ") + cudaGetErrorString(e));
-    c->tl.S = c->d_tS;
-    c->tl.S0 = c->d_tS0;
-    c->tl.tw = c->d_ttw;
+    tl->S = *S;
+    tl->S0 = *S0;
+    tl->tw = *tws;
     return LENIA_OK;
+}
+lenia_status build_tiles(lenia_ctx* c, cudaStream_t s)
+{
+    return build_tiles(c, &c->tl, &c->d_tS, &c->d_tS0, &c->d_ttw, s);
 }
 
 // The FFT path's three passes: spectra, twiddles and intermediate planes, unless the
@@ -862,7 +871,7 @@ void lenia_destroy(lenia_ctx* c)
                     c->d_Useg, c->d_hA_in1, c->d_hP_in1, c->d_hA_out1,
                     c->d_hP_out1, c->d_hstats, c->d_tc_hi, c->d_tc_lo, c->d_tc_B, c->d_tc_ks,
                     c->d_tc_grp, c->d_tc_has, c->d_small_count, c->d_taps, c->d_cr_w, c->d_tS, c->d_tS0,
-                    c->d_ttw};
+                    c->d_ttw, c->d_bS, c->d_bS0, c->d_btw};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
@@ -1049,14 +1058,11 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
         const double t_tile = tile_choose(&c->tl, H, W, kcount, c->max_R, 1, cfg->maintain_genes != 0);
         const double t_else = path == LENIA_CONV_FFT ? fft_passes_cost(H, W, C + NC) : direct_cost(H, W, NC, c->max_R);
         c->tile = t_tile < t_else;
-        // one-channel worlds of one window: whole rollouts in one block, so the
-        // window is the torus whatever a single step would take
-        c->block = path == LENIA_CONV_FFT && c->n_p == 0 && !n_rings && tile_rollout_supported(H, W, C, K) &&
-                   tile_plan(&c->tl, H, H, W, c->max_R);
-        if (c->block) {
-            c->tl.kpb = NC;
-            c->tile = true;
-        }
+        // one-channel worlds of one window: whole rollouts in one block, whatever a single
+        // step takes
+        memset(&c->bt, 0, sizeof(c->bt));
+        c->block = path == LENIA_CONV_FFT && c->n_p == 0 && !n_rings && tile_rollout_steps(H, W, C, K) &&
+                   tile_plan(&c->bt, H, H, W, c->max_R);
     }
     if (want_adj && c->tile) {
         const double t_win = tile_adj_cost(c->tl, kcount), t_pl = tile_planes_cost(c->tl, K);
@@ -1078,6 +1084,21 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
         memcpy(c->tl.kcount, kcount, sizeof(kcount));
         memcpy(c->tl.klist, klist, sizeof(klist));
         const lenia_status ts = build_tiles(c, s);
+        if (ts != LENIA_OK) {
+            fprintf(stderr, "lenia_init: %s\n", c->err.c_str());
+            lenia_destroy(c);
+            return ts;
+        }
+    }
+    if (c->block) {
+        lenia_status ts = LENIA_OK;
+        if (c->tile && c->tl.N == c->bt.N) {
+            c->bt.S = c->tl.S;
+            c->bt.S0 = c->tl.S0;
+            c->bt.tw = c->tl.tw;
+        } else {
+            ts = build_tiles(c, &c->bt, &c->d_bS, &c->d_bS0, &c->d_btw, s);
+        }
         if (ts != LENIA_OK) {
             fprintf(stderr, "lenia_init: %s\n", c->err.c_str());
             lenia_destroy(c);
@@ -1412,13 +1433,14 @@ lenia_status lenia_rollout(lenia_ctx* c, float* A, float* P, int32_t n_steps, fl
         CUDA_OR_FAIL(c, launch_cluster_rollout(cp, s));
         return LENIA_OK;
     }
-    if (c->block && !stats_out && n_steps >= 2) {
+    if (c->block && !stats_out &&
+        n_steps >= tile_rollout_steps(c->cfg.height, c->cfg.width, c->cfg.n_channels, c->cfg.n_kernels)) {
         TileRolloutParams tp;
         memset(&tp, 0, sizeof(tp));
         tp.A = A;
-        tp.S = c->d_tS;
-        tp.S0 = c->d_tS0;
-        tp.tw = c->d_ttw;
+        tp.S = c->bt.S;
+        tp.S0 = c->bt.S0;
+        tp.tw = c->bt.tw;
         tp.K = c->cfg.n_kernels;
         tp.n_steps = n_steps;
         tp.growth_form = c->cfg.growth_form;
@@ -1429,7 +1451,7 @@ lenia_status lenia_rollout(lenia_ctx* c, float* A, float* P, int32_t n_steps, fl
             tp.h[k] = c->kt.h[k];
         }
         ProfScope ps(c, KIND_COLS, s);
-        CUDA_OR_FAIL(c, launch_tile_rollout(tp, c->tl.N, s));
+        CUDA_OR_FAIL(c, launch_tile_rollout(tp, c->bt.N, s));
         return LENIA_OK;
     }
     if (c->small && !stats_out && n_steps >= 2) {

@@ -342,7 +342,7 @@ cudaError_t launch_tile_conv(const TileParams& p, cudaStream_t s);
 cudaError_t launch_tile_conv_adj(const TileParams& p, cudaStream_t s);
 
 // Rollouts of one-channel worlds with global genes whose torus is one window (64^2
-// or 128^2, at most kTileRolloutKernels kernels), in one block.
+// or 128^2), in one block.
 constexpr int kTileRolloutKernels = 4;
 struct TileRolloutParams {
     float* A;                  // [N][N], in and out
@@ -353,7 +353,8 @@ struct TileRolloutParams {
     float dt;
     float mu[kTileRolloutKernels], rsigma[kTileRolloutKernels], h[kTileRolloutKernels];
 };
-bool tile_rollout_supported(int H, int W, int C, int K);
+// the fewest steps that such a rollout takes in one block, or 0 where none does
+int tile_rollout_steps(int H, int W, int C, int K);
 cudaError_t launch_tile_rollout(const TileRolloutParams& p, int N, cudaStream_t s);
 
 // Adjoint of one step with global genes.

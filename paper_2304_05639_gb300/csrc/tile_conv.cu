@@ -1037,7 +1037,18 @@ cudaError_t launch_tile_conv(const TileParams& p0, cudaStream_t s)
     return p.N == 128 ? launch_n<128, false>(p, s) : launch_n<64, false>(p, s);
 }
 
-bool tile_rollout_supported(int H, int W, int C, int K) { return H == W && (H == 64 || H == 128) && C == 1 && K <= kTileRolloutKernels; }
+// Where one block pays (us for 2 / 6 / 16 steps against the same steps as launches):
+//   64^2   one kernel 9 / 13 / 30 against 17 / 56 / 148, four 14 / 34 / 83 against 17 /
+//          50 / 132
+//   128^2  one kernel 17 / 41 / 102 against 17 / 50 / 132, three 36 / 95 / 244 against
+//          17 / 56 / 148 (32 / 99 / 263 with the FFT passes), four 43 / 118 / 306 (35 /
+//          111 / 295 with the passes)
+int tile_rollout_steps(int H, int W, int C, int K)
+{
+    if (H != W || C != 1) return 0;
+    if (H == 64) return K <= kTileRolloutKernels ? 2 : 0;
+    return H == 128 && K <= 3 ? (K == 1 ? 2 : 4) : 0;
+}
 
 template <int N, bool ONE>
 static cudaError_t launch_rollout_n(const TileRolloutParams& p, cudaStream_t s)

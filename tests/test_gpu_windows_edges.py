@@ -449,3 +449,33 @@ def test_groups_of_worlds_equal_single_steps(side, radii, kind, autotune):
             assert float((A[i] - A1).abs().max()) <= 3e-5
     finally:
         lenia.lenia_batch_destroy(b)
+
+
+@pytest.mark.parametrize("side,n_kernels,route", [(64, 4, lenia.ROUTE_BLOCK), (128, 1, lenia.ROUTE_BLOCK),
+                                                  (128, 4, lenia.ROUTE_STEPS), (64, 5, lenia.ROUTE_STEPS)])
+def test_small_one_channel_worlds_step_as_they_roll(side, n_kernels, route):
+    """Steps with statistics, potentials and rollouts of 2 to 6 steps of the worlds around
+    the one-block rollout's limits, against the oracle's steps."""
+    torch = torch_mod()
+    w = inputs.single_kernel_global(H=side, W=side, R=13, patch=side, sigma=0.05, mu=0.42)
+    w.kernels = [inputs.KernelDesc(0, 0, 13 - i, inputs.KERNEL_SHELLS, (1.0,), h=1.0 - 0.15 * i, mu=0.42 + 0.02 * i,
+                                   sigma=0.05 + 0.01 * i) for i in range(n_kernels)]
+    U = gpu_potentials(w)[0]
+    ref = np.stack([oracle.potential(w.A[k.src], K) for k, K in zip(w.kernels, oracle.world_kernels(w))])
+    assert np.abs(U - ref).max() <= TOL_U
+    cfg, ks = lenia.config_from_world(w)
+    ctx = lenia.lenia_init(cfg, ks)
+    try:
+        assert lenia.lenia_rollout_route(ctx) == route
+        for n in (2, 3, 6):
+            A, st = to_dev(w.A), torch.zeros((n, 1, 3), device="cuda")
+            B = A.clone()
+            lenia.lenia_rollout(ctx, A, None, n)
+            lenia.lenia_rollout(ctx, B, None, n, st)
+            torch.cuda.synchronize()
+            want = oracle.rollout(w, n)[0]
+            assert np.abs(A.cpu().numpy() - want).max() <= n * 1e-5
+            assert np.abs(B.cpu().numpy() - want).max() <= n * 1e-5
+            np.testing.assert_allclose(st[n - 1].cpu().numpy(), oracle.stats(B.cpu().numpy()), rtol=1e-5)
+    finally:
+        lenia.lenia_destroy(ctx)
