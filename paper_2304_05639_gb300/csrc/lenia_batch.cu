@@ -98,8 +98,9 @@ lenia_status bfail(const char* msg)
     return LENIA_EINVAL;
 }
 
-// Time `reps` steps of a fresh context with the given path on zero-filled
-// state (the arithmetic does not depend on the values).
+// Time six steps of a fresh context with the given path on zero-filled state (the
+// arithmetic does not depend on the values): lenia_step, as the batch runs worlds
+// (lenia_rollout may take forms of its own, in one launch).
 float time_path(const lenia_config& cfg0, const lenia_kernel_desc* ks, int path, cudaStream_t s)
 {
     lenia_config cfg = cfg0;
@@ -109,25 +110,32 @@ float time_path(const lenia_config& cfg0, const lenia_kernel_desc* ks, int path,
     if (lenia_init(&cfg, ks, s, &c) != LENIA_OK) return INFINITY;
     const size_t N = (size_t)cfg.height * cfg.width;
     const int n_p = ((cfg.localized & 1) != 0) + ((cfg.localized & 2) != 0) + ((cfg.localized & 4) != 0);
-    float *A = nullptr, *P = nullptr;
+    float *A[2] = {nullptr, nullptr}, *P[2] = {nullptr, nullptr};
     float ms = INFINITY;
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    if (cudaMalloc(&A, N * cfg.n_channels * sizeof(float)) == cudaSuccess &&
-        (n_p == 0 || cudaMalloc(&P, N * n_p * cfg.n_kernels * sizeof(float)) == cudaSuccess)) {
-        cudaMemsetAsync(A, 0, N * cfg.n_channels * sizeof(float), s);
-        if (P) cudaMemsetAsync(P, 0, N * n_p * cfg.n_kernels * sizeof(float), s);
-        bool ok = lenia_rollout(c, A, P, 2, nullptr, s) == LENIA_OK;    // warm-up
-        cudaEventRecord(e0, s);
-        ok = ok && lenia_rollout(c, A, P, 6, nullptr, s) == LENIA_OK;
-        cudaEventRecord(e1, s);
-        if (ok && cudaEventSynchronize(e1) == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
+    bool ok = true;
+    for (int b = 0; b < 2 && ok; b++) {
+        const size_t na = N * cfg.n_channels * sizeof(float), np = N * n_p * cfg.n_kernels * sizeof(float);
+        ok = cudaMalloc(&A[b], na) == cudaSuccess && (n_p == 0 || cudaMalloc(&P[b], np) == cudaSuccess);
+        if (ok) cudaMemsetAsync(A[b], 0, na, s);
+        if (ok && P[b]) cudaMemsetAsync(P[b], 0, np, s);
     }
+    auto steps = [&](int n) {
+        for (int t = 0; t < n && ok; t++) ok = lenia_step(c, A[t & 1], P[t & 1], A[~t & 1], P[~t & 1], nullptr, s) == LENIA_OK;
+    };
+    steps(2);                                                            // warm-up
+    cudaEventRecord(e0, s);
+    steps(6);
+    cudaEventRecord(e1, s);
+    if (ok && cudaEventSynchronize(e1) == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (A) cudaFree(A);
-    if (P) cudaFree(P);
+    for (int b = 0; b < 2; b++) {
+        if (A[b]) cudaFree(A[b]);
+        if (P[b]) cudaFree(P[b]);
+    }
     lenia_destroy(c);
     return ms;
 }
