@@ -98,6 +98,13 @@ lenia_status bfail(const char* msg)
     return LENIA_EINVAL;
 }
 
+// Planes of P per kernel: the localized growth genes, and the six kernel genes of a ring world.
+int gene_planes(int localized)
+{
+    return ((localized & LENIA_LOC_MU) != 0) + ((localized & LENIA_LOC_SIGMA) != 0) + ((localized & LENIA_LOC_H) != 0) +
+           (localized & LENIA_LOC_KERNEL ? 6 : 0);
+}
+
 // Time six steps of a fresh context with the given path on zero-filled state (the
 // arithmetic does not depend on the values): lenia_step, as the batch runs worlds
 // (lenia_rollout may take forms of its own, in one launch).
@@ -109,7 +116,7 @@ float time_path(const lenia_config& cfg0, const lenia_kernel_desc* ks, int path,
     lenia_ctx* c = nullptr;
     if (lenia_init(&cfg, ks, s, &c) != LENIA_OK) return INFINITY;
     const size_t N = (size_t)cfg.height * cfg.width;
-    const int n_p = ((cfg.localized & 1) != 0) + ((cfg.localized & 2) != 0) + ((cfg.localized & 4) != 0);
+    const int n_p = gene_planes(cfg.localized);
     float *A[2] = {nullptr, nullptr}, *P[2] = {nullptr, nullptr};
     float ms = INFINITY;
     cudaEvent_t e0, e1;
@@ -463,7 +470,7 @@ lenia_status lenia_batch_init(int32_t n_worlds, const lenia_config* cfgs, const 
         }
         b->ctx.push_back(c);
         const size_t N = (size_t)cfg.height * cfg.width;
-        const int n_p = ((cfg.localized & 1) != 0) + ((cfg.localized & 2) != 0) + ((cfg.localized & 4) != 0);
+        const int n_p = gene_planes(cfg.localized);
         b->abytes.push_back(N * cfg.n_channels * sizeof(float));
         b->pbytes.push_back(N * n_p * cfg.n_kernels * sizeof(float));
         float *a2 = nullptr, *p2 = nullptr;

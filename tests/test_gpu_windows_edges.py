@@ -479,3 +479,31 @@ def test_small_one_channel_worlds_step_as_they_roll(side, n_kernels, route):
             np.testing.assert_allclose(st[n - 1].cpu().numpy(), oracle.stats(B.cpu().numpy()), rtol=1e-5)
     finally:
         lenia.lenia_destroy(ctx)
+
+
+@pytest.mark.parametrize("autotune", [0, 1])
+def test_ring_worlds_in_a_batch(autotune):
+    """The batch's second state holds a ring world's kernel genes too (nine planes a
+    kernel): bit for bit the steps of the world on its own."""
+    torch = torch_mod()
+    ws = [inputs.ring_world(H=64, W=64, R=6, n_rings=12, patch=24, n_geno=2) for _ in range(2)]
+    ws.append(inputs.single_kernel_global(H=64, W=64, R=9, patch=32))
+    b = lenia.lenia_batch_init(ws, autotune=bool(autotune), conv_path=lenia.CONV_AUTO)
+    try:
+        A = [to_dev(w.A) for w in ws]
+        P = [to_dev(w.P) if w.n_planes else None for w in ws]
+        lenia.lenia_batch_rollout(b, A, P, 3)
+        lenia.lenia_batch_check(b)
+        for i in (0, 1):
+            cfg, ks = lenia.config_from_world(ws[i], lenia.lenia_batch_conv_path(b, i))
+            ctx = lenia.lenia_init(cfg, ks)
+            A1, P1 = to_dev(ws[i].A), to_dev(ws[i].P)
+            for _ in range(3):
+                A2, P2 = torch.empty_like(A1), torch.empty_like(P1)
+                lenia.lenia_step(ctx, A1, P1, A2, P2)
+                A1, P1 = A2, P2
+            torch.cuda.synchronize()
+            lenia.lenia_destroy(ctx)
+            assert torch.equal(A[i], A1) and torch.equal(P[i], P1)
+    finally:
+        lenia.lenia_batch_destroy(b)
