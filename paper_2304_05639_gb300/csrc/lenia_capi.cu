@@ -793,6 +793,7 @@ double ctx_group_cost(const lenia_ctx* c, int n_worlds)
     for (int src : c->conv_src) kcount[src]++;
     TileParams tl;
     memset(&tl, 0, sizeof(tl));
+    tl.n_sms = c->num_sms;
     return tile_choose(&tl, c->cfg.height, c->cfg.width, kcount, c->max_R, n_worlds);
 }
 
@@ -805,6 +806,7 @@ cudaError_t ctx_group_form(lenia_ctx* c, int n_worlds, bool windows, cudaStream_
     }
     const int n = c->tile ? c->tl.N : 0;
     if (!c->tile) memset(&c->tl, 0, sizeof(c->tl));
+    c->tl.n_sms = c->num_sms;
     c->tile = true;
     c->tl.C = c->cfg.n_channels;
     memset(c->tl.kcount, 0, sizeof(c->tl.kcount));
@@ -1055,6 +1057,7 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
          (!cfg->maintain_genes || (epilogue_sites_supported(epi_params(c)) &&
                                    !(cfg->alpha_on && fabsf(cfg->eps_u) < std::max(1e-4f, 2.f * K * c->guard.du)))))) {
         memset(&c->tl, 0, sizeof(c->tl));
+        c->tl.n_sms = c->num_sms;
         const double t_tile = tile_choose(&c->tl, H, W, kcount, c->max_R, 1, cfg->maintain_genes != 0);
         const double t_else = path == LENIA_CONV_FFT ? fft_passes_cost(H, W, C + NC) : direct_cost(H, W, NC, c->max_R);
         c->tile = t_tile < t_else;

@@ -294,6 +294,7 @@ struct TileParams {
     const float* S0;           // [K][N] mirrored share of the packed column 0
     const float2* tw;          // [8][N / 8] exp(-2 pi i n1 b / N)
     int N, H, W, C;
+    int n_sms;                 // of the device, for the launch's and the models' choices
     TileGeom g;
     // worlds batched in one launch (grid y: world * C + channel), or null; every
     // window count is at most `tiles`

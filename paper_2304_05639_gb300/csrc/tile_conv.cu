@@ -898,10 +898,10 @@ cudaError_t launch_nt(const TileParams& p, const dim3& grid, cudaStream_t s)
 // that work are few again (N = 128, 1080 x 1920 15 kernels, a quarter live:
 // 66 / 52; 2048^2, 28% live: 112 / 106).  The transposed sum of N = 128 would
 // spill at 4 N threads.
-bool wide_block(int N, double blocks, bool gated, bool adj)
+bool wide_block(int N, int n_sms, double blocks, bool gated, bool adj)
 {
     if (N == 128 && adj) return false;
-    return blocks <= 2 * 152 || (N == 128 && gated);
+    return blocks <= 2.0 * n_sms || (N == 128 && gated);
 }
 
 template <int N, bool ADJ>
@@ -910,7 +910,7 @@ cudaError_t launch_n(const TileParams& p, cudaStream_t s)
     const dim3 grid = conv_grid(p, ADJ);
     if (grid.z == 0) return cudaSuccess;
     if constexpr (!(N == 128 && ADJ)) {
-        if (wide_block(N, (double)grid.x * grid.y * grid.z, p.gate != nullptr, ADJ)) return launch_nt<N, 4 * N, ADJ>(p, grid, s);
+        if (wide_block(N, p.n_sms, (double)grid.x * grid.y * grid.z, p.gate != nullptr, ADJ)) return launch_nt<N, 4 * N, ADJ>(p, grid, s);
     }
     return launch_nt<N, 2 * N, ADJ>(p, grid, s);
 }
@@ -952,8 +952,8 @@ bool tile_plan(TileParams* p, int N, int H, int W, int R)
 // unit takes t1 on an idle SM and tf with every block slot of the SM taken.
 static double tile_time(const TileParams& p, double blocks, double units, bool adj)
 {
-    const bool wide = wide_block(p.N, blocks, false, adj);
-    const double slots = 152.0 * (wide ? 2 : p.N == 128 ? 3 : 8);
+    const bool wide = wide_block(p.N, p.n_sms, blocks, false, adj);
+    const double slots = (double)p.n_sms * (wide ? 2 : p.N == 128 ? 3 : 8);
     const double t1 = p.N == 128 ? (wide ? 2.0 : 2.3) : wide ? 0.6 : 0.9;
     const double tf = p.N == 128 ? (wide ? 3.8 : 7.7) : wide ? 2.2 : 4.2;
     const double waves = blocks / slots, whole = floor(waves), rest = waves - whole;
