@@ -457,9 +457,13 @@ def test_small_one_channel_worlds_step_as_they_roll(side, n_kernels, route):
     """Steps with statistics, potentials and rollouts of 2 to 6 steps of the worlds around
     the one-block rollout's limits, against the oracle's steps."""
     torch = torch_mod()
-    w = inputs.single_kernel_global(H=side, W=side, R=13, patch=side, sigma=0.05, mu=0.42)
+    w = inputs.single_kernel_global(H=side, W=side, R=13, patch=side, sigma=0.2, mu=0.42)
     w.kernels = [inputs.KernelDesc(0, 0, 13 - i, inputs.KERNEL_SHELLS, (1.0,), h=1.0 - 0.15 * i, mu=0.42 + 0.02 * i,
-                                   sigma=0.05 + 0.01 * i) for i in range(n_kernels)]
+                                   sigma=0.2 + 0.01 * i) for i in range(n_kernels)]
+    w.dt = 0.02
+    # a step passes an error on by at most L, the steepest growth's share
+    L = 1 + w.dt * sum(2 * k.h * np.exp(-0.5) / k.sigma for k in w.kernels)
+    tol = lambda n: 1e-5 * (L**n - 1) / (L - 1)
     U = gpu_potentials(w)[0]
     ref = np.stack([oracle.potential(w.A[k.src], K) for k, K in zip(w.kernels, oracle.world_kernels(w))])
     assert np.abs(U - ref).max() <= TOL_U
@@ -474,8 +478,8 @@ def test_small_one_channel_worlds_step_as_they_roll(side, n_kernels, route):
             lenia.lenia_rollout(ctx, B, None, n, st)
             torch.cuda.synchronize()
             want = oracle.rollout(w, n)[0]
-            assert np.abs(A.cpu().numpy() - want).max() <= n * 1e-5
-            assert np.abs(B.cpu().numpy() - want).max() <= n * 1e-5
+            assert np.abs(A.cpu().numpy() - want).max() <= tol(n)
+            assert np.abs(B.cpu().numpy() - want).max() <= tol(n)
             np.testing.assert_allclose(st[n - 1].cpu().numpy(), oracle.stats(B.cpu().numpy()), rtol=1e-5)
     finally:
         lenia.lenia_destroy(ctx)
