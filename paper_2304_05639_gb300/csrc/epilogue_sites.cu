@@ -133,49 +133,65 @@ __device__ __forceinline__ int tap_site(int2 tap, int y, int x, int H, int W)
 }
 
 // Kernel k's direct sum at (y, x): its non-zero taps in k_direct_conv's order (a zero
-// weight adds nothing there), so the same bits.  By a whole warp: the lanes load
-// 4 x 32 taps at once, the next ones while every lane adds these in order.  (This and
-// the code around it runs at a few sites a step, so it is kept small: what it costs
-// there is its latency, instruction fetches among it.)
-__device__ __forceinline__ float direct_warp(const SitesParams& q, const float* A, int k, int y, int x)
+// weight adds nothing there), so the same bits.  By a whole warp: the lanes fetch 128
+// taps at once, the next ones while every lane adds these, in order, from shared
+// memory (sm: the warp's).  What it costs is its latency: 436 taps of R = 12 took
+// 14000 cycles with the operands passed round by shuffles.
+constexpr int ES_TAPS = 128;
+__device__ __forceinline__ float direct_warp(const SitesParams& q, const float* A, int k, int y, int x, float2* sm)
 {
-    constexpr int B = 4;
+    constexpr int B = ES_TAPS / 32;
     const int H = q.e.H, W = q.e.W, lane = threadIdx.x & 31;
     const float* plane = A + (size_t)q.e.kt.src[k] * H * W;
     const int t1 = q.g.off[k + 1];
-    float vn[B], wn[B];
-    auto fetch = [&](int t0) {
+    // taps a batch ahead of their values, values a batch ahead of their sums
+    int2 tap[B];
+    float2 next[B];
+    auto fetch_taps = [&](int t0) {
 #pragma unroll
         for (int j = 0; j < B; j++) {
             const int t = t0 + 32 * j + lane;
-            const int2 tap = t < t1 ? __ldg(&q.g.taps[t]) : make_int2((1024 << 11) + 1024, 0);
-            wn[j] = __int_as_float(tap.y);
-            vn[j] = t < t1 ? __ldg(&plane[tap_site(tap, y, x, H, W)]) : 0.f;
+            tap[j] = t < t1 ? __ldg(&q.g.taps[t]) : make_int2((1024 << 11) + 1024, 0);
         }
     };
+    auto fetch_values = [&]() {                // (beyond t1: the site itself by 0)
+#pragma unroll
+        for (int j = 0; j < B; j++)
+            next[j] = make_float2(__int_as_float(tap[j].y), __ldg(&plane[tap_site(tap[j], y, x, H, W)]));
+    };
     float acc = 0.f;
-    fetch(q.g.off[k]);
+    fetch_taps(q.g.off[k]);
+    fetch_values();
+    fetch_taps(q.g.off[k] + ES_TAPS);
 #pragma unroll 1
-    for (int t0 = q.g.off[k]; t0 < t1; t0 += 32 * B) {
-        float v[B], w[B];
+    for (int t0 = q.g.off[k]; t0 < t1; t0 += ES_TAPS) {
 #pragma unroll
-        for (int j = 0; j < B; j++) v[j] = vn[j], w[j] = wn[j];
-        fetch(t0 + 32 * B);
+        for (int j = 0; j < B; j++) sm[32 * j + lane] = next[j];
+        __syncwarp();
+        fetch_values();
+        fetch_taps(t0 + 2 * ES_TAPS);
+        const float2* e = sm;
+        const int n = min(ES_TAPS, t1 - t0);
+        int i = 0;
+#pragma unroll 1
+        for (; i + 16 <= n; i += 16) {
+            float4 f[8];
 #pragma unroll
-        for (int j = 0; j < B; j++) {
-            if (t0 + 32 * j >= t1) break;
-#pragma unroll 8
-            for (int i = 0; i < 32; i++)       // (beyond t1: 0 x 0)
-                acc = fmaf(__shfl_sync(0xffffffffu, w[j], i), __shfl_sync(0xffffffffu, v[j], i), acc);
+            for (int j = 0; j < 8; j++) f[j] = reinterpret_cast<const float4*>(e + i)[j];
+#pragma unroll
+            for (int j = 0; j < 8; j++) acc = fmaf(f[j].z, f[j].w, fmaf(f[j].x, f[j].y, acc));
         }
+#pragma unroll 1
+        for (; i < n; i++) acc = fmaf(e[i].x, e[i].y, acc);
+        __syncwarp();
     }
     return acc;
 }
 
 // The direct sums of the lanes that want one (the whole warp calls it).  Up to four
 // sites take the warp one after the other; more go side by side, a lane each
-// (a sum's additions are one chain), the lanes passing the taps round.
-__device__ __forceinline__ float direct_sums(const SitesParams& q, const float* A, int k, int y, int x, bool want)
+// (a sum's additions are one chain), the taps read from shared memory.
+__device__ __forceinline__ float direct_sums(const SitesParams& q, const float* A, int k, int y, int x, bool want, float2* sm)
 {
     constexpr int B = 8;
     const int H = q.e.H, W = q.e.W, lane = threadIdx.x & 31, R = q.g.R;
@@ -186,12 +202,11 @@ __device__ __forceinline__ float direct_sums(const SitesParams& q, const float* 
 #pragma unroll 1
         for (; m; m &= m - 1) {
             const int L = __ffs(m) - 1;
-            const float s = direct_warp(q, A, k, __shfl_sync(0xffffffffu, y, L), __shfl_sync(0xffffffffu, x, L));
+            const float s = direct_warp(q, A, k, __shfl_sync(0xffffffffu, y, L), __shfl_sync(0xffffffffu, x, L), sm);
             if (lane == L) acc = s;
         }
         return acc;
     }
-    if (q.g.off[k] == t1) return 0.f;
     // the other lanes read along at the first site
     const int L = __ffs(m) - 1, y0 = __shfl_sync(0xffffffffu, y, L), x0 = __shfl_sync(0xffffffffu, x, L);
     if (!want) {
@@ -201,30 +216,34 @@ __device__ __forceinline__ float direct_sums(const SitesParams& q, const float* 
     const bool inner = __all_sync(0xffffffffu, y >= R && y < H - R && x >= R && x < W - R);
     const float* plane = A + (size_t)q.e.kt.src[k] * H * W;
     const float* at = plane + (size_t)y * W + x;
-    auto fetch = [&](int t) { return __ldg(&q.g.taps[min(t + lane, t1 - 1)]); };
-    int2 next = fetch(q.g.off[k]);
+    int2 next = make_int2((1024 << 11) + 1024, 0);
+    auto fetch = [&](int t) {
+        if (t + lane < t1) next = __ldg(&q.g.taps[t + lane]);
+    };
+    fetch(q.g.off[k]);
 #pragma unroll 1
     for (int t0 = q.g.off[k]; t0 < t1; t0 += 32) {
-        const int2 tap = next;
-        next = fetch(t0 + 32);
-        const int off = ((tap.x >> 11) - 1024) * W + (tap.x & 2047) - 1024;
+        const int off = ((next.x >> 11) - 1024) * W + (next.x & 2047) - 1024;
+        sm[lane] = make_float2(__int_as_float(inner ? off : next.x), __int_as_float(next.y));
+        __syncwarp();
+        fetch(t0 + 32);
+        const int n = min(32, t1 - t0);
 #pragma unroll 1
-        for (int h = 0; h < 32; h += B) {
+        for (int h = 0; h < n; h += B) {
+            float2 e[B];
             float v[B];
-            if (inner) {
 #pragma unroll
-                for (int j = 0; j < B; j++) v[j] = __ldg(at + __shfl_sync(0xffffffffu, off, h + j));
-            } else {
-#pragma unroll
-                for (int j = 0; j < B; j++)
-                    v[j] = __ldg(plane + tap_site(make_int2(__shfl_sync(0xffffffffu, tap.x, h + j), 0), y, x, H, W));
-            }
+            for (int j = 0; j < B; j++) e[j] = sm[h + j];
 #pragma unroll
             for (int j = 0; j < B; j++) {
-                const float w = __int_as_float(__shfl_sync(0xffffffffu, tap.y, h + j));
-                if (t0 + h + j < t1) acc = fmaf(w, v[j], acc);
+                const int o = __float_as_int(e[j].x);
+                v[j] = inner ? __ldg(at + o) : __ldg(plane + tap_site(make_int2(o, 0), y, x, H, W));
             }
+#pragma unroll
+            for (int j = 0; j < B; j++)
+                if (h + j < n) acc = fmaf(e[j].y, v[j], acc);
         }
+        __syncwarp();
     }
     return acc;
 }
@@ -319,14 +338,18 @@ __device__ __forceinline__ float2 test_range(const SitesParams& q, float u, floa
 
 // Kernel k's diffused genes at one site as the kernel divides them that the shape
 // otherwise takes (the streaming kernel by the hardware reciprocal).
+template <int NP, int RD>
 __device__ __forceinline__ void genes_at(const SitesParams& q, const float* P, int k, int y, int x, float* g)
 {
     const EpiParams& p = q.e;
-    const int H = p.H, W = p.W, RD = p.r_diff;
-    for (int pp = 0; pp < p.n_p; pp++) {
+    const int H = p.H, W = p.W;
+#pragma unroll
+    for (int pp = 0; pp < NP; pp++) {
         const float* pl = P + (size_t)(pp * p.kt.K + k) * H * W;
         float s = 0.f, n = 0.f;
+#pragma unroll
         for (int dy = -RD; dy <= RD; dy++)
+#pragma unroll
             for (int dx = -RD; dx <= RD; dx++) {
                 if (dy * dy + dx * dx > RD * RD) continue;
                 int yy = y + dy, xx = x + dx;
@@ -343,8 +366,9 @@ __device__ __forceinline__ void genes_at(const SitesParams& q, const float* P, i
 
 // alpha's undecided tests, settled, at the sites of the lanes that want it: kernel
 // `first`'s, and the later kernels' where it was not the only one (the whole warp calls it).
+template <int LOC, int RD>
 __device__ __forceinline__ bool alpha_at(const SitesParams& q, const float* A, const float* P, const float* U, int y, int x,
-                                         bool want, int first, bool more)
+                                         bool want, int first, bool more, float2* sm)
 {
     const EpiParams& p = q.e;
     const int W = p.W, K = p.kt.K;
@@ -356,11 +380,9 @@ __device__ __forceinline__ bool alpha_at(const SitesParams& q, const float* A, c
         // the lanes at the warp's lowest kernel go on
         const int kk = __reduce_min_sync(0xffffffffu, ok && k < K ? k : K);
         const bool on = ok && k == kk;
-        float g[3] = {0.f, 0.f, 0.f};
-        if (on) genes_at(q, P, kk, y, x, g);
-        const float m = p.p_mu >= 0 ? g[p.p_mu] : p.kt.mu[kk];
-        const float sg = p.p_sigma >= 0 ? g[p.p_sigma] : p.kt.sigma[kk];
-        const float hh = p.p_h >= 0 ? g[p.p_h] : p.kt.h[kk];
+        float g[3] = {0.f, 0.f, 0.f};          // (mu, sigma and, with LOC 7, h)
+        if (on) genes_at<LOC == 7 ? 3 : 2, RD>(q, P, kk, y, x, g);
+        const float m = g[0], sg = g[1], hh = LOC == 7 ? g[2] : p.kt.h[kk];
         float u = on ? __ldg(&U[(size_t)kk * N + (size_t)y * W + x]) : 0.f;
         float t = settled(q, u, m, sg, hh).y;
         // a lane's first kernel is known to be undecided
@@ -370,7 +392,7 @@ __device__ __forceinline__ bool alpha_at(const SitesParams& q, const float* A, c
             open = on && (kk == first || (r.x < p.eps_u && p.eps_u < r.y));
         }
         if (q.g.du > 0.f && __any_sync(0xffffffffu, open)) {
-            u = direct_sums(q, A, kk, y, x, open);
+            u = direct_sums(q, A, kk, y, x, open, sm);
             if (open) t = settled(q, u, m, sg, hh).y;
         }
         if (on) {
@@ -383,8 +405,9 @@ __device__ __forceinline__ bool alpha_at(const SitesParams& q, const float* A, c
 
 // sum_k of the alpha tests, settled, at the sites of the lanes that want it (a
 // Delta_sum(U) decision near its threshold; the whole warp calls it).
+template <int LOC, int RD>
 __device__ __forceinline__ float tests_at(const SitesParams& q, const float* A, const float* P, const float* U, int y, int x,
-                                       bool want)
+                                       bool want, float2* sm)
 {
     const EpiParams& p = q.e;
     const int W = p.W, K = p.kt.K;
@@ -392,11 +415,9 @@ __device__ __forceinline__ float tests_at(const SitesParams& q, const float* A, 
     float sum = 0.f;
     for (int k = 0; k < K; k++) {
         float g[3] = {0.f, 0.f, 0.f};
-        if (want) genes_at(q, P, k, y, x, g);
-        const float m = p.p_mu >= 0 ? g[p.p_mu] : p.kt.mu[k];
-        const float sg = p.p_sigma >= 0 ? g[p.p_sigma] : p.kt.sigma[k];
-        const float hh = p.p_h >= 0 ? g[p.p_h] : p.kt.h[k];
-        const float u = q.g.du > 0.f ? direct_sums(q, A, k, y, x, want && (sg > 0.f || p.alpha_on))
+        if (want) genes_at<LOC == 7 ? 3 : 2, RD>(q, P, k, y, x, g);
+        const float m = g[0], sg = g[1], hh = LOC == 7 ? g[2] : p.kt.h[k];
+        const float u = q.g.du > 0.f ? direct_sums(q, A, k, y, x, want && (sg > 0.f || p.alpha_on), sm)
                                      : (want ? __ldg(&U[(size_t)k * N + (size_t)y * W + x]) : 0.f);
         if (want) sum += settled(q, u, m, sg, hh).y;
     }
@@ -418,6 +439,7 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
     // grows with the world)
     __shared__ float2 ssum[CT * 5][ES_T];
     __shared__ uint8_t slot[ES_NW][32];
+    __shared__ __align__(16) float2 taps[ES_NW][ES_TAPS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int H = p.H, W = p.W, K = p.kt.K, C = p.kt.C;
     const size_t N = (size_t)H * W;
@@ -628,7 +650,7 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                         [&](int ys, int xs, int owner, int c, bool valid) {
                             const int k0 = (__shfl_sync(0xffffffffu, first, owner) >> (8 * c)) & 255;
                             const bool more = (__shfl_sync(0xffffffffu, many, owner) >> c) & 1;
-                            return alpha_at(q, pA, pP, pU, ys, xs, valid, k0, more) ? 1.f : 0.f;
+                            return alpha_at<LOC, RD>(q, pA, pP, pU, ys, xs, valid, k0, more, taps[warp]) ? 1.f : 0.f;
                         },
                         [&](int c, float ok) { lost |= (ok == 0.f ? 1u : 0u) << c; });
 #pragma unroll
@@ -688,7 +710,7 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                 if (__any_sync(0xffffffffu, close != 0))
                     deal_sites(
                         slot[warp], close, y, x,
-                        [&](int ys, int xs, int, int, bool valid) { return tests_at(q, pA, pP, pU, ys, xs, valid); },
+                        [&](int ys, int xs, int, int, bool valid) { return tests_at<LOC, RD>(q, pA, pP, pU, ys, xs, valid, taps[warp]); },
                         [&](int c, float t) {
 #pragma unroll
                             for (int i = 0; i < 4; i++)
