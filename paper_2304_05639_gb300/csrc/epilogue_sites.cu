@@ -22,10 +22,8 @@
 // other update kernels' arithmetic on the direct sums, so that a world's
 // decisions do not depend on the kernel or the convolution it takes.  (Settled
 // inside the kernels' loop, or with a site of each lane at a time, the guard that
-// large radii need makes a step of 600 x 900 at R = 45 / 56 1.15 / 2.25 ms; 0.31 /
-// 0.57 so, 0.56 / 0.93 with the direct sums throughout.  At R = 12, 13 a step has
-// one such site or none at 300 x 404, some 25 at 1080 x 1920, and they cost its
-// latency: 104 us for six steps of 300 x 404 where two have one, 79 without any.)
+// large radii need makes a step of 600 x 900 at R = 45 / 56 1.15 / 2.25 ms; 0.22 /
+// 0.62 so, 0.56 / 0.93 with the direct sums throughout.)
 //
 // What bounds it: on a mostly empty world the writes of the gene planes, on a
 // full one its loads and instruction issue (16 warps an SM at 128 registers, half of
@@ -135,8 +133,10 @@ __device__ __forceinline__ int tap_site(int2 tap, int y, int x, int H, int W)
 // Kernel k's direct sum at (y, x): its non-zero taps in k_direct_conv's order (a zero
 // weight adds nothing there), so the same bits.  By a whole warp: the lanes fetch 128
 // taps at once, the next ones while every lane adds these, in order, from shared
-// memory (sm: the warp's).  What it costs is its latency: 436 taps of R = 12 took
-// 14000 cycles with the operands passed round by shuffles.
+// memory (sm: the warp's).  At usual radii a step has a few such sites and they cost
+// its latency: 436 taps of R = 12 took 14000 cycles with the operands passed round
+// by shuffles, 10000 with the taps fetched just before their values (six steps of
+// 300 x 404 120, 109 and 94 us).
 constexpr int ES_TAPS = 128;
 __device__ __forceinline__ float direct_warp(const SitesParams& q, const float* A, int k, int y, int x, float2* sm)
 {
