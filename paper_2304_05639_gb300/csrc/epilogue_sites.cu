@@ -311,29 +311,50 @@ __device__ __forceinline__ bool passes(const SitesParams& q, float t)
     return q.fast ? !(t <= q.e.eps_u) : t > q.e.eps_u;
 }
 
-// The range (low, high) that a test t = h g (or u) may lie in: rounding, and the
+// How far a test t = h g (or u) at a potential u and |z| may be off: rounding, and the
 // potential's du.  With eta = du / s <= 1/64 the bump's ratio at z + d, |d| <= eta, is
 // exp(-z d - d^2 / 2): off by at most 2 |z| eta + eta^2 (|z| eta <= 5/4; beyond it both
-// bumps are zero).  A narrower bump's range is formed at z -+ eta.
-__device__ __forceinline__ float2 test_range(const SitesParams& q, float u, float t, float az, float sg, float hh)
+// bumps are zero).  `wide`: a narrower bump, or a threshold that lies where bumps
+// underflow; see test_range.
+__device__ __forceinline__ float test_off(const SitesParams& q, float u, float t, float az, float sg, float rs, bool& wide)
 {
-    const float du = fminf(q.g.du, fmaf(q.g.slope, fmaxf(u, 0.f), q.g.floor));
-    if (q.e.alpha_on) {
-        const float off = fmaf(1e-7f, fabsf(u), du);
-        return make_float2(t - off, t + off);
-    }
-    const float eta = du * rcp_approx(sg), z2 = az * az;
-    if (sg > 0.f && eta > 1.f / 64.f) {
+    // (u below zero by more than rounding: out of the unit interval, and summed directly)
+    const float du = fminf(q.g.du, fmaf(q.g.slope, u, q.g.floor));
+    wide = false;
+    if (q.e.alpha_on) return fmaf(1e-7f, fabsf(u), du);
+    const float eta = du * rs;
+    wide = sg > 0.f && (eta > 1.f / 64.f || q.tiny_eps);
+    return fabsf(t) * fmaf(2e-6f, az * az, fmaf(eta, fmaf(2.f, az, eta), 2e-6f));
+}
+
+// The range (low, high) of a `wide` test: a narrow bump's at z -+ eta.
+__device__ __forceinline__ float2 test_range(const SitesParams& q, float u, float t, float az, float sg, float hh, float off)
+{
+    const float eta = fminf(q.g.du, fmaf(q.g.slope, u, q.g.floor)) * rcp_approx(sg);
+    if (eta > 1.f / 64.f) {
         const float z0 = fmaxf(az - eta, 0.f), z1 = az + eta;
         const float t0 = hh * ex2_approx(-0.721347520444481703680f * (z0 * z0));
         const float t1 = hh * ex2_approx(-0.721347520444481703680f * (z1 * z1));
         const float r = fabsf(t0) * fmaf(2e-6f, fminf(z0 * z0, 225.f), 2e-6f);
         return make_float2(fminf(t0, t1) - r, fmaxf(t0, t1) + r);
     }
-    float off = fabsf(t) * fmaf(2e-6f, z2, fmaf(eta, fmaf(2.f, az, eta), 2e-6f));
-    // thresholds at zero: where the bump underflows
-    if (q.tiny_eps && sg > 0.f && z2 < 225.f && fabsf(t) < 1e-36f) off = 1e-36f;
+    if (az < 15.f && fabsf(t) < 1e-36f) off = 1e-36f;
     return make_float2(t - off, t + off);
+}
+
+// Whether a test may come out either way, and by how much it may be off.
+__device__ __forceinline__ bool undecided_test(const SitesParams& q, float u, float t, float az, float sg, float rs, float hh,
+                                               float& off)
+{
+    bool wide;
+    off = test_off(q, u, t, az, sg, rs, wide);
+    bool open = fabsf(t - q.e.eps_u) < off;    // (an exact test has off = 0)
+    if (wide) {
+        const float2 r = test_range(q, u, t, az, sg, hh, off);
+        open = r.x < q.e.eps_u && q.e.eps_u < r.y;
+        off = fmaxf(r.y - t, t - r.x);
+    }
+    return open;
 }
 
 // Kernel k's diffused genes at one site as the kernel divides them that the shape
@@ -388,8 +409,9 @@ __device__ __forceinline__ bool alpha_at(const SitesParams& q, const float* A, c
         // a lane's first kernel is known to be undecided
         bool open = on;
         if (__any_sync(0xffffffffu, on && kk != first)) {
-            const float2 r = test_range(q, u, t, fabsf((u - m) * rcp_approx(sg)), sg, hh);
-            open = on && (kk == first || (r.x < p.eps_u && p.eps_u < r.y));
+            const float rs = rcp_approx(sg);
+            float off;
+            open = on && (kk == first || undecided_test(q, u, t, fabsf((u - m) * rs), sg, rs, hh, off));
         }
         if (q.g.du > 0.f && __any_sync(0xffffffffu, open)) {
             u = direct_sums(q, A, kk, y, x, open, sm);
@@ -563,7 +585,7 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                     auto mu_of = [&](int c) { return PMU >= 0 ? ph[PMU >= 0 ? PMU : 0][c] : km; };
                     auto sg_of = [&](int c) { return PSG >= 0 ? ph[PSG >= 0 ? PSG : 0][c] : ks; };
                     auto h_of = [&](int c) { return PH >= 0 ? ph[PH >= 0 ? PH : 0][c] : kh; };
-                    bool pass[4] = {false, false, false, false};    // undecided tests pass for now
+                    uint32_t now = 0;               // undecided tests: they pass for now
                     Pre cur[NQ];
 #pragma unroll
                     for (int pp = 0; pp < NP; pp++) cur[pp] = nx[pp];
@@ -591,24 +613,25 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                             gk[c] = sg > 0.f ? e : 0.f;
                             tk[c] = p.alpha_on ? u[c] : h_of(c) * gk[c];
                             if (NP > 0) {
-                                const float2 r = test_range(q, u[c], tk[c], fabsf(z), sg, h_of(c));
-                                if (p.empty_out) tband[c] += fmaxf(r.y - tk[c], tk[c] - r.x);
-                                // (an exact test's range is one value)
-                                const bool open = (r.x < eps_u) & (eps_u < r.y);
-                                if (al[c] & open) {
-                                    many |= undecided & (1u << c);
-                                    if (!((undecided >> c) & 1)) first |= (uint32_t)k << (8 * c);
-                                    undecided |= 1u << c;
-                                    pass[c] = true;
-                                }
+                                float off;
+                                const bool open = undecided_test(q, u[c], tk[c], fabsf(z), sg, rs, h_of(c), off);
+                                if (p.empty_out) tband[c] += sg > 0.f || p.alpha_on ? off : 0.f;
+                                now |= (open ? 1u : 0u) << c;
                             }
+                        }
+                        if (NP > 0 && now) {
+                            many |= undecided & now;
+#pragma unroll
+                            for (int c = 0; c < 4; c++)
+                                if ((now & ~undecided) >> c & 1) first |= (uint32_t)k << (8 * c);
+                            undecided |= now;
                         }
                     }
                     float G[4];
                     if (want) {
 #pragma unroll
                         for (int c = 0; c < 4; c++) {
-                            if (NP > 0) al[c] = al[c] & (pass[c] | passes(q, tk[c]));
+                            if (NP > 0) al[c] = al[c] & (passes(q, tk[c]) | ((now >> c) & 1));
                             tsum[c] += tk[c];
                             G[c] = p.growth_form == 0 ? fmaf(2.f * gk[c], h_of(c), -h_of(c)) : h_of(c) * gk[c];
                         }
@@ -690,7 +713,11 @@ __global__ void __launch_bounds__(ES_T, CT > 3 || RD == 2 ? 3 : 4) k_epilogue_si
                     const float* cx = p.cos_x + x;
                     const float m = (o[0] + o[1]) + (o[2] + o[3]);
                     float2* a5 = &ssum[c * 5][threadIdx.x];
-                    auto add = [&](int v, float t) { a5[v * ES_T] = ff_add(a5[v * ES_T], make_float2(t, 0.f)); };
+                    auto add = [&](int v, float t) {       // (two-sum, the errors collected in .y)
+                        const float2 a = a5[v * ES_T];
+                        const float h = a.x + t, b = h - a.x;
+                        a5[v * ES_T] = make_float2(h, a.y + ((a.x - (h - b)) + (t - b)));
+                    };
                     add(0, m);
                     add(1, m * __ldg(&p.sin_y[y]));
                     add(2, m * __ldg(&p.cos_y[y]));
