@@ -1082,7 +1082,9 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
     if (c->tile) {
         int blocks = 0;
         for (int ch = 0; ch < C; ch++) blocks += c->tl.g.tiles_x * c->tl.g.tiles_y * ((kcount[ch] + c->tl.kpb - 1) / c->tl.kpb);
-        c->gate_pays = blocks > c->num_sms * (c->tl.N == 128 ? 3 : 8);
+        // as many as a gated launch runs at once (1080 x 1200, 15 kernels in 396 blocks, us a
+        // step with the gate and without: 2 patches 113 / 135, 8 134 / 150, 40 189 / 185)
+        c->gate_pays = blocks > c->num_sms * (c->tl.N == 128 ? 2 : 8);
         c->tl.C = C;
         memcpy(c->tl.kcount, kcount, sizeof(kcount));
         memcpy(c->tl.klist, klist, sizeof(klist));
