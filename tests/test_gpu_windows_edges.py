@@ -134,10 +134,11 @@ def test_narrow_bumps_decide_as_the_direct_sums(sigma, z, on_windows):
 
 FLAT = inputs.KernelDesc(0, 0, 1, inputs.KERNEL_BUMPS, (1.0,), bump=(0.0, 1e5, 1.0, 0.5, 0.1, 0.0))
 SHELL = inputs.KernelDesc(0, 0, 1, inputs.KERNEL_SHELLS, (1.0,))
+SIGNED = inputs.KernelDesc(0, 0, 1, inputs.KERNEL_SHELLS, (1.0, -0.4))      # absolute weights sum to more than 1
 
 
 @pytest.mark.parametrize("shape", [(130, 132, 12), (300, 404, 20), (300, 404, 31), (600, 900, 56)])
-@pytest.mark.parametrize("kernel", [FLAT, SHELL], ids=["flat", "shell"])
+@pytest.mark.parametrize("kernel", [FLAT, SHELL, SIGNED], ids=["flat", "shell", "signed"])
 @pytest.mark.parametrize("sigma,z", [(0.03, 1.0), (0.004, 0.0)])
 @pytest.mark.parametrize("on_windows", [False, True])
 def test_the_sums_rounding_at_any_radius(shape, kernel, sigma, z, on_windows):
@@ -512,3 +513,29 @@ def test_ring_worlds_in_a_batch(autotune):
             assert torch.equal(A[i], A1) and torch.equal(P[i], P1)
     finally:
         lenia.lenia_batch_destroy(b)
+
+
+@pytest.mark.parametrize("kw", [dict(H=64, W=64, R=6, n_rings=12), dict(H=128, W=128, R=12, n_rings=24, n_channels=1),
+                                dict(H=256, W=128, R=9, n_rings=4)])
+def test_ring_worlds_without_maintenance_in_windows(kw):
+    """Power-of-two ring worlds whose genes are not maintained may convolve their rings in
+    windows: ring potentials against the oracle (unnormalised sums of up to 50
+    values), and a step (its genes unchanged)."""
+    torch = torch_mod()
+    w = inputs.ring_world(patch=24, n_geno=2, **kw)
+    w.maintain_genes = 0
+    cfg, ks = lenia.config_from_world(w)
+    ctx = lenia.lenia_init(cfg, ks)
+    try:
+        A, P = to_dev(w.A), to_dev(w.P)
+        V = torch.empty((w.n_channels, w.n_rings, w.height, w.width), device="cuda")
+        lenia.lenia_potentials(ctx, A, V)
+        A2, P2 = torch.empty_like(A), torch.empty_like(P)
+        lenia.lenia_step(ctx, A, P, A2, P2)
+        torch.cuda.synchronize()
+        rings = np.stack([oracle.ring_potentials(w.A[c], w.kernels[0].radius, w.n_rings) for c in range(w.n_channels)])
+        assert np.abs(V.cpu().numpy() - rings).max() <= 2e-5
+        want = oracle.ring_step(w)[0]
+        assert np.abs(A2.cpu().numpy() - want).max() <= 1e-5 and torch.equal(P2, P)
+    finally:
+        lenia.lenia_destroy(ctx)
