@@ -134,7 +134,7 @@ def test_narrow_bumps_decide_as_the_direct_sums(sigma, z, on_windows):
 
 FLAT = inputs.KernelDesc(0, 0, 1, inputs.KERNEL_BUMPS, (1.0,), bump=(0.0, 1e5, 1.0, 0.5, 0.1, 0.0))
 SHELL = inputs.KernelDesc(0, 0, 1, inputs.KERNEL_SHELLS, (1.0,))
-SIGNED = inputs.KernelDesc(0, 0, 1, inputs.KERNEL_SHELLS, (1.0, -0.4))      # absolute weights sum to more than 1
+SIGNED = inputs.KernelDesc(0, 0, 1, inputs.KERNEL_SHELLS, (-0.4, 1.0))      # absolute weights sum to more than 1
 
 
 @pytest.mark.parametrize("shape", [(130, 132, 12), (300, 404, 20), (300, 404, 31), (600, 900, 56)])
