@@ -1452,6 +1452,7 @@ lenia_status lenia_rollout(lenia_ctx* c, float* A, float* P, int32_t n_steps, fl
         tp.dt = c->cfg.dt;
         for (int k = 0; k < tp.K; k++) {
             tp.mu[k] = c->kt.mu[k];
+            tp.sigma[k] = c->kt.sigma[k];
             tp.rsigma[k] = (float)(1.0 / (double)c->kt.sigma[k]);
             tp.h[k] = c->kt.h[k];
         }

@@ -352,7 +352,7 @@ struct TileRolloutParams {
     const float2* tw;
     int K, n_steps, growth_form;
     float dt;
-    float mu[kTileRolloutKernels], rsigma[kTileRolloutKernels], h[kTileRolloutKernels];
+    float mu[kTileRolloutKernels], sigma[kTileRolloutKernels], rsigma[kTileRolloutKernels], h[kTileRolloutKernels];
 };
 // the fewest steps that such a rollout takes in one block, or 0 where none does
 int tile_rollout_steps(int H, int W, int C, int K);

@@ -724,7 +724,9 @@ k_tile_conv(const __grid_constant__ TileParams p)
 // each, the growth in registers, and nothing in global memory.  What bounds it
 // is the latency of those passes (64^2, one kernel: see the launch's comment).
 template <int N, bool ONE>
-__global__ void __launch_bounds__(4 * N) k_tile_rollout(const __grid_constant__ TileRolloutParams p)
+__host__ __device__ constexpr bool rollout_stash() { return N == 128 && !ONE; }
+template <int N, bool ONE>
+__global__ void __launch_bounds__(4 * N, 1) k_tile_rollout(const __grid_constant__ TileRolloutParams p)
 {
     pdl_enter();
     using X = TC<N>;
@@ -736,7 +738,21 @@ __global__ void __launch_bounds__(4 * N) k_tile_rollout(const __grid_constant__ 
     const int m1 = lane % X::RR;
     for (int i = threadIdx.x; i < N; i += T) twc[i] = __ldg(&p.tw[i]);
     int ys[NR], base[NR];
-    float2 a[NR][8];                                     // the state: rows ys[i], pairs m1 + RR m2
+    // The state: rows ys[i], pairs m1 + RR m2.  Several kernels of 128^2: beside the growth's
+    // sums neither it nor the spectrum fits the registers; it waits in shared memory,
+    // the spectrum in TMEM (each thread's share in its own lane).
+    constexpr bool TM = rollout_stash<N, ONE>();
+    float2 a[TM ? 1 : NR][8];
+    float2* stash = twc + N + threadIdx.x;
+    auto state = [&](int i, int j) -> float2& {
+        if constexpr (TM) return stash[(i * 8 + j) * T];
+        else return a[i][j];
+    };
+    __shared__ uint32_t tmem_base;
+    if (TM && warp == 0) {
+        tmem_alloc<TM ? X::TMEM : 32>(&tmem_base);
+        tmem_fence_before_sync();
+    }
 #pragma unroll
     for (int i = 0; i < NR; i++) {
         ys[i] = (warp + i * NW) * RPW + lane / X::RR;
@@ -744,7 +760,7 @@ __global__ void __launch_bounds__(4 * N) k_tile_rollout(const __grid_constant__ 
 #pragma unroll
         for (int m2 = 0; m2 < 8; m2++) {
             const float* q = p.A + (size_t)ys[i] * N + 2 * (m1 + X::RR * m2);
-            a[i][m2] = make_float2(q[0], q[1]);
+            state(i, m2) = make_float2(q[0], q[1]);
         }
     }
     // this thread's column task, one per thread
@@ -753,12 +769,14 @@ __global__ void __launch_bounds__(4 * N) k_tile_rollout(const __grid_constant__ 
     float s1[X::CA];
     if (ONE) spectrum_of<N>(p.S, c, b, s1);
     __syncthreads();
+    if (TM) tmem_fence_after_sync();
+    const uint32_t taddr = TM ? tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((warp >> 2) * 2 * X::CA) : 0;
     for (int t = 0; t < p.n_steps; t++) {
 #pragma unroll
         for (int i = 0; i < NR; i++) {
             float2 v[8];
 #pragma unroll
-            for (int m2 = 0; m2 < 8; m2++) v[m2] = a[i][m2];
+            for (int m2 = 0; m2 < 8; m2++) v[m2] = state(i, m2);
             DFT<8, false, true>::run(v);
 #pragma unroll
             for (int j = 0; j < 8; j++) st2(buf, base[i] ^ (j * 8), v[j]);
@@ -783,12 +801,23 @@ __global__ void __launch_bounds__(4 * N) k_tile_rollout(const __grid_constant__ 
 #pragma unroll
             for (int i = 0; i < X::CA; i++) F0[i * 8 + b] = f[i];
         }
+        if constexpr (TM) {
+            const float* w = reinterpret_cast<const float*>(f);
+            tmem_st16(taddr, w);
+            tmem_st16(taddr + 16, w + 16);
+            tmem_wait_st();
+        }
         float2 acc[NR][8];
         for (int k = 0; k < (ONE ? 1 : p.K); k++) {
             __syncthreads();                             // F0 complete; the last kernel's rows are read
             float2 v[X::CA];
 #pragma unroll
             for (int i = 0; i < X::CA; i++) v[i] = f[i];
+            if constexpr (TM) {
+                float* w = reinterpret_cast<float*>(v);
+                tmem_ld16(taddr, w);
+                tmem_ld16(taddr + 16, w + 16);
+            }
             if (ONE && c != 0) {
 #pragma unroll
                 for (int i = 0; i < X::CA; i++) v[i] = cscale(v[i], s1[i]);
@@ -810,10 +839,15 @@ __global__ void __launch_bounds__(4 * N) k_tile_rollout(const __grid_constant__ 
                 }
             }
             __syncthreads();
-            const float m = p.mu[k], rs = p.rsigma[k], h = p.h[k];
+            const float m = p.mu[k], sg = p.sigma[k], rs = p.rsigma[k], h = p.h[k];
+            // (u - m) / sigma by the reciprocal and one residual correction, and expf: with
+            // the quotient uncorrected and the hardware exponential the errors of 24 rollouts
+            // (64^2, 16 steps) had a geometric mean of 8.9e-7 and a largest of 4.0e-6; with
+            // IEEE division 8.6e-7 and 2.5e-6, which a step 20% longer paid for
             auto growth = [&](float u) {
-                const float z = (u - m) * rs;
-                const float g = ex2_approx(-0.721347520444481703680f * (z * z));     // -log2(e) / 2
+                const float d = u - m, q = d * rs;
+                const float z = fmaf(fmaf(-q, sg, d), rs, q);
+                const float g = expf(-0.5f * z * z);
                 return p.growth_form == 0 ? h * fmaf(2.f, g, -1.f) : h * g;
             };
 #pragma unroll
@@ -831,18 +865,27 @@ __global__ void __launch_bounds__(4 * N) k_tile_rollout(const __grid_constant__ 
 #pragma unroll
         for (int i = 0; i < NR; i++)
 #pragma unroll
-            for (int j = 0; j < 8; j++)
-                a[i][j] = make_float2(__saturatef(fmaf(p.dt, acc[i][j].x, a[i][j].x)),
-                                      __saturatef(fmaf(p.dt, acc[i][j].y, a[i][j].y)));
+            for (int j = 0; j < 8; j++) {
+                const float2 s = state(i, j);
+                state(i, j) = make_float2(__saturatef(fmaf(p.dt, acc[i][j].x, s.x)), __saturatef(fmaf(p.dt, acc[i][j].y, s.y)));
+            }
     }
 #pragma unroll
     for (int i = 0; i < NR; i++)
 #pragma unroll
         for (int m2 = 0; m2 < 8; m2++) {
             float* q = p.A + (size_t)ys[i] * N + 2 * (m1 + X::RR * m2);
-            q[0] = a[i][m2].x;
-            q[1] = a[i][m2].y;
+            q[0] = state(i, m2).x;
+            q[1] = state(i, m2).y;
         }
+    if (TM) {
+        tmem_fence_before_sync();
+        __syncthreads();
+        if (warp == 0) {
+            tmem_fence_after_sync();
+            tmem_dealloc<TM ? X::TMEM : 32>(tmem_base);
+        }
+    }
 }
 
 // Kernel spectra in the order the column tasks read them, from S[kx][ky] of the
@@ -1038,11 +1081,10 @@ cudaError_t launch_tile_conv(const TileParams& p0, cudaStream_t s)
 }
 
 // Where one block pays (us for 2 / 6 / 16 steps against the same steps as launches):
-//   64^2   one kernel 9 / 13 / 30 against 17 / 56 / 148, four 14 / 34 / 83 against 17 /
+//   64^2   one kernel 8 / 13 / 30 against 17 / 56 / 148, four 14 / 34 / 86 against 17 /
 //          50 / 132
-//   128^2  one kernel 17 / 41 / 102 against 17 / 50 / 132, three 36 / 95 / 244 against
-//          17 / 56 / 148 (32 / 99 / 263 with the FFT passes), four 43 / 118 / 306 (35 /
-//          111 / 295 with the passes)
+//   128^2  one kernel 18 / 45 / 112 against 17 / 50 / 132, three (from four steps on) 99 /
+//          255 against 56 / 148 (99 / 263 with the FFT passes)
 int tile_rollout_steps(int H, int W, int C, int K)
 {
     if (H != W || C != 1) return 0;
@@ -1053,9 +1095,10 @@ int tile_rollout_steps(int H, int W, int C, int K)
 template <int N, bool ONE>
 static cudaError_t launch_rollout_n(const TileRolloutParams& p, cudaStream_t s)
 {
-    cudaError_t e = smem_limit<k_tile_rollout<N, ONE>>(TC<N>::SMEM);
+    const size_t smem = TC<N>::SMEM + (rollout_stash<N, ONE>() ? (size_t)N * N * sizeof(float) : 0);
+    cudaError_t e = smem_limit<k_tile_rollout<N, ONE>>(smem);
     if (e != cudaSuccess) return e;
-    launch_pdl(k_tile_rollout<N, ONE>, dim3(1), dim3(4 * N), TC<N>::SMEM, s, p);
+    launch_pdl(k_tile_rollout<N, ONE>, dim3(1), dim3(4 * N), smem, s, p);
     return cudaGetLastError();
 }
 
