@@ -1438,7 +1438,10 @@ lenia_status lenia_rollout(lenia_ctx* c, float* A, float* P, int32_t n_steps, fl
         CUDA_OR_FAIL(c, launch_cluster_rollout(cp, s));
         return LENIA_OK;
     }
-    if (c->block && !stats_out &&
+    // (a reciprocal of sigma that is no number takes the steps, which divide)
+    bool reciprocals = true;
+    for (int k = 0; k < c->cfg.n_kernels; k++) reciprocals = reciprocals && c->kt.sigma[k] >= 1e-36f;
+    if (c->block && reciprocals && !stats_out &&
         n_steps >= tile_rollout_steps(c->cfg.height, c->cfg.width, c->cfg.n_channels, c->cfg.n_kernels)) {
         TileRolloutParams tp;
         memset(&tp, 0, sizeof(tp));

@@ -539,3 +539,25 @@ def test_ring_worlds_without_maintenance_in_windows(kw):
         assert np.abs(A2.cpu().numpy() - want).max() <= 1e-5 and torch.equal(P2, P)
     finally:
         lenia.lenia_destroy(ctx)
+
+
+@pytest.mark.parametrize("sigma", [1e-40, 1e-37, 1e-30])
+def test_one_block_rollouts_of_vanishing_bumps(sigma):
+    """A sigma whose reciprocal is infinite: rollouts give what steps give."""
+    torch = torch_mod()
+    w = inputs.single_kernel_global(H=64, W=64, R=9, patch=32, sigma=0.05, mu=0.0)
+    w.kernels[0].sigma = float(np.float32(sigma))
+    cfg, ks = lenia.config_from_world(w)
+    ctx = lenia.lenia_init(cfg, ks)
+    try:
+        A = to_dev(w.A)
+        S = A.clone()
+        lenia.lenia_rollout(ctx, A, None, 3)
+        for _ in range(3):
+            T = torch.empty_like(S)
+            lenia.lenia_step(ctx, S, None, T, None)
+            S = T
+        torch.cuda.synchronize()
+        assert float((A - S).abs().max()) <= 3e-5
+    finally:
+        lenia.lenia_destroy(ctx)
