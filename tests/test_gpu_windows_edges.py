@@ -545,7 +545,7 @@ def test_ring_worlds_without_maintenance_in_windows(kw):
 def test_one_block_rollouts_of_vanishing_bumps(sigma):
     """A sigma whose reciprocal is infinite: rollouts give what steps give."""
     torch = torch_mod()
-    w = inputs.single_kernel_global(H=64, W=64, R=9, patch=32, sigma=0.05, mu=0.0)
+    w = inputs.single_kernel_global(H=64, W=64, R=9, patch=32, sigma=0.05, mu=0.3)
     w.kernels[0].sigma = float(np.float32(sigma))
     cfg, ks = lenia.config_from_world(w)
     ctx = lenia.lenia_init(cfg, ks)
