@@ -111,10 +111,9 @@ struct Stencil {
                         s = first ? v[j][RD + c + d] : s + v[j][RD + c + d];
                         n = first ? one[j][RD + c + d] : n + one[j][RD + c + d];
                     }
-            // (a sum above the count gives 1, an infinite one too, where the quotient's
-            // correction would be infinity less infinity)
-            s = s > n ? n : s;
-            const float rn = rcp_approx(n), t = s * rn;
+            // (2 stands for a larger quotient: an infinite one's correction would be infinity
+            // less infinity, and it saturates to 1 all the same)
+            const float rn = rcp_approx(n), t = fminf(s * rn, 2.f);
             const float r = fmaf(fmaf(-t, n, s), rn, t);
             out[c] = n > 0.f ? __saturatef(r) : 0.f;
         }
