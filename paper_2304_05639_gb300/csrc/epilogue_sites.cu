@@ -27,9 +27,9 @@
 //
 // What bounds it: on a mostly empty world the writes of the gene planes, on a
 // full one its loads and instruction issue (16 warps an SM at 128 registers, half of
-// the issue slots used).  1080 x 1920, 15 kernels, 43% live: 121 us (533 with
-// the general kernel; 146 with every lane loading its own stencils); 2048^2 all live
-// 333 us; 512^2, 8 kernels, three genes, radius 2: 23 us (230).
+// the issue slots used).  1080 x 1920, 15 kernels, 43% live: 128 us on cold caches
+// (533 with the general kernel; 146 with every lane loading its own stencils), of
+// which settling takes 5; 512^2, 8 kernels, three genes, radius 2: 24 us (230).
 #include <math.h>
 #include <string.h>
 

@@ -32,8 +32,9 @@
 // What bounds it: the FP32 pipes and instruction issue (about 1500 FP32
 // operations per thread and inverse transform, against 7 shared-memory passes).
 // 1080 x 1920, 15 kernels R = 13: 97 us, 52 to 66 where the gate skips half of the
-// windows (direct sums 1135); 2048^2, 15 kernels R = 5: 143 us, 102 gated (direct
-// sums 415); 256^2, 15 kernels: 11 us (three FFT passes 14).
+// windows (direct sums 1135); 2048^2, 15 kernels R = 5, gated: 107 us (102 without
+// the look at its values; direct sums 415); 256^2, 15 kernels: 11 us (three FFT
+// passes 14).
 #include <math.h>
 
 #include <utility>
