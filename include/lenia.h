@@ -395,7 +395,8 @@ LENIA_API lenia_status lenia_kernel_weights(const lenia_ctx* ctx, int32_t k, dou
 /* Convolution path in use: LENIA_CONV_FFT, _DIRECT, _DIRECT_BF16 or _DIRECT_BF16X3. */
 LENIA_API int32_t lenia_conv_path(const lenia_ctx* ctx);
 
-/* Form of lenia_rollout (without stats_out, n_steps >= 2) for this context:
+/* Form of lenia_rollout (without stats_out, n_steps >= 2 or as many as it says
+ * there) for this context:
  * LENIA_ROUTE_STEPS (launches per step, pairs of steps replayed from a CUDA
  * graph), LENIA_ROUTE_COOPERATIVE (one cooperative launch) or
  * LENIA_ROUTE_BLOCK (one thread block), LENIA_ROUTE_CLUSTER (one thread-block cluster; a caller's A that is not

@@ -1051,7 +1051,8 @@ lenia_status lenia_init(const lenia_config* cfg, const lenia_kernel_desc* kernel
     // them), keeps the sums throughout, and so do ring worlds and an explicit
     // LENIA_CONV_DIRECT.
     const bool want_adj = cfg->max_rollout_steps > 0 && c->n_p == 0 && !cfg->maintain_genes;
-    c->guard = window_guard(c);
+    if (path == LENIA_CONV_DIRECT && cfg->conv_path == LENIA_CONV_AUTO && !n_rings && cfg->maintain_genes)
+        c->guard = window_guard(c);
     if ((path == LENIA_CONV_FFT && !cfg->maintain_genes) ||
         (path == LENIA_CONV_DIRECT && cfg->conv_path == LENIA_CONV_AUTO && !n_rings &&
          (!cfg->maintain_genes || (epilogue_sites_supported(epi_params(c)) &&
