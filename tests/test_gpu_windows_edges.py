@@ -137,7 +137,8 @@ SHELL = inputs.KernelDesc(0, 0, 1, inputs.KERNEL_SHELLS, (1.0,))
 SIGNED = inputs.KernelDesc(0, 0, 1, inputs.KERNEL_SHELLS, (-0.4, 1.0))      # absolute weights sum to more than 1
 
 
-@pytest.mark.parametrize("shape", [(130, 132, 12), (300, 404, 20), (300, 404, 31), (600, 900, 56)])
+# (300 x 512: the streaming kernel's arithmetic)
+@pytest.mark.parametrize("shape", [(130, 132, 12), (300, 404, 20), (300, 512, 20), (300, 404, 31), (600, 900, 56)])
 @pytest.mark.parametrize("kernel", [FLAT, SHELL, SIGNED], ids=["flat", "shell", "signed"])
 @pytest.mark.parametrize("sigma,z", [(0.03, 1.0), (0.004, 0.0)])
 @pytest.mark.parametrize("on_windows", [False, True])
